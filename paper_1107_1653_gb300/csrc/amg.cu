@@ -1012,7 +1012,7 @@ GamePI amgpi_game(gs_solver* s, Problem& P, double eps, bool warm) {
     }
     BatchArgs B{};
     B.T = G.tables();
-    B.out = {G.v, G.v32, G.alpha, G.beta, G.sel, G.rhs, G.gstats, G.gres};
+    B.out = {G.v, G.v32, G.alpha, G.beta, G.sel, G.rhs, G.gstats, G.gres, G.leaksel};
     B.count = 1;
     B.max_n = G.max_n;
     B.st_off = G.st_off;

@@ -84,11 +84,6 @@ __global__ void k_game_prepare(GameTables T, int count, const int64_t* __restric
 }
 
 // ------------------------------------------------------------------ block helpers
-__device__ __forceinline__ double warp_maxd(double v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
-    return v;
-}
 template <typename T>
 __device__ __forceinline__ T warp_sum(T v) {
 #pragma unroll
@@ -96,25 +91,56 @@ __device__ __forceinline__ T warp_sum(T v) {
     return v;
 }
 
-// Block-wide reductions; every thread gets the result.  `red` is shared scratch.
-__device__ double block_max(double v, double* red) {
-    v = warp_maxd(v);
-    __syncthreads();
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
-    __syncthreads();
-    double m = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) m = fmax(m, red[w]);
-    return m;
+// Maximum of 64-bit patterns over a warp by two 32-bit reductions (non-negative
+// doubles order like their bits; a float64 compare costs as much as float64
+// arithmetic here).
+__device__ __forceinline__ unsigned long long warp_max_bits(unsigned long long v) {
+    const unsigned hi = (unsigned)(v >> 32);
+    const unsigned mh = __reduce_max_sync(0xffffffffu, hi);
+    const unsigned ml = __reduce_max_sync(0xffffffffu, hi == mh ? (unsigned)v : 0u);
+    return (unsigned long long)mh << 32 | ml;
 }
-template <typename T>
-__device__ T block_sum(T v, T* red) {
+
+// Shared scratch of the block reductions: two copies used in turn, so that one
+// block barrier per reduction is enough (a copy is written again only after
+// the barrier of the reduction in between).
+struct RedScratch {
+    unsigned long long m[2][2][32];
+    double d[2][32];
+    int i[2][32];
+};
+
+// Block-wide reductions over `bufs`; every thread gets the result.
+__device__ __forceinline__ void block_max2(unsigned long long a, unsigned long long b, RedScratch& S, int f,
+                                           unsigned long long* A, unsigned long long* B) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    a = warp_max_bits(a);
+    b = warp_max_bits(b);
+    if (lane == 0) {
+        S.m[f][0][w] = a;
+        S.m[f][1][w] = b;
+    }
+    __syncthreads();
+    *A = warp_max_bits(lane < nw ? S.m[f][0][lane] : 0ull);
+    *B = warp_max_bits(lane < nw ? S.m[f][1][lane] : 0ull);
+}
+__device__ __forceinline__ int block_sum_int(int v, RedScratch& S, int f) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    v = __reduce_add_sync(0xffffffffu, v);
+    if (lane == 0) S.i[f][w] = v;
+    __syncthreads();
+    return __reduce_add_sync(0xffffffffu, lane < nw ? S.i[f][lane] : 0);
+}
+// Sum in a fixed order: a tree over the lanes, then a tree over the warps.
+__device__ __forceinline__ double block_sum_double(double v, RedScratch& S, int f) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
     v = warp_sum(v);
+    if (lane == 0) S.d[f][w] = v;
     __syncthreads();
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
-    __syncthreads();
-    T s = 0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += red[w];   // fixed order
-    return s;
+    v = lane < nw ? S.d[f][lane] : 0.0;
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return __shfl_sync(0xffffffffu, v, 0);   // at most 16 warps: the tree over lanes 0 .. 15
 }
 
 // ------------------------------------------------------------------ one game
@@ -288,6 +314,189 @@ __device__ int improve_state(const Game& G, const BatchOut& O, int mode, int64_t
     return changed;
 }
 
+// ------------------------------------------------------------------ improvement, one lane per row
+// 32 consecutive aligned bytes by one 256-bit load (the tables do not change
+// while a kernel runs).
+__device__ __forceinline__ void load_32b(const void* p, unsigned r[8]) {
+    unsigned long long q[4];
+    asm("ld.global.nc.v4.b64 {%0, %1, %2, %3}, [%4];" : "=l"(q[0]), "=l"(q[1]), "=l"(q[2]), "=l"(q[3]) : "l"(p));
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        r[2 * k] = (unsigned)q[k];
+        r[2 * k + 1] = (unsigned)(q[k] >> 32);
+    }
+}
+
+// One row's entries in registers: columns and probabilities rounded to float32
+// (rows of 8 entries; with bfloat16 storage rounded from the float64 values).
+struct Row8 {
+    unsigned c[8];
+    float p[8];
+    __device__ __forceinline__ void load(const GameTables& T, int64_t row) {
+        load_32b(T.col + row * 8, c);
+        unsigned q[8];
+        if (T.prob32) {
+            load_32b(T.prob32 + row * 8, q);
+#pragma unroll
+            for (int k = 0; k < 8; ++k) p[k] = __uint_as_float(q[k]);
+        } else {
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                load_32b(T.prob + row * 8 + 4 * h, q);
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                    p[4 * h + k] = f64_to_f32(__hiloint2double((int)q[2 * k + 1], (int)q[2 * k]));
+            }
+        }
+    }
+    // F(v; x, a, b) in float32 (row_value_f's order of operations).
+    __device__ __forceinline__ float value(const Game& G, const float* v32, double r64) const {
+        float vc[8], s = 0.0f;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) vc[k] = v32[c[k]];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) s = fmaf(p[k], vc[k], s);
+        return G.mu_f * s + f64_to_f32(r64);
+    }
+};
+
+// Whether the improvement below takes a game's action counts: the rows of a
+// state, and those of one MAX action, each fill an aligned group of lanes.
+__host__ __device__ __forceinline__ bool rows_in_lanes(int m1, int m2) {
+    return m1 <= kScreenMaxM1 && m1 * m2 <= 32 && (m1 & (m1 - 1)) == 0 && (m2 & (m2 - 1)) == 0;
+}
+
+// Policy improvement of a whole game with one lane per row (x, a, b): the
+// decisions and their float32 screen are those of improve_state, but a warp
+// reads its rows' entries as consecutive memory, and the minimum over b and
+// the maximum over a are taken by lane exchanges inside the state's group of
+// lanes (m1 m2 of them; the m2 of the current action in mode 1).  Bound by the
+// bytes of the rows (64 per row of 8 entries, and its reward) and the gathers
+// from v32: the one-thread-per-state form reads each row's entries one by one,
+// 16 rows apart from its neighbours'.  NE states per lane group are in flight
+// at once.  Measured per improvement, games of 4224 states on average with 4 x 4
+// actions, one block each: all actions 823 -> 221 us, MIN's reply at fixed alpha
+// 258 -> 58 us; one game of 5e5 states on the whole GPU: 892 -> 331 and 324 ->
+// 83 us.  Writes beta, sel, rhs (and alpha in mode 0); returns this thread's
+// count of changed policy entries.
+template <int KC, int MODE, class Ctx>
+__device__ __noinline__ int improve_rows(const Game& G, const BatchOut& O, double tau, float vmaxf, const double* v,
+                                         const float* v32, const Ctx& C) {
+    constexpr int NE = 2;
+    const int m1 = G.T.m1, m2 = G.T.m2;
+    const int grp = MODE == 1 ? m2 : G.R;
+    const int lane = threadIdx.x & 31, sub = lane & (grp - 1);
+    const int gl = __ffs(grp) - 1, bl = __ffs(m2) - 1;   // log2
+    const int per = 32 >> gl;                            // states per warp step
+    const int b = sub & (m2 - 1);
+    const float tauf = f64_to_f32(tau);
+    int changed = 0;
+    for (int64_t base = (int64_t)C.warp() * per * NE; base < G.n; base += (int64_t)C.warps() * per * NE) {
+        int64_t st[NE], row[NE];
+        int a[NE], acur[NE];
+        bool ok[NE];
+        double r64[NE];
+        float F[NE];
+#pragma unroll
+        for (int e = 0; e < NE; ++e) {
+            const int64_t i = base + e * per + (lane >> gl);
+            ok[e] = i < G.n;
+            st[e] = ok[e] ? i : G.n - 1;
+            acur[e] = O.alpha[G.x0 + st[e]];
+        }
+#pragma unroll
+        for (int e = 0; e < NE; ++e) {
+            a[e] = MODE == 1 ? acur[e] : sub >> bl;
+            row[e] = G.row0 + st[e] * G.R + a[e] * m2 + b;
+            r64[e] = G.T.rew[row[e]];
+        }
+        if constexpr (KC == 8) {
+            Row8 R8[NE];
+#pragma unroll
+            for (int e = 0; e < NE; ++e) R8[e].load(G.T, row[e]);
+#pragma unroll
+            for (int e = 0; e < NE; ++e) F[e] = R8[e].value(G, v32, r64[e]);
+        } else {
+#pragma unroll
+            for (int e = 0; e < NE; ++e) {
+                int64_t k0, k1;
+                row_range(G.T, row[e], &k0, &k1);
+                float sum = 0.0f;
+                for (int64_t k = k0; k < k1; ++k) sum = fmaf(prob_at_f(G.T, k), v32[G.T.col[k]], sum);
+                F[e] = G.mu_f * sum + f64_to_f32(r64[e]);
+            }
+        }
+#pragma unroll
+        for (int e = 0; e < NE; ++e) {
+            // smallest and second smallest F over b (ties: the lower b), largest |r|
+            float best = F[e], second = INFINITY, rmax = fabsf(f64_to_f32(r64[e]));
+            int first = b;
+            for (int o = 1; o < m2; o <<= 1) {
+                const float b2 = __shfl_xor_sync(0xffffffffu, best, o);
+                const float s2 = __shfl_xor_sync(0xffffffffu, second, o);
+                const int f2 = __shfl_xor_sync(0xffffffffu, first, o);
+                rmax = fmaxf(rmax, __shfl_xor_sync(0xffffffffu, rmax, o));
+                second = fminf(fminf(second, s2), fmaxf(best, b2));
+                if (b2 < best || (b2 == best && f2 < first)) {
+                    best = b2;
+                    first = f2;
+                }
+            }
+            float err = 0x1p-18f * (G.mu_f * vmaxf + rmax);
+            bool sure = m2 == 1 || second - best > 2.0f * err + tauf;
+            int anew = acur[e];
+            if (MODE != 1) {
+                // every reply must be sure; the largest and second largest over a
+                float g1 = best, g2 = -INFINITY;
+                int ga = a[e];
+                for (int o = m2; o < grp; o <<= 1) {
+                    const float h1 = __shfl_xor_sync(0xffffffffu, g1, o);
+                    const float h2 = __shfl_xor_sync(0xffffffffu, g2, o);
+                    const int ha = __shfl_xor_sync(0xffffffffu, ga, o);
+                    rmax = fmaxf(rmax, __shfl_xor_sync(0xffffffffu, rmax, o));
+                    sure &= __shfl_xor_sync(0xffffffffu, (int)sure, o) != 0;
+                    g2 = fmaxf(fmaxf(g2, h2), fminf(g1, h1));
+                    if (h1 > g1 || (h1 == g1 && ha < ga)) {
+                        g1 = h1;
+                        ga = ha;
+                    }
+                }
+                if (MODE == 0) {
+                    err = 0x1p-18f * (G.mu_f * vmaxf + rmax);
+                    sure = sure && (m1 == 1 || g1 - g2 > 2.0f * err + tauf);
+                    anew = ga;
+                }
+            }
+            if (!ok[e]) continue;
+            const int64_t x = G.x0 + st[e];
+            if (!sure) {
+                if (sub == 0) {
+                    double res;
+                    changed += improve_state_exact(G, O, MODE, st[e], tau, v, &res);
+                }
+                continue;
+            }
+            if (b == first) {   // the lane of the chosen b of its action
+                uint8_t& bref = O.beta[x * m1 + a[e]];
+                if (bref != b) {
+                    bref = (uint8_t)b;
+                    if (MODE == 1) ++changed;
+                }
+                if (a[e] == anew) {   // ... of the state's action
+                    if (MODE == 0 && anew != acur[e]) {
+                        O.alpha[x] = (uint8_t)anew;
+                        ++changed;
+                    }
+                    O.sel[x] = row[e];
+                    O.rhs[x] = r64[e];
+                }
+            }
+        }
+    }
+    return changed;
+}
+
+// ------------------------------------------------------------------ policy-fixed rows
 // Transition probability k in the relaxation's precision.
 template <typename T>
 __device__ __forceinline__ T prob_at(const GameTables& tb, int64_t k) {
@@ -330,10 +539,33 @@ __device__ __forceinline__ T diag_row(const Game& G, const BatchOut& O, int64_t 
     return (sizeof(T) == 4 ? (T)G.T.leak32[row] : (T)G.T.leak[row]) + off;
 }
 
-// The same row operations on the slot-major copy of the selected rows (same
-// entries, same order: the same arithmetic).
-// (KC > 0: rows of exactly KC entries, known at compile time, so that a
-// row's loads are issued together; KC = 0: S.K at run time.)
+// Copies state i's selected row into the slot-major arrays, with the inverse
+// of its diagonal (the relaxation multiplies by it).
+template <typename T, int KC>
+__device__ __forceinline__ void compact_row(const Game& G, const Compact& S, int64_t i, int64_t row) {
+    const int K = KC > 0 ? KC : S.K;
+    const int64_t k0 = row * K;
+    const T mu = sizeof(T) == 4 ? (T)G.mu_f : (T)G.mu;
+    T off = 0;
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        const int32_t c = G.T.col[k0 + k];
+        const T p = prob_at<T>(G.T, k0 + k);
+        S.col[k * G.n + i] = c;
+        S.p64[k * G.n + i] = G.T.prob[k0 + k];
+        if constexpr (sizeof(T) == 4) S.p32[k * G.n + i] = mu * p;
+        if (c != i) off += mu * p;
+    }
+    S.leak64[i] = G.T.leak[row];
+    S.leak32[i] = G.T.leak32[row];
+    const T leak = sizeof(T) == 4 ? (T)G.T.leak32[row] : (T)G.T.leak[row];
+    ((T*)S.dinv)[i] = T(1) / (leak + off);
+    S.cur[i] = row;
+}
+
+// sum_k p_k v(col_k) and (A e)_i over the slot-major rows, in the order of the
+// row's entries (KC > 0: rows of exactly KC entries, known at compile time, so
+// that a row's loads are issued together; KC = 0: S.K at run time).
 template <int KC>
 __device__ __forceinline__ double row_sum_c(const Compact& S, int64_t n, int64_t i, const double* v) {
     const int K = KC > 0 ? KC : S.K;
@@ -347,123 +579,212 @@ __device__ __forceinline__ double row_sum_c(const Compact& S, int64_t n, int64_t
     if (k < K) s0 = fma(S.p64[k * n + i], v[S.col[k * n + i]], s0);
     return s0 + s1;
 }
-template <typename T, int KC>
-__device__ __forceinline__ void apply_row_c(const Game& G, const Compact& S, int64_t i, const T* e, T* Ae,
-                                            T* diag) {
+// float32: leakage form, s_i e_i + sum_k (mu p_k) (e_i - e_col).  float64:
+// e_i - mu sum_k p_k e_col, nine operations instead of 24 (float64 has the
+// bits the leakage form saves in float32).
+template <int KC>
+__device__ __forceinline__ float apply_row_c(const Game& G, const Compact& S, int64_t i, const float* e) {
     const int K = KC > 0 ? KC : S.K;
-    const int64_t n = G.n;
-    const T ei = e[i];
-    const T mu = sizeof(T) == 4 ? (T)G.mu_f : (T)G.mu;
-    const T leak = sizeof(T) == 4 ? (T)S.leak32[i] : (T)S.leak64[i];
-    T acc = leak * ei, off = 0;
+    const float ei = e[i];
+    float acc = S.leak32[i] * ei;
 #pragma unroll
-    for (int k = 0; k < K; ++k) {
-        const int32_t c = S.col[k * n + i];
-        const T p = sizeof(T) == 4 ? (T)S.p32[k * n + i] : (T)S.p64[k * n + i];
-        acc += mu * p * (ei - e[c]);
-        if (c != i) off += mu * p;
-    }
-    *Ae = acc;
-    *diag = leak + off;
+    for (int k = 0; k < K; ++k) acc = fmaf(S.p32[k * G.n + i], ei - e[S.col[k * G.n + i]], acc);
+    return acc;
 }
-template <typename T, int KC>
-__device__ __forceinline__ T diag_row_c(const Game& G, const Compact& S, int64_t i) {
-    const int K = KC > 0 ? KC : S.K;
-    const int64_t n = G.n;
-    const T mu = sizeof(T) == 4 ? (T)G.mu_f : (T)G.mu;
-    T off = 0;
-#pragma unroll
-    for (int k = 0; k < K; ++k)
-        if (S.col[k * n + i] != i) off += mu * (sizeof(T) == 4 ? (T)S.p32[k * n + i] : (T)S.p64[k * n + i]);
-    return (sizeof(T) == 4 ? (T)S.leak32[i] : (T)S.leak64[i]) + off;
+template <int KC>
+__device__ __forceinline__ double apply_row_c(const Game& G, const Compact& S, int64_t i, const double* e) {
+    return fma(-G.mu, row_sum_c<KC>(S, G.n, i, e), e[i]);
 }
 
 // Execution context of one game's policy iteration: which threads share the
 // work, how they synchronise, and where the correction vectors live.  The
 // block context runs a game inside one thread block (vectors in shared
 // memory); the grid context spreads one game over a cooperative grid (vectors
-// in global memory, bounded grid barriers, reductions through per-block
-// partials combined in a fixed order, so the result does not depend on timing).
+// in global memory, bounded grid barriers).  Maxima and counts do not depend
+// on the order they are combined in; sums are formed in a fixed order.
 template <typename T>
 struct BlockCtx {
     T *r, *e, *t;      // correction right-hand side, correction, Jacobi work vector
-    double* red_d;
-    int* red_i;
-    Compact cp{};      // not used: the rows are read in place
+    double* v;         // the iterate in shared memory (null: global)
+    RedScratch* red;
+    Compact cp{};      // slot-major selected rows (cp.col null: rows read in place)
+    int flip = 0;
     __device__ size_t begin() const { return threadIdx.x; }
     __device__ size_t stride() const { return blockDim.x; }
+    __device__ unsigned warp() const { return threadIdx.x >> 5; }
+    __device__ unsigned warps() const { return blockDim.x >> 5; }
     __device__ bool sync() { __syncthreads(); return true; }
-    __device__ double max(double v) { return block_max(v, red_d); }
-    __device__ double sum(double v) { return block_sum(v, red_d); }
-    __device__ int sumi(int v) { return block_sum(v, red_i); }
+    __device__ int turn() { return flip ^= 1; }
+    __device__ void max2(unsigned long long a, unsigned long long b, unsigned long long* A, unsigned long long* B) {
+        block_max2(a, b, *red, turn(), A, B);
+    }
+    // Sum of arr[0 .. n) in its double value, `part` this thread's share.
+    template <typename U>
+    __device__ double sum(double part, const U*, int64_t) {
+        return block_sum_double(part, *red, turn());
+    }
+    __device__ int sumi(int v) { return block_sum_int(v, *red, turn()); }
     __device__ bool failed() const { return false; }
     __device__ bool leader() const { return threadIdx.x == 0; }
+    // The float32 copy of v that the improvement gathers from: in shared memory.
+    __device__ const float* gather_copy(const Game& G, const BatchOut&, const double* vv) {
+        float* c = (float*)t;
+        for (int64_t i = threadIdx.x; i < G.n; i += blockDim.x) c[i] = f64_to_f32(vv[i]);
+        __syncthreads();
+        return c;
+    }
 };
+
+// f64 of a value of the relaxation's type, float32 widened on the integer pipe.
+__device__ __forceinline__ double as_f64(float x) { return f32_to_f64(x); }
+__device__ __forceinline__ double as_f64(double x) { return x; }
 
 template <typename T>
 struct GridCtx {
     T *r, *e, *t;
     double* part;      // [2][gridDim.x] per-block partials (alternating)
-    GridBarrier* bar;
+    GridScal* gs;      // barrier and the reductions' slots
     Compact cp;        // slot-major selected rows (cp.col null: rows read in place)
-    double* red_d;
-    int flip;
+    RedScratch* red;
+    int flip, slot;
     bool bad;
-    __device__ size_t begin() const { return (size_t)blockIdx.x * blockDim.x + threadIdx.x; }
+    // Warp w of every block comes before warp w + 1 of any block: a small
+    // game's states are spread over all the blocks' SMs.
+    __device__ unsigned warp() const { return (threadIdx.x >> 5) * gridDim.x + blockIdx.x; }
+    __device__ unsigned warps() const { return gridDim.x * (blockDim.x >> 5); }
+    __device__ size_t begin() const { return (size_t)warp() * 32 + (threadIdx.x & 31); }
     __device__ size_t stride() const { return (size_t)gridDim.x * blockDim.x; }
     __device__ bool sync() {
-        if (!bad) bad = !GridSync{bar, gridDim.x}.sync();
+        if (!bad) bad = !GridSync{&gs->bar, gridDim.x}.sync();
         return !bad;
     }
-    __device__ double combine(double v, bool is_max) {
-        v = is_max ? block_max(v, red_d) : block_sum(v, red_d);
-        double* P = part + (size_t)flip * gridDim.x;
-        flip ^= 1;
-        if (threadIdx.x == 0) P[blockIdx.x] = v;
+    __device__ int turn() { return flip ^= 1; }
+    // Three slots in turn: reduction t uses slot t mod 3 and clears the next
+    // one, whose last readers have passed the barrier before this one's.
+    __device__ int take_slot() {
+        const int k = slot;
+        slot = slot == 2 ? 0 : slot + 1;
+        if (leader()) {
+            gs->mx[slot][0] = 0ull;
+            gs->mx[slot][1] = 0ull;
+            gs->cnt[slot] = 0;
+        }
+        return k;
+    }
+    __device__ void max2(unsigned long long a, unsigned long long b, unsigned long long* A, unsigned long long* B) {
+        const int k = take_slot();
+        block_max2(a, b, *red, turn(), A, B);
+        if (threadIdx.x == 0) {
+            atomicMax(&gs->mx[k][0], *A);
+            atomicMax(&gs->mx[k][1], *B);
+        }
+        if (!sync()) return;
+        *A = __ldcg(&gs->mx[k][0]);
+        *B = __ldcg(&gs->mx[k][1]);
+    }
+    __device__ int sumi(int v) {
+        const int k = take_slot();
+        v = block_sum_int(v, *red, turn());
+        if (threadIdx.x == 0 && v) atomicAdd(&gs->cnt[k], v);
+        if (!sync()) return 0;
+        return __ldcg(&gs->cnt[k]);
+    }
+    // Games of the size a batch solves by one block: every block sums the whole
+    // array itself, in the order one block of this size sums its own game, so
+    // that a game solved alone and in a batch gives the same bits.  Larger
+    // games: per-block partials combined in block order.
+    template <typename U>
+    __device__ double sum(double p, const U* arr, int64_t n) {
+        if (n < kGameBatchedStates) {
+            if (!sync()) return 0.0;
+            double acc = 0.0;
+            for (int64_t i = threadIdx.x; i < n; i += blockDim.x) acc += as_f64(__ldcg(arr + i));
+            return block_sum_double(acc, *red, turn());
+        }
+        const int f = turn();
+        p = block_sum_double(p, *red, f);
+        double* P = part + (size_t)f * gridDim.x;
+        if (threadIdx.x == 0) P[blockIdx.x] = p;
         if (!sync()) return 0.0;
         double acc = 0.0;
-        for (unsigned k = threadIdx.x & 31; k < gridDim.x; k += 32) {
-            const double p = __ldcg(P + k);
-            acc = is_max ? fmax(acc, p) : acc + p;
-        }
-        return is_max ? warp_maxd(acc) : warp_sum(acc);
+        for (unsigned k = threadIdx.x & 31; k < gridDim.x; k += 32) acc += __ldcg(P + k);
+        return warp_sum(acc);
     }
-    __device__ double max(double v) { return combine(v, true); }
-    __device__ double sum(double v) { return combine(v, false); }
-    __device__ int sumi(int v) { return (int)combine((double)v, false); }
     __device__ bool failed() const { return bad; }
     __device__ bool leader() const { return blockIdx.x == 0 && threadIdx.x == 0; }
+    __device__ const float* gather_copy(const Game& G, const BatchOut& O, const double*) { return O.v32 + G.x0; }
 };
 
-// float64 residual rhs - (v - mu M v) -> C.r; returns |r|_inf, sets *vmax.
-// With jacobi0, also the correction's first Jacobi sweep from zero,
-// e = r / diag -> C.e (the V(1,1) cycle below starts from it).
-template <typename T, class Ctx>
-__device__ double check(const Game& G, const BatchOut& O, const double* v, Ctx& C, double* vmax,
-                        bool jacobi0 = false) {
-    // maxima on the bit patterns, conversions on the integer pipe
+// State of the policy evaluation: the last residual check's |r|_inf and
+// |v|_inf and the sum of the system's row sums.
+template <typename T>
+struct Eval {
+    double res, vm;
+    T asum;
+};
+
+__device__ __forceinline__ unsigned long long abs_bits(double x) { return bits_of(x) & 0x7fffffffffffffffull; }
+
+// One state's part of the residual check: r = rhs - (v - mu M v) (float64),
+// C.r = r and, with jacobi0, the correction's first Jacobi sweep from zero,
+// C.e = r / diag.  KC as for row_sum_c; KC < 0: the row is read in place.
+template <typename T, int KC, class Ctx>
+__device__ __forceinline__ double check_state(const Game& G, const BatchOut& O, const double* v, const Ctx& C,
+                                              int64_t i, bool jacobi0) {
+    double Mv;
+    if constexpr (KC >= 0) Mv = row_sum_c<KC>(C.cp, G.n, i, v);
+    else Mv = row_sum(G, O.sel[G.x0 + i], v);
+    const double r = O.rhs[G.x0 + i] - (v[i] - G.mu * Mv);
+    T rt;
+    if constexpr (sizeof(T) == 4) rt = f64_to_f32(r);
+    else rt = r;
+    C.r[i] = rt;
+    if constexpr (KC >= 0) C.e[i] = rt * ((const T*)C.cp.dinv)[i];
+    else if (jacobi0) C.e[i] = rt / diag_row<T>(G, O, i);
+    return r;
+}
+
+// float64 residual check: fills E.res and E.vm.  fresh: the policies may have
+// changed since the last check; changed rows are copied slot-major first and
+// E.asum (the Galerkin operator of the constant vector) is formed.
+template <typename T, int KC, class Ctx>
+__device__ __noinline__ void check_k(const Game& G, const BatchOut& O, const double* v, Ctx& C, bool fresh,
+                                     bool jacobi0, Eval<T>& E) {
     unsigned long long rm = 0, vm = 0;
-    const int cpt = C.cp.col == nullptr ? 0 : C.cp.K == 8 ? 2 : 1;   // 2: rows of 8 entries
+    double part = 0.0;
+    if (fresh) {
+        for (int64_t i = C.begin(); i < G.n; i += C.stride()) {
+            const int64_t row = O.sel[G.x0 + i];
+            if constexpr (KC >= 0) {
+                if (C.cp.cur[i] != row) compact_row<T, KC>(G, C.cp, i, row);
+                part += C.cp.leak64[i];
+            } else {
+                const double l = G.T.leak[row];
+                O.leaksel[G.x0 + i] = l;
+                part += l;
+            }
+        }
+    }
     for (int64_t i = C.begin(); i < G.n; i += C.stride()) {
-        const double Mv = cpt == 2   ? row_sum_c<8>(C.cp, G.n, i, v)
-                          : cpt == 1 ? row_sum_c<0>(C.cp, G.n, i, v)
-                                     : row_sum(G, O.sel[G.x0 + i], v);
-        const double r = O.rhs[G.x0 + i] - (v[i] - G.mu * Mv);
-        T rt;
-        if constexpr (sizeof(T) == 4) rt = f64_to_f32(r);
-        else rt = r;
-        C.r[i] = rt;
-        if (jacobi0)
-            C.e[i] = rt / (cpt == 2   ? diag_row_c<T, 8>(G, C.cp, i)
-                           : cpt == 1 ? diag_row_c<T, 0>(G, C.cp, i)
-                                      : diag_row<T>(G, O, i));
-        const unsigned long long rb = bits_of(r) & 0x7fffffffffffffffull;
-        const unsigned long long vb = bits_of(v[i]) & 0x7fffffffffffffffull;
+        const unsigned long long rb = abs_bits(check_state<T, KC>(G, O, v, C, i, jacobi0));
+        const unsigned long long vb = abs_bits(v[i]);
         rm = rb > rm ? rb : rm;
         vm = vb > vm ? vb : vm;
     }
-    *vmax = C.max(from_bits(vm));
-    return C.max(from_bits(rm));
+    unsigned long long R, V;
+    C.max2(rm, vm, &R, &V);
+    E.res = from_bits(R);
+    E.vm = from_bits(V);
+    if (fresh && !C.failed())
+        E.asum = (T)C.sum(part, KC >= 0 ? (const double*)C.cp.leak64 : (const double*)O.leaksel + G.x0, G.n);
+}
+
+template <typename T, class Ctx>
+__device__ __forceinline__ void check(const Game& G, const BatchOut& O, const double* v, Ctx& C, bool fresh,
+                                      bool jacobi0, Eval<T>& E) {
+    if (C.cp.col == nullptr) check_k<T, -1>(G, O, v, C, fresh, jacobi0, E);
+    else if (C.cp.K == 8) check_k<T, 8>(G, O, v, C, fresh, jacobi0, E);
+    else check_k<T, 0>(G, O, v, C, fresh, jacobi0, E);
 }
 
 // One two-level cycle on A e = r from e = 0, then v += e.  Returns false if a
@@ -493,10 +814,11 @@ __device__ bool cycle(const Game& G, const BatchOut& O, double* v, Ctx& C, T asu
     for (int64_t i = C.begin(); i < G.n; i += C.stride()) {
         T Ae, d;
         apply_row<T>(G, O, i, C.e, &Ae, &d);
-        if constexpr (sizeof(T) == 4) part += f32_to_f64(C.r[i] - Ae);
-        else part += (double)(C.r[i] - Ae);
+        const T q = C.r[i] - Ae;
+        C.t[i] = q;
+        part += as_f64(q);
     }
-    const double tot = C.sum(part);
+    const double tot = C.sum(part, C.t, G.n);
     if (C.failed()) return false;
     const T c = asum != T(0) ? (T)(tot / (double)asum) : T(0);
     for (int64_t i = C.begin(); i < G.n; i += C.stride()) C.e[i] += c;
@@ -513,9 +835,7 @@ __device__ bool cycle(const Game& G, const BatchOut& O, double* v, Ctx& C, T asu
     }
     float* v32 = O.v32 + G.x0;
     for (int64_t i = C.begin(); i < G.n; i += C.stride()) {
-        double vi = v[i];
-        if constexpr (sizeof(T) == 4) vi += f32_to_f64(C.e[i]);
-        else vi += C.e[i];
+        const double vi = v[i] + as_f64(C.e[i]);
         v[i] = vi;
         v32[i] = f64_to_f32(vi);
     }
@@ -528,41 +848,48 @@ __device__ bool cycle(const Game& G, const BatchOut& O, double* v, Ctx& C, T asu
 // and, since A 1 is the leakage s of each row, A e2 = A e1 + c s without
 // another product; the post-sweep e = e2 + (r - A e2) / diag and v += e close
 // the cycle.  Same iteration as cycle() with nu1 = nu2 = 1.
-template <typename T, class Ctx>
-__device__ bool cycle11(const Game& G, const BatchOut& O, double* v, Ctx& C, T asum) {
-    const int cpt = C.cp.col == nullptr ? 0 : C.cp.K == 8 ? 2 : 1;   // 2: rows of 8 entries
+template <typename T, int KC, class Ctx>
+__device__ __noinline__ bool cycle11_k(const Game& G, const BatchOut& O, double* v, Ctx& C, T asum) {
     double part = 0.0;
     for (int64_t i = C.begin(); i < G.n; i += C.stride()) {
-        T Ae, d;
-        if (cpt == 2) apply_row_c<T, 8>(G, C.cp, i, C.e, &Ae, &d);
-        else if (cpt == 1) apply_row_c<T, 0>(G, C.cp, i, C.e, &Ae, &d);
-        else apply_row<T>(G, O, i, C.e, &Ae, &d);
-        const T q = C.r[i] - Ae;
-        if constexpr (sizeof(T) == 4) part += f32_to_f64(q);
-        else part += (double)q;
+        T q;
+        if constexpr (KC >= 0) {
+            q = C.r[i] - apply_row_c<KC>(G, C.cp, i, C.e);
+        } else {
+            T Ae, d;
+            apply_row<T>(G, O, i, C.e, &Ae, &d);
+            q = C.r[i] - Ae;
+            C.t[i] = d;
+        }
+        part += as_f64(q);
         C.r[i] = q;   // r - A e1 (r itself is not needed again)
-        C.t[i] = d;
     }
-    const double tot = C.sum(part);
+    const double tot = C.sum(part, C.r, G.n);
     if (C.failed()) return false;
     const T c = asum != T(0) ? (T)(tot / (double)asum) : T(0);
     float* v32 = O.v32 + G.x0;
     for (int64_t i = C.begin(); i < G.n; i += C.stride()) {
-        T s;
-        if (cpt) {
-            s = sizeof(T) == 4 ? (T)C.cp.leak32[i] : (T)C.cp.leak64[i];
+        T e;
+        if constexpr (KC >= 0) {
+            const T s = sizeof(T) == 4 ? (T)C.cp.leak32[i] : (T)C.cp.leak64[i];
+            e = C.e[i] + c + (C.r[i] - c * s) * ((const T*)C.cp.dinv)[i];
         } else {
             const int64_t row = O.sel[G.x0 + i];
-            s = sizeof(T) == 4 ? (T)G.T.leak32[row] : (T)G.T.leak[row];
+            const T s = sizeof(T) == 4 ? (T)G.T.leak32[row] : (T)G.T.leak[row];
+            e = C.e[i] + c + (C.r[i] - c * s) / C.t[i];
         }
-        const T e = C.e[i] + c + (C.r[i] - c * s) / C.t[i];
-        double vi = v[i];
-        if constexpr (sizeof(T) == 4) vi += f32_to_f64(e);
-        else vi += e;
+        const double vi = v[i] + as_f64(e);
         v[i] = vi;
         v32[i] = f64_to_f32(vi);
     }
     return C.sync();
+}
+
+template <typename T, class Ctx>
+__device__ __forceinline__ bool cycle11(const Game& G, const BatchOut& O, double* v, Ctx& C, T asum) {
+    if (C.cp.col == nullptr) return cycle11_k<T, -1>(G, O, v, C, asum);
+    if (C.cp.K == 8) return cycle11_k<T, 8>(G, O, v, C, asum);
+    return cycle11_k<T, 0>(G, O, v, C, asum);
 }
 
 // Why a policy evaluation stopped.
@@ -570,77 +897,66 @@ enum { kEvalExact = 0, kEvalInexact = 1, kEvalCapped = 2 };
 
 // Policy evaluation: cycles until the float64 floor / tolerance (kEvalExact),
 // a residual drop by rel_tol (kEvalInexact) or max_cycles (kEvalCapped).
+// checked: E and the correction vectors hold the check of the current v and
+// policies already (the last evaluation's, or the outer improvement's).
 template <typename T, class Ctx>
-__device__ int evaluate(const Game& G, const BatchOut& O, const BatchOpts& P, double* v, Ctx& C,
-                        double rel_tol, int* cycles) {
+__device__ int evaluate(const Game& G, const BatchOut& O, const BatchOpts& P, double* v, Ctx& C, bool checked,
+                        double rel_tol, int* cycles, Eval<T>& E) {
     const bool v11 = P.nu1 == 1 && P.nu2 == 1;
-    if (!v11) C.cp.col = nullptr;   // the general cycle reads the rows in place
-    double part = 0.0;
-    for (int64_t i = C.begin(); i < G.n; i += C.stride()) {
-        const int64_t row = O.sel[G.x0 + i];
-        part += G.T.leak[row];
-        if (C.cp.col) {   // the selected rows, slot-major
-            const Compact& S = C.cp;
-            const int64_t k0 = row * S.K;
-            for (int k = 0; k < S.K; ++k) {
-                S.col[k * G.n + i] = G.T.col[k0 + k];
-                S.p64[k * G.n + i] = G.T.prob[k0 + k];
-                S.p32[k * G.n + i] = prob_at<float>(G.T, k0 + k);
-            }
-            S.leak64[i] = G.T.leak[row];
-            S.leak32[i] = G.T.leak32[row];
-        }
-    }
-    const T asum = (T)C.sum(part);   // (its barrier also publishes the gathered rows)
-    double vm;
-    double res = check<T>(G, O, v, C, &vm, v11);
-    const double res0 = res;
-    double prev = res;
+    if (!checked) check<T>(G, O, v, C, true, v11, E);
+    const double res0 = E.res;
+    double prev = E.res;
     int slow = 0;
     for (int cyc = 0;; ++cyc) {
         if (C.failed()) return kEvalExact;   // a barrier gave up: the caller leaves
-        if (res <= P.lin_tol * fmax(vm, 1e-300) || res == 0.0) return kEvalExact;
+        if (E.res <= P.lin_tol * fmax(E.vm, 1e-300) || E.res == 0.0) return kEvalExact;
         if (cyc > 0) {
-            slow = res > 0.5 * prev ? slow + 1 : 0;
-            if (slow >= 2 && res < 1e-12 * fmax(vm, 1e-300)) return kEvalExact;
-            if (res <= rel_tol * res0) return kEvalInexact;
-            prev = fmin(prev, res);
+            slow = E.res > 0.5 * prev ? slow + 1 : 0;
+            if (slow >= 2 && E.res < 1e-12 * fmax(E.vm, 1e-300)) return kEvalExact;
+            if (E.res <= rel_tol * res0) return kEvalInexact;
+            prev = fmin(prev, E.res);
         }
         if (cyc >= P.max_cycles) return kEvalCapped;
-        if (!(v11 ? cycle11<T>(G, O, v, C, asum) : cycle<T>(G, O, v, C, asum, P.nu1, P.nu2)))
+        if (!(v11 ? cycle11<T>(G, O, v, C, E.asum) : cycle<T>(G, O, v, C, E.asum, P.nu1, P.nu2)))
             return kEvalExact;
         ++*cycles;
-        res = check<T>(G, O, v, C, &vm, v11);
+        check<T>(G, O, v, C, false, v11, E);
     }
 }
 
+// Policy improvement of the whole game; vm is |v|_inf.  Returns the number of
+// changed policy entries; every thread of the context has passed a barrier
+// after the last write.
 template <class Ctx>
-__device__ int improve_all(const Game& G, const BatchOut& O, int mode, const double* v, Ctx& C,
-                           double* res_out) {
-    unsigned long long vb = 0;
-    for (int64_t i = C.begin(); i < G.n; i += C.stride()) {
-        const unsigned long long b = bits_of(v[i]) & 0x7fffffffffffffffull;
-        vb = b > vb ? b : vb;
-    }
-    const double vm = C.max(from_bits(vb));
+__device__ int improve_all(const Game& G, const BatchOut& O, int mode, const double* v, double vm, Ctx& C) {
     const double tau = 1e-13 * fmax(1.0, vm);
-    const float tauf = f64_to_f32(tau), vmaxf = f64_to_f32(vm);
+    const float vmaxf = f64_to_f32(vm);
     int changed = 0;
-    unsigned long long rb = 0;
-    for (int64_t i = C.begin(); i < G.n; i += C.stride()) {
-        double r = 0.0;
-        changed += improve_state(G, O, mode, i, tau, tauf, vmaxf, v, &r);
-        const unsigned long long b = bits_of(r);
-        rb = b > rb ? b : rb;
+    if (rows_in_lanes(G.T.m1, G.T.m2)) {
+        const float* v32 = C.gather_copy(G, O, v);
+        const bool wide = G.T.k_uniform == 8;
+        if (mode == 1) changed = wide ? improve_rows<8, 1>(G, O, tau, vmaxf, v, v32, C)
+                                      : improve_rows<0, 1>(G, O, tau, vmaxf, v, v32, C);
+        else if (mode == 0) changed = wide ? improve_rows<8, 0>(G, O, tau, vmaxf, v, v32, C)
+                                           : improve_rows<0, 0>(G, O, tau, vmaxf, v, v32, C);
+        else changed = wide ? improve_rows<8, 2>(G, O, tau, vmaxf, v, v32, C)
+                            : improve_rows<0, 2>(G, O, tau, vmaxf, v, v32, C);
+    } else {
+        const float tauf = f64_to_f32(tau);
+        for (int64_t i = C.begin(); i < G.n; i += C.stride()) {
+            double r;
+            changed += improve_state(G, O, mode, i, tau, tauf, vmaxf, v, &r);
+        }
     }
-    if (res_out) *res_out = C.max(from_bits(rb));
     return C.sumi(changed);
 }
 
 // Algorithm 2 with Algorithm 1 inside for game g (see the Isaacs driver for
 // the stopping rules and the exact confirmation of inexact evaluations).
+// |F(v) - v| of an outer improvement is the residual of the system its
+// policies select, so it comes from that system's first residual check.
 template <typename T, class Ctx>
-__device__ void solve_game(const BatchArgs& B, int g, Ctx& C) {
+__device__ void solve_game(const BatchArgs& B, int g, Ctx& C, double* vs) {
     Game G;
     G.T = B.T;
     G.x0 = B.st_off[g];
@@ -651,57 +967,74 @@ __device__ void solve_game(const BatchArgs& B, int g, Ctx& C) {
     G.mu_f = f64_to_f32(G.mu);
     const BatchOut& O = B.out;
     const BatchOpts& P = B.opt;
-    double* v = O.v + G.x0;
+    const bool v11 = P.nu1 == 1 && P.nu2 == 1;
+    if (!v11) C.cp.col = nullptr;   // the general cycle reads the rows in place
+    double* v = vs ? vs : O.v + G.x0;
     const int a0 = P.default_alpha;
     for (int64_t i = C.begin(); i < G.n; i += C.stride()) {
         v[i] = 0.0;
         O.v32[G.x0 + i] = 0.0f;
         O.alpha[G.x0 + i] = (uint8_t)(a0 < G.T.m1 ? a0 : 0);
         for (int a = 0; a < G.T.m1; ++a) O.beta[(G.x0 + i) * G.T.m1 + a] = 0;
+        if (C.cp.col) C.cp.cur[i] = -1;
     }
     if (!C.sync()) return;
-    improve_all(G, O, 2, v, C, (double*)nullptr);   // MIN's first reply, assembly
-    if (!C.sync()) return;
+    improve_all(G, O, 2, v, 0.0, C);   // MIN's first reply, assembly
+    if (C.failed()) return;
     int outer = 0, systems = 0, cycles = 0, converged = 0;
     bool capped = false;   // an evaluation stopped at max_cycles: no decision may rest on it
-    double res = 0.0;
+    bool checked = false;
+    Eval<T> E{0.0, 0.0, T(0)};
     while (true) {
         for (int j = 0; j < P.max_inner; ++j) {
-            const int why = evaluate<T>(G, O, P, v, C, P.pi_rtol, &cycles);
+            const int why = evaluate<T>(G, O, P, v, C, checked, P.pi_rtol, &cycles, E);
+            checked = true;
             ++systems;
-            if (!C.sync()) return;
+            if (C.failed()) return;
             if (why == kEvalCapped) {
                 capped = true;
                 break;
             }
-            if (improve_all(G, O, 1, v, C, (double*)nullptr) != 0) continue;
-            if (!C.sync()) return;
+            const int ch = improve_all(G, O, 1, v, E.vm, C);
+            if (C.failed()) return;
+            if (ch != 0) {
+                checked = false;
+                continue;
+            }
             if (why == kEvalInexact) {
-                if (evaluate<T>(G, O, P, v, C, 0.0, &cycles) == kEvalCapped) capped = true;
-                if (!C.sync()) return;
+                if (evaluate<T>(G, O, P, v, C, true, 0.0, &cycles, E) == kEvalCapped) capped = true;
+                if (C.failed()) return;
                 if (capped) break;
-                if (improve_all(G, O, 1, v, C, (double*)nullptr) != 0) continue;
-                if (!C.sync()) return;
+                const int ch2 = improve_all(G, O, 1, v, E.vm, C);
+                if (C.failed()) return;
+                if (ch2 != 0) {
+                    checked = false;
+                    continue;
+                }
             }
             break;
         }
         ++outer;
-        if (!C.sync()) return;
-        const int ach = improve_all(G, O, 0, v, C, &res);
-        if (!C.sync()) return;
-        if (capped) break;   // unconverged; v is the best iterate, res its residual
-        if (res <= P.eps || ach == 0) {
+        const int ach = improve_all(G, O, 0, v, E.vm, C);
+        if (C.failed()) return;
+        check<T>(G, O, v, C, true, v11, E);
+        if (C.failed()) return;
+        checked = true;
+        if (capped) break;   // unconverged; v is the best iterate, E.res its residual
+        if (E.res <= P.eps || ach == 0) {
             converged = 1;
             break;
         }
         if (outer >= P.max_outer) break;
     }
+    if (vs)
+        for (int64_t i = C.begin(); i < G.n; i += C.stride()) O.v[G.x0 + i] = v[i];
     if (C.leader()) {
         O.gstats[4 * g + 0] = outer;
         O.gstats[4 * g + 1] = systems;
         O.gstats[4 * g + 2] = cycles;
         O.gstats[4 * g + 3] = converged;
-        O.gres[g] = res;
+        O.gres[g] = E.res;
     }
     C.sync();
 }
@@ -712,8 +1045,7 @@ template <typename T, int NT>
 __global__ void __launch_bounds__(NT, 512 / NT) k_games_pi(const __grid_constant__ BatchArgs B) {
     extern __shared__ __align__(16) char smem[];
     __shared__ int s_game;
-    __shared__ double red_d[32];
-    __shared__ int red_i[32];
+    __shared__ RedScratch red;
     while (true) {
         if (threadIdx.x == 0) {
             const int q = atomicAdd(B.queue, 1);
@@ -724,36 +1056,37 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_games_pi(const __grid_constant
         __syncthreads();
         if (g < 0) break;
         BlockCtx<T> C;
-        C.r = (T*)smem;
+        double* vs = B.v_in_smem ? (double*)smem : nullptr;
+        C.r = (T*)(smem + (vs ? sizeof(double) * (size_t)B.max_n : 0));
         C.e = C.r + B.max_n;
         C.t = C.e + B.max_n;
-        C.red_d = red_d;
-        C.red_i = red_i;
+        C.red = &red;
         if (B.cp.col) {   // this game's part of the slot-major rows
             const int64_t x0 = B.st_off[g], K = B.cp.K;
             C.cp = Compact{B.cp.col + x0 * K, B.cp.p32 + x0 * K, B.cp.p64 + x0 * K, B.cp.leak32 + x0,
-                           B.cp.leak64 + x0, B.cp.K};
+                           B.cp.leak64 + x0, B.cp.dinv + x0, B.cp.cur + x0, B.cp.K};
         }
-        solve_game<T>(B, g, C);
+        solve_game<T>(B, g, C, vs);
     }
 }
 
-// One game over a cooperative grid (games too large for one block).
+// One game over a cooperative grid.
 template <typename T>
 __global__ void __launch_bounds__(kThreads) k_game_pi_grid(const __grid_constant__ BatchArgs B,
                                                            GridWork W) {
-    __shared__ double red_d[32];
+    __shared__ RedScratch red;
     GridCtx<T> C;
     C.r = (T*)W.r;
     C.e = (T*)W.e;
     C.t = (T*)W.t;
     C.part = W.part;
-    C.bar = W.bar;
+    C.gs = W.gs;
     C.cp = W.cp;
-    C.red_d = red_d;
+    C.red = &red;
     C.flip = 0;
+    C.slot = 0;
     C.bad = false;
-    solve_game<T>(B, 0, C);
+    solve_game<T>(B, 0, C, nullptr);
 }
 
 // One policy improvement of game 0 over the whole grid (the algebraic
@@ -827,7 +1160,8 @@ int game_grid_blocks(int64_t n, int cap) {
         GS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_game_pi_grid<double>, kThreads, 0));
         per_sm = std::max(1, std::min(a, b));
     }
-    int blocks = (int)std::min<int64_t>((n + kThreads - 1) / kThreads, (int64_t)per_sm * sms);
+    // one warp of states per block until every SM has one
+    int blocks = (int)std::min<int64_t>((n + 31) / 32, (int64_t)per_sm * sms);
     if (cap > 0) blocks = std::min(blocks, cap);
     return std::max(1, blocks);
 }
@@ -840,12 +1174,17 @@ void launch_game_pi_grid(const BatchArgs& B, const GridWork& W, int blocks, bool
     note_launches(1);
 }
 
-size_t games_smem_bytes(int max_n, bool mixed) {
-    return (size_t)3 * max_n * (mixed ? sizeof(float) : sizeof(double));
+size_t games_smem_bytes(int max_n, bool mixed, bool v_in_smem) {
+    return (size_t)max_n * (3 * (mixed ? sizeof(float) : sizeof(double)) + (v_in_smem ? sizeof(double) : 0));
 }
 
-void launch_games_pi(const BatchArgs& B, bool mixed, int threads, cudaStream_t st) {
-    const size_t smem = games_smem_bytes(B.max_n, mixed);
+void launch_games_pi(const BatchArgs& Bin, bool mixed, int threads, cudaStream_t st) {
+    // the iterate joins the correction vectors in shared memory where all
+    // 512 / threads blocks of an SM still fit
+    constexpr size_t kSmemPerSM = 224 * 1024;
+    BatchArgs B = Bin;
+    B.v_in_smem = games_smem_bytes(B.max_n, mixed, true) * (512 / threads) <= kSmemPerSM;
+    const size_t smem = games_smem_bytes(B.max_n, mixed, B.v_in_smem);
     const void* fn = threads == 256 ? (mixed ? (const void*)k_games_pi<float, 256>
                                              : (const void*)k_games_pi<double, 256>)
                                     : (mixed ? (const void*)k_games_pi<float, 512>

@@ -44,6 +44,7 @@ struct BatchOut {
     double* rhs;      // per state: its reward r^{alpha beta}
     int* gstats;      // per game: outer, systems, cycles, converged
     double* gres;     // per game: |F(v) - v|_inf at the end
+    double* leaksel;  // per state: the selected row's leakage (rows read in place)
 };
 
 struct BatchOpts {
@@ -52,16 +53,28 @@ struct BatchOpts {
 };
 
 // The selected rows of a game's policy-fixed system gathered slot-major
-// (entry k of state i at [k * n + i], n the game's states) at the start of
-// each evaluation, so that the cycles read them coalesced and without the
-// selection's indirection.  Only for rows of one length K (col null: not used).
+// (entry k of state i at [k * n + i], n the game's states), so that the cycles
+// read them coalesced and without the selection's indirection; a state's copy
+// is renewed when its selected row has changed.  Only for rows of one length K
+// (col null: not used).
 struct Compact {
     int32_t* col;
-    float* p32;          // the relaxation's copy (float32, or bfloat16 widened)
+    float* p32;          // mu p in the relaxation's precision (float32 cycles only)
     double* p64;
     float* leak32;
     double* leak64;
+    double* dinv;        // inverse diagonal, in the relaxation's type (float32: first half)
+    int64_t* cur;        // the row the state's copy holds
     int K;
+};
+
+// Grid-wide kernel: the barrier and the slots of its order-free reductions
+// (zeroed before the launch).
+struct GridScal {
+    GridBarrier bar;
+    unsigned long long mx[3][2];
+    int cnt[3];
+    int pad;
 };
 
 struct BatchArgs {
@@ -76,13 +89,14 @@ struct BatchArgs {
     const int* order;       // queue position -> game, `count` entries (one-block kernel)
     Compact cp;             // one-block kernel: slot-major rows of all games, game g's at
                             // state offset st_off[g] (cp.col null: rows read in place)
+    bool v_in_smem;         // one-block kernel: the iterate lives in shared memory
 };
 
 // Work vectors of the grid-wide single-game kernel (global memory).
 struct GridWork {
     void *r, *e, *t;     // n elements each (float32 or float64)
     double* part;        // 2 x (blocks) per-block partials
-    GridBarrier* bar;    // zeroed before the launch
+    GridScal* gs;        // zeroed before the launch
     Compact cp;          // the selected rows, slot-major (cp.col null: rows read in place)
 };
 
@@ -105,7 +119,7 @@ void launch_game_validate(const GameTables& T, int count, const int64_t* st_off,
 void launch_game_prepare(const GameTables& T, int count, const int64_t* st_off, int64_t rows,
                          const double* mu, double* leak, float* leak32, float* prob32,
                          __nv_bfloat16* prob16, cudaStream_t st);
-size_t games_smem_bytes(int max_n, bool mixed);
+size_t games_smem_bytes(int max_n, bool mixed, bool v_in_smem);
 // Threads per game of the one-block kernel's instantiations.
 constexpr int kBatchShapes[2] = {256, 512};
 // Batches of at least this many games autotune the shape on a sample of this many.
@@ -124,7 +138,10 @@ void launch_game_pi_grid(const BatchArgs& B, const GridWork& W, int blocks, bool
 void launch_game_improve_one(const BatchArgs& B, int mode, int64_t n, int* scal, cudaStream_t st);
 
 // Games of at least this many states, set alone, run on the whole grid.
-constexpr int64_t kGameGridMinStates = 4096;
+constexpr int64_t kGameGridMinStates = 512;
+// Games below this size that wait together at a server are solved as a batch,
+// one block each, and must give the bits they give alone (GridCtx::sum).
+constexpr int64_t kGameBatchedStates = 4096;
 
 // Random games drawn on the device (randgame.cu): n states, m1 x m2 rows per
 // state, k <= 8 successors per row; CSR table into device buffers of

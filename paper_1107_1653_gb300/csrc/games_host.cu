@@ -93,6 +93,7 @@ std::unique_ptr<Problem> build_game_problem(gs_solver* s, int count, int m1, int
     G->beta = ar.alloc<uint8_t>(n_total * m1);
     G->sel = ar.alloc<int64_t>(n_total);
     G->rhs = ar.alloc<double>(n_total);
+    G->leaksel = ar.alloc<double>(n_total);
     G->gstats = ar.alloc<int>(4 * (size_t)count);
     G->gres = ar.alloc<double>(count);
     G->queue = ar.alloc<int>(2);
@@ -116,7 +117,7 @@ std::unique_ptr<Problem> build_game_problem(gs_solver* s, int count, int m1, int
         G->we = ar.alloc<double>(n_total);
         G->wt = ar.alloc<double>(n_total);
         G->part = ar.alloc<double>(2 * 152 * 64);
-        G->bar = ar.alloc<GridBarrier>(1);
+        G->gscal = ar.alloc<GridScal>(1);
     }
     GS_CUDA(cudaMemcpyAsync(G->st_off, off.data(), sizeof(int64_t) * (count + 1),
                             cudaMemcpyHostToDevice, st));
@@ -156,6 +157,8 @@ std::unique_ptr<Problem> build_game_problem(gs_solver* s, int count, int m1, int
             G->cp.p64 = ar.alloc<double>(m);
             G->cp.leak32 = ar.alloc<float>(n_total);
             G->cp.leak64 = ar.alloc<double>(n_total);
+            G->cp.dinv = ar.alloc<double>(n_total);
+            G->cp.cur = ar.alloc<int64_t>(n_total);
             G->cp.K = (int)G->k_uniform;
         }
     }
@@ -228,7 +231,7 @@ gs_status run_games(gs_solver* s, gs_solve_stats* stats) {
     const bool mixed = s->opt.precision != GS_PREC_FP64;
     BatchArgs B{};
     B.T = G.tables();
-    B.out = {G.v, G.v32, G.alpha, G.beta, G.sel, G.rhs, G.gstats, G.gres};
+    B.out = {G.v, G.v32, G.alpha, G.beta, G.sel, G.rhs, G.gstats, G.gres, G.leaksel};
     B.opt.max_outer = s->opt.max_outer;
     B.opt.max_inner = s->opt.max_inner;
     B.opt.max_cycles = s->opt.max_cycles;
@@ -251,10 +254,10 @@ gs_status run_games(gs_solver* s, gs_solve_stats* stats) {
     GS_CUDA(cudaEventCreate(&e0));
     GS_CUDA(cudaEventCreate(&e1));
     GS_CUDA(cudaMemsetAsync(G.queue, 0, sizeof(int), st));
-    if (G.grid) GS_CUDA(cudaMemsetAsync(G.bar, 0, sizeof(GridBarrier), st));
+    if (G.grid) GS_CUDA(cudaMemsetAsync(G.gscal, 0, sizeof(GridScal), st));
     GS_CUDA(cudaEventRecord(e0, st));
     if (G.grid) {
-        GridWork W{G.wr, G.we, G.wt, G.part, G.bar, G.cp};
+        GridWork W{G.wr, G.we, G.wt, G.part, G.gscal, G.cp};
         const int blocks = std::min(game_grid_blocks(G.n_total, s->opt.grid_blocks), 152 * 64);
         launch_game_pi_grid(B, W, blocks, mixed, st);
     } else {
@@ -268,7 +271,7 @@ gs_status run_games(gs_solver* s, gs_solve_stats* stats) {
     GS_CUDA(cudaMemcpyAsync(G.res_h.data(), G.gres, sizeof(double) * G.count,
                             cudaMemcpyDeviceToHost, st));
     GridBarrier hb{};
-    if (G.grid) GS_CUDA(cudaMemcpyAsync(&hb, G.bar, sizeof hb, cudaMemcpyDeviceToHost, st));
+    if (G.grid) GS_CUDA(cudaMemcpyAsync(&hb, &G.gscal->bar, sizeof hb, cudaMemcpyDeviceToHost, st));
     GS_CUDA(cudaStreamSynchronize(st));
     if (hb.error) {
         cudaEventDestroy(e0);

@@ -60,7 +60,7 @@ size_t estimate_bytes(const gs_request& r) {
     const size_t rows = (size_t)r.n * r.m1 * r.m2;
     // per row: leakage, reward, policy copies; per state: vectors and the
     // grid kernel's slot-major copy of the selected rows (8 entries)
-    const size_t base = rows * 32 + (size_t)r.n * 200 + (64 << 10);
+    const size_t base = rows * 32 + (size_t)r.n * 224 + (64 << 10);
     return r.kind == 3 ? base + 2 * rows * (8 + 12 * (size_t)succ_of(r)) : base;
 }
 
@@ -69,7 +69,7 @@ size_t estimate_bytes(const gs_request& r) {
 // would run alone.
 constexpr int kServeBatchMax = 256;
 bool batchable(const Request& R) {
-    return (R.spec.kind == 2 || R.spec.kind == 3) && R.spec.n < kGameGridMinStates;
+    return (R.spec.kind == 2 || R.spec.kind == 3) && R.spec.n < kGameBatchedStates;
 }
 bool same_batch(const Request& a, const Request& b) {
     return a.spec.kind == b.spec.kind && a.spec.m1 == b.spec.m1 && a.spec.m2 == b.spec.m2 &&

@@ -73,7 +73,7 @@ struct GameProblem {
     int64_t *st_off = nullptr, *row_ptr = nullptr, *sel = nullptr;
     int32_t* col = nullptr;
     double *prob = nullptr, *rew = nullptr, *leak = nullptr, *mu = nullptr, *v = nullptr,
-           *rhs = nullptr, *gres = nullptr;
+           *rhs = nullptr, *gres = nullptr, *leaksel = nullptr;
     float* prob32 = nullptr;   // rounded copy of prob: float32, or bfloat16 in its first half
     float* leak32 = nullptr;   // float32 copy of leak
     float* v32 = nullptr;      // float32 copy of v
@@ -87,7 +87,7 @@ struct GameProblem {
     int shape = 0;                         // threads per game of the last solve (0: grid)
     bool grid = false;                     // one large game on the whole grid
     double *wr = nullptr, *we = nullptr, *wt = nullptr, *part = nullptr;
-    GridBarrier* bar = nullptr;
+    GridScal* gscal = nullptr;
     Compact cp{};                          // grid: the selected rows slot-major (rows of one length)
     std::vector<int> stats_h;
     std::vector<double> res_h;
