@@ -350,13 +350,13 @@ struct Row8 {
         }
     }
     // F(v; x, a, b) in float32 (row_value_f's order of operations).
-    __device__ __forceinline__ float value(const Game& G, const float* v32, double r64) const {
+    __device__ __forceinline__ float value(const Game& G, const float* v32, float r) const {
         float vc[8], s = 0.0f;
 #pragma unroll
         for (int k = 0; k < 8; ++k) vc[k] = v32[c[k]];
 #pragma unroll
         for (int k = 0; k < 8; ++k) s = fmaf(p[k], vc[k], s);
-        return G.mu_f * s + f64_to_f32(r64);
+        return G.mu_f * s + r;
     }
 };
 
@@ -368,17 +368,18 @@ __host__ __device__ __forceinline__ bool rows_in_lanes(int m1, int m2) {
 
 // Policy improvement of a whole game with one lane per row (x, a, b): the
 // decisions and their float32 screen are those of improve_state, but a warp
-// reads its rows' entries as consecutive memory, and the minimum over b and
-// the maximum over a are taken by lane exchanges inside the state's group of
-// lanes (m1 m2 of them; the m2 of the current action in mode 1).  Bound by the
-// bytes of the rows (64 per row of 8 entries, and its reward) and the gathers
-// from v32: the one-thread-per-state form reads each row's entries one by one,
-// 16 rows apart from its neighbours'.  NE states per lane group are in flight
-// at once.  Measured per improvement, games of 4224 states on average with 4 x 4
-// actions, one block each: all actions 823 -> 221 us, MIN's reply at fixed alpha
-// 258 -> 58 us; one game of 5e5 states on the whole GPU: 892 -> 331 and 324 ->
-// 83 us.  Writes beta, sel, rhs (and alpha in mode 0); returns this thread's
-// count of changed policy entries.
+// reads its rows' entries as consecutive memory (256-bit loads), and the
+// minimum over b and the maximum over a are taken by lane exchanges inside the
+// state's group of lanes (m1 m2 of them; the m2 of the current action in mode
+// 1).  NE states per lane group are in flight at once.  Bound by the shared-
+// memory or L2 gathers from v32 and the bytes of the rows (72 per row of 8
+// entries); one lane per action walking its m2 rows issues fewer instructions
+// but touches a cache line per lane and was slower (212 and 71 us below).
+// Measured per improvement, games of 4224 states on average with 4 x 4 actions,
+// one block each: all actions 823 -> 200 us, MIN's reply at fixed alpha 258 ->
+// 55 us; one game of 5e5 states on the whole GPU: 892 -> 306 and 324 -> 80 us
+// (the first figures: one thread per state).  Writes beta, sel, rhs (and alpha
+// in mode 0); returns this thread's count of changed policy entries.
 template <int KC, int MODE, class Ctx>
 __device__ __noinline__ int improve_rows(const Game& G, const BatchOut& O, double tau, float vmaxf, const double* v,
                                          const float* v32, const Ctx& C) {
@@ -393,7 +394,7 @@ __device__ __noinline__ int improve_rows(const Game& G, const BatchOut& O, doubl
     int changed = 0;
     for (int64_t base = (int64_t)C.warp() * per * NE; base < G.n; base += (int64_t)C.warps() * per * NE) {
         int64_t st[NE], row[NE];
-        int a[NE], acur[NE];
+        int a[NE], acur[NE], bcurs[NE];
         bool ok[NE];
         double r64[NE];
         float F[NE];
@@ -409,13 +410,14 @@ __device__ __noinline__ int improve_rows(const Game& G, const BatchOut& O, doubl
             a[e] = MODE == 1 ? acur[e] : sub >> bl;
             row[e] = G.row0 + st[e] * G.R + a[e] * m2 + b;
             r64[e] = G.T.rew[row[e]];
+            bcurs[e] = O.beta[(G.x0 + st[e]) * m1 + a[e]];
         }
         if constexpr (KC == 8) {
             Row8 R8[NE];
 #pragma unroll
             for (int e = 0; e < NE; ++e) R8[e].load(G.T, row[e]);
 #pragma unroll
-            for (int e = 0; e < NE; ++e) F[e] = R8[e].value(G, v32, r64[e]);
+            for (int e = 0; e < NE; ++e) F[e] = R8[e].value(G, v32, f64_to_f32(r64[e]));
         } else {
 #pragma unroll
             for (int e = 0; e < NE; ++e) {
@@ -467,19 +469,50 @@ __device__ __noinline__ int improve_rows(const Game& G, const BatchOut& O, doubl
                     anew = ga;
                 }
             }
-            if (!ok[e]) continue;
             const int64_t x = G.x0 + st[e];
-            if (!sure) {
-                if (sub == 0) {
-                    double res;
-                    changed += improve_state_exact(G, O, MODE, st[e], tau, v, &res);
+            const int bcur = bcurs[e];
+            int bsel = first;
+            if (__any_sync(0xffffffffu, !sure)) {
+                // the exact float64 decisions (improve_state_exact's) for the
+                // states whose screen was not conclusive, a row per lane: one
+                // lane evaluating a state's rows in turn held its warp up for
+                // tens of microseconds
+                const double F64 = row_value(G, row[e], v);
+                double fb = F64;
+                int fi = b;
+                for (int o = 1; o < m2; o <<= 1) {
+                    const double b2 = __shfl_xor_sync(0xffffffffu, fb, o);
+                    const int f2 = __shfl_xor_sync(0xffffffffu, fi, o);
+                    if (b2 < fb || (b2 == fb && f2 < fi)) {
+                        fb = b2;
+                        fi = f2;
+                    }
                 }
-                continue;
+                const double fcur = __shfl_sync(0xffffffffu, F64, (lane & ~(m2 - 1)) | (bcur & (m2 - 1)));
+                const int bx = fcur - fb > tau ? fi : bcur;
+                int ax = acur[e];
+                if (MODE == 0) {
+                    double h = fb;
+                    int ha = a[e];
+                    for (int o = m2; o < grp; o <<= 1) {
+                        const double h2 = __shfl_xor_sync(0xffffffffu, h, o);
+                        const int a2 = __shfl_xor_sync(0xffffffffu, ha, o);
+                        if (h2 > h || (h2 == h && a2 < ha)) {
+                            h = h2;
+                            ha = a2;
+                        }
+                    }
+                    const double hcur = __shfl_sync(0xffffffffu, fb, (lane & ~(grp - 1)) | acur[e] << bl);
+                    ax = h - hcur > tau ? ha : acur[e];
+                }
+                if (!sure) {
+                    bsel = bx;
+                    anew = ax;
+                }
             }
-            if (b == first) {   // the lane of the chosen b of its action
-                uint8_t& bref = O.beta[x * m1 + a[e]];
-                if (bref != b) {
-                    bref = (uint8_t)b;
+            if (ok[e] && b == bsel) {   // the lane of the chosen b of its action
+                if (bcur != b) {
+                    O.beta[x * m1 + a[e]] = (uint8_t)b;
                     if (MODE == 1) ++changed;
                 }
                 if (a[e] == anew) {   // ... of the state's action
@@ -547,14 +580,27 @@ __device__ __forceinline__ void compact_row(const Game& G, const Compact& S, int
     const int64_t k0 = row * K;
     const T mu = sizeof(T) == 4 ? (T)G.mu_f : (T)G.mu;
     T off = 0;
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-        const int32_t c = G.T.col[k0 + k];
-        const T p = prob_at<T>(G.T, k0 + k);
+    auto put = [&](int k, int32_t c, double p64) {
+        T p;
+        if constexpr (sizeof(T) == 8) p = p64;
+        else p = prob_at<T>(G.T, k0 + k);
         S.col[k * G.n + i] = c;
-        S.p64[k * G.n + i] = G.T.prob[k0 + k];
+        S.p64[k * G.n + i] = p64;
         if constexpr (sizeof(T) == 4) S.p32[k * G.n + i] = mu * p;
         if (c != i) off += mu * p;
+    };
+    if constexpr (KC == 8) {
+        unsigned c[8], lo[8], hi[8];
+        load_32b(G.T.col + k0, c);
+        load_32b(G.T.prob + k0, lo);
+        load_32b(G.T.prob + k0 + 4, hi);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const unsigned* q = k < 4 ? lo : hi;
+            put(k, (int32_t)c[k], __hiloint2double((int)q[2 * (k & 3) + 1], (int)q[2 * (k & 3)]));
+        }
+    } else {
+        for (int k = 0; k < K; ++k) put(k, G.T.col[k0 + k], G.T.prob[k0 + k]);
     }
     S.leak64[i] = G.T.leak[row];
     S.leak32[i] = G.T.leak32[row];
@@ -596,6 +642,54 @@ __device__ __forceinline__ double apply_row_c(const Game& G, const Compact& S, i
     return fma(-G.mu, row_sum_c<KC>(S, G.n, i, e), e[i]);
 }
 
+// A slot-major row of 8 entries held in registers: the passes below load the
+// rows of a thread's next states while they work on the current one, D of them
+// at a time, because a pass has too few warps (16 per SM) to cover the latency
+// of its loads from L2 otherwise.  Games of 4224 states on average, one block
+// each, mixed: residual check 26.1 -> 15.7 us (its float64 operations alone take
+// 11), product with the correction 16.6 -> 8.4 us.
+template <typename P>
+struct SlotRow8 {
+    int c[8];
+    P p[8];
+    __device__ __forceinline__ void load(const int32_t* __restrict__ col, const P* __restrict__ prob, int64_t n, int64_t i) {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) c[k] = col[k * n + i];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) p[k] = prob[k * n + i];
+    }
+};
+// sum_k p_k v(col_k), in row_sum_c's order.
+__device__ __forceinline__ double row_sum_r(const SlotRow8<double>& R, const double* v) {
+    double x[8], s0 = 0.0, s1 = 0.0;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) x[k] = v[R.c[k]];
+#pragma unroll
+    for (int k = 0; k < 8; k += 2) {
+        s0 = fma(R.p[k], x[k], s0);
+        s1 = fma(R.p[k + 1], x[k + 1], s1);
+    }
+    return s0 + s1;
+}
+// (A e)_i from a prefetched row, as apply_row_c.
+__device__ __forceinline__ float apply_row_r(const Game&, const SlotRow8<float>& R, float leak, float ei, const float* e) {
+    float x[8], acc = leak * ei;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) x[k] = e[R.c[k]];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) acc = fmaf(R.p[k], ei - x[k], acc);
+    return acc;
+}
+__device__ __forceinline__ double apply_row_r(const Game& G, const SlotRow8<double>& R, double, double ei,
+                                              const double* e) {
+    return fma(-G.mu, row_sum_r(R, e), ei);
+}
+// The relaxation's slot-major weights and leakage in its type.
+__device__ __forceinline__ const float* slot_p(const Compact& S, float) { return S.p32; }
+__device__ __forceinline__ const double* slot_p(const Compact& S, double) { return S.p64; }
+__device__ __forceinline__ const float* slot_leak(const Compact& S, float) { return S.leak32; }
+__device__ __forceinline__ const double* slot_leak(const Compact& S, double) { return S.leak64; }
+
 // Execution context of one game's policy iteration: which threads share the
 // work, how they synchronise, and where the correction vectors live.  The
 // block context runs a game inside one thread block (vectors in shared
@@ -626,6 +720,7 @@ struct BlockCtx {
     __device__ int sumi(int v) { return block_sum_int(v, *red, turn()); }
     __device__ bool failed() const { return false; }
     __device__ bool leader() const { return threadIdx.x == 0; }
+    __device__ bool own_copy() const { return true; }
     // The float32 copy of v that the improvement gathers from: in shared memory.
     __device__ const float* gather_copy(const Game& G, const BatchOut&, const double* vv) {
         float* c = (float*)t;
@@ -712,6 +807,7 @@ struct GridCtx {
     }
     __device__ bool failed() const { return bad; }
     __device__ bool leader() const { return blockIdx.x == 0 && threadIdx.x == 0; }
+    __device__ bool own_copy() const { return false; }
     __device__ const float* gather_copy(const Game& G, const BatchOut& O, const double*) { return O.v32 + G.x0; }
 };
 
@@ -725,22 +821,16 @@ struct Eval {
 
 __device__ __forceinline__ unsigned long long abs_bits(double x) { return bits_of(x) & 0x7fffffffffffffffull; }
 
-// One state's part of the residual check: r = rhs - (v - mu M v) (float64),
-// C.r = r and, with jacobi0, the correction's first Jacobi sweep from zero,
-// C.e = r / diag.  KC as for row_sum_c; KC < 0: the row is read in place.
-template <typename T, int KC, class Ctx>
-__device__ __forceinline__ double check_state(const Game& G, const BatchOut& O, const double* v, const Ctx& C,
-                                              int64_t i, bool jacobi0) {
-    double Mv;
-    if constexpr (KC >= 0) Mv = row_sum_c<KC>(C.cp, G.n, i, v);
-    else Mv = row_sum(G, O.sel[G.x0 + i], v);
-    const double r = O.rhs[G.x0 + i] - (v[i] - G.mu * Mv);
+// One state's part of the residual check: r = rhs - (v - mu M v) (float64, Mv
+// given), C.r = r and, for slot-major rows, the correction's first Jacobi sweep
+// from zero, C.e = r / diag.
+template <typename T, class Ctx>
+__device__ __forceinline__ double check_tail(const Game& G, const Ctx& C, int64_t i, double Mv, double vi, double rhs) {
+    const double r = rhs - (vi - G.mu * Mv);
     T rt;
     if constexpr (sizeof(T) == 4) rt = f64_to_f32(r);
     else rt = r;
     C.r[i] = rt;
-    if constexpr (KC >= 0) C.e[i] = rt * ((const T*)C.cp.dinv)[i];
-    else if (jacobi0) C.e[i] = rt / diag_row<T>(G, O, i);
     return r;
 }
 
@@ -765,11 +855,48 @@ __device__ __noinline__ void check_k(const Game& G, const BatchOut& O, const dou
             }
         }
     }
-    for (int64_t i = C.begin(); i < G.n; i += C.stride()) {
-        const unsigned long long rb = abs_bits(check_state<T, KC>(G, O, v, C, i, jacobi0));
-        const unsigned long long vb = abs_bits(v[i]);
+    auto take = [&](int64_t i, double Mv, double rhs) {
+        const double vi = v[i];
+        const unsigned long long rb = abs_bits(check_tail<T>(G, C, i, Mv, vi, rhs));
+        const unsigned long long vb = abs_bits(vi);
         rm = rb > rm ? rb : rm;
         vm = vb > vm ? vb : vm;
+    };
+    if constexpr (KC == 8) {
+        constexpr int D = 2;
+        SlotRow8<double> R[D];
+        double rhs[D];
+        T dinv[D];
+        const int64_t st = C.stride(), last = G.n - 1;
+        auto fetch = [&](int d, int64_t i) {
+            i = i < last ? i : last;
+            R[d].load(C.cp.col, C.cp.p64, G.n, i);
+            rhs[d] = O.rhs[G.x0 + i];
+            dinv[d] = ((const T*)C.cp.dinv)[i];
+        };
+        int64_t i = C.begin();
+#pragma unroll
+        for (int d = 0; d < D; ++d) fetch(d, i + d * st);
+        for (; i < G.n; i += D * st) {
+#pragma unroll
+            for (int d = 0; d < D; ++d) {
+                const int64_t x = i + d * st;
+                if (x < G.n) {
+                    take(x, row_sum_r(R[d], v), rhs[d]);
+                    C.e[x] = C.r[x] * dinv[d];
+                }
+                fetch(d, x + D * st);
+            }
+        }
+    } else {
+        for (int64_t i = C.begin(); i < G.n; i += C.stride()) {
+            double Mv;
+            if constexpr (KC >= 0) Mv = row_sum_c<KC>(C.cp, G.n, i, v);
+            else Mv = row_sum(G, O.sel[G.x0 + i], v);
+            take(i, Mv, O.rhs[G.x0 + i]);
+            if constexpr (KC >= 0) C.e[i] = C.r[i] * ((const T*)C.cp.dinv)[i];
+            else if (jacobi0) C.e[i] = C.r[i] / diag_row<T>(G, O, i);
+        }
     }
     unsigned long long R, V;
     C.max2(rm, vm, &R, &V);
@@ -851,36 +978,80 @@ __device__ bool cycle(const Game& G, const BatchOut& O, double* v, Ctx& C, T asu
 template <typename T, int KC, class Ctx>
 __device__ __noinline__ bool cycle11_k(const Game& G, const BatchOut& O, double* v, Ctx& C, T asum) {
     double part = 0.0;
-    for (int64_t i = C.begin(); i < G.n; i += C.stride()) {
-        T q;
-        if constexpr (KC >= 0) {
-            q = C.r[i] - apply_row_c<KC>(G, C.cp, i, C.e);
-        } else {
-            T Ae, d;
-            apply_row<T>(G, O, i, C.e, &Ae, &d);
-            q = C.r[i] - Ae;
-            C.t[i] = d;
-        }
+    const int64_t st = C.stride();
+    auto put = [&](int64_t i, T q) {
         part += as_f64(q);
         C.r[i] = q;   // r - A e1 (r itself is not needed again)
+    };
+    if constexpr (KC == 8) {
+        constexpr int D = sizeof(T) == 4 ? 3 : 2;
+        SlotRow8<T> R[D];
+        T leak[D];
+        const int64_t last = G.n - 1;
+        auto fetch = [&](int d, int64_t i) {
+            i = i < last ? i : last;
+            R[d].load(C.cp.col, slot_p(C.cp, T()), G.n, i);
+            if (sizeof(T) == 4) leak[d] = slot_leak(C.cp, T())[i];
+        };
+        int64_t i = C.begin();
+#pragma unroll
+        for (int d = 0; d < D; ++d) fetch(d, i + d * st);
+        for (; i < G.n; i += D * st) {
+#pragma unroll
+            for (int d = 0; d < D; ++d) {
+                const int64_t x = i + d * st;
+                if (x < G.n) put(x, C.r[x] - apply_row_r(G, R[d], leak[d], C.e[x], C.e));
+                fetch(d, x + D * st);
+            }
+        }
+    } else {
+        for (int64_t i = C.begin(); i < G.n; i += st) {
+            if constexpr (KC >= 0) {
+                put(i, C.r[i] - apply_row_c<KC>(G, C.cp, i, C.e));
+            } else {
+                T Ae, d;
+                apply_row<T>(G, O, i, C.e, &Ae, &d);
+                C.t[i] = d;
+                put(i, C.r[i] - Ae);
+            }
+        }
     }
     const double tot = C.sum(part, C.r, G.n);
     if (C.failed()) return false;
     const T c = asum != T(0) ? (T)(tot / (double)asum) : T(0);
-    float* v32 = O.v32 + G.x0;
-    for (int64_t i = C.begin(); i < G.n; i += C.stride()) {
-        T e;
-        if constexpr (KC >= 0) {
-            const T s = sizeof(T) == 4 ? (T)C.cp.leak32[i] : (T)C.cp.leak64[i];
-            e = C.e[i] + c + (C.r[i] - c * s) * ((const T*)C.cp.dinv)[i];
-        } else {
-            const int64_t row = O.sel[G.x0 + i];
-            const T s = sizeof(T) == 4 ? (T)G.T.leak32[row] : (T)G.T.leak[row];
-            e = C.e[i] + c + (C.r[i] - c * s) / C.t[i];
-        }
+    // the improvement gathers from the context's own copy of v where it has one
+    float* v32 = C.own_copy() && rows_in_lanes(G.T.m1, G.T.m2) ? nullptr : O.v32 + G.x0;
+    auto close = [&](int64_t i, T e) {
         const double vi = v[i] + as_f64(e);
         v[i] = vi;
-        v32[i] = f64_to_f32(vi);
+        if (v32) v32[i] = f64_to_f32(vi);
+    };
+    if constexpr (KC >= 0) {
+        constexpr int B = 4;   // states whose loads are issued together
+        const T* leak = slot_leak(C.cp, T());
+        const T* dinv = (const T*)C.cp.dinv;
+        for (int64_t i = C.begin(); i < G.n; i += B * st) {
+            T s[B], w[B];
+#pragma unroll
+            for (int k = 0; k < B; ++k) {
+                const int64_t x = i + k * st;
+                if (x < G.n) {
+                    s[k] = leak[x];
+                    w[k] = dinv[x];
+                }
+            }
+#pragma unroll
+            for (int k = 0; k < B; ++k) {
+                const int64_t x = i + k * st;
+                if (x < G.n) close(x, C.e[x] + c + (C.r[x] - c * s[k]) * w[k]);
+            }
+        }
+    } else {
+        for (int64_t i = C.begin(); i < G.n; i += st) {
+            const int64_t row = O.sel[G.x0 + i];
+            const T s = sizeof(T) == 4 ? (T)G.T.leak32[row] : (T)G.T.leak[row];
+            close(i, C.e[i] + c + (C.r[i] - c * s) / C.t[i]);
+        }
     }
     return C.sync();
 }
