@@ -68,6 +68,7 @@ struct IsaacsConsts {
     double h, mu, kappa;  // kappa = 1 - mu, evaluated without cancellation
     // Row of A = I - mu M for each code, in direction order C, W, E, S, N.
     double am[kCodes][5];
+    double am0inv[kCodes];   // 1 / am[.][0]
     // Transition probabilities per code (a < 4) in the order of the neighbours
     // E (+x1), W (-x1), N (+x2), S (-x2), self.
     double p[16][5];

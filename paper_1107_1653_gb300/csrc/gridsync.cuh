@@ -34,6 +34,7 @@ struct GridSync {
     __device__ bool sync() const {
         __shared__ int s_ok;
         __syncthreads();
+        if (nb == 1) return true;
         if (threadIdx.x == 0) {
             int ok = 1;
             const unsigned add = blockIdx.x == 0 ? 0x80000000u - (nb - 1) : 1u;

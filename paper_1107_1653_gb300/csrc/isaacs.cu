@@ -300,7 +300,8 @@ __global__ void k_isaacs_improve(const IsaacsConsts* __restrict__ K, int side, i
         }
         beta[x] = bnew;
         // policy-fixed assembly for (alpha, beta(., alpha))
-        const int old_code = code[x];
+        const size_t cx = code_at(side, i, j);
+        const int old_code = code[cx];
         int new_code;
         if (anew == 4) {
             new_code = kStopCode;
@@ -310,7 +311,7 @@ __global__ void k_isaacs_improve(const IsaacsConsts* __restrict__ K, int side, i
             new_code = 4 * anew + b;
             rhs[x] = rx + K->dr[anew][b];
         }
-        code[x] = (uint8_t)new_code;
+        code[cx] = (uint8_t)new_code;
         code_changed = new_code != old_code;
     }
     const int wch = warp_isum(changed);
@@ -337,12 +338,14 @@ __global__ void k_isaacs_assemble(const IsaacsConsts* __restrict__ K, int side,
     const size_t x = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (x >= n) return;
     const int a = alpha[x];
+    const int i = (int)(x % side), j = (int)(x / side);
+    const size_t cx = code_at(side, i, j);
     if (a == 4) {
-        code[x] = kStopCode;
-        rhs[x] = obstacle_psi((int)(x % side), (int)(x / side), K->h);
+        code[cx] = kStopCode;
+        rhs[x] = obstacle_psi(i, j, K->h);
     } else {
         const int b = (beta[x] >> (8 * a)) & 0xff;
-        code[x] = (uint8_t)(4 * a + b);
+        code[cx] = (uint8_t)(4 * a + b);
         rhs[x] = r0[x] + K->dr[a][b];
     }
 }

@@ -10,7 +10,9 @@
 
 #include "gridsync.cuh"
 #include "mgsolve.cuh"
+#include "fine.cuh"
 #include "stencil.cuh"
+#include "tail.cuh"
 
 namespace gs {
 
@@ -78,12 +80,12 @@ __device__ void relax_fine_z(const L0Op<T>& op, const LevelArgs& L, int c, size_
         }
 #pragma unroll
         for (int k = 0; k < K; ++k)
-            if (i[k] < side) u[(size_t)j[k] * side + i[k]] = val[k];
+            if (i[k] < side) u[(size_t)j[k] * L.pitch + i[k]] = val[k];
     }
     for (; t < cnt; t += st) {
         unsigned r;
         const int j = (int)dv.divmod(t, &r), i = ((j + c) & 1) + 2 * (int)r;
-        if (i < side) u[(size_t)j * side + i] = op.relaxed(f, u, i, j, zero);
+        if (i < side) u[(size_t)j * L.pitch + i] = op.relaxed(f, u, i, j, zero);
     }
 }
 
@@ -109,28 +111,31 @@ __device__ void relax_fine_update(const L0Op<float>& op, const LevelArgs& L, dou
     for (; x + (K - 1) * st < n; x += K * st) {
         float e[K];
         bool mine[K];
+        size_t at[K];
 #pragma unroll
         for (int k = 0; k < K; ++k) {
             unsigned i;
             const int j = (int)dv.divmod(x + k * st, &i);
             mine[k] = (((int)i + j) & 1) == c;
-            e[k] = mine[k] ? op.relaxed(f, u, (int)i, j, false) : u[x + k * st];
+            at[k] = (size_t)j * L.pitch + i;
+            e[k] = mine[k] ? op.relaxed(f, u, (int)i, j, false) : u[at[k]];
         }
 #pragma unroll
         for (int k = 0; k < K; ++k) {
-            if (mine[k]) u[x + k * st] = e[k];
+            if (mine[k]) u[at[k]] = e[k];
             v[x + k * st] += f32_to_f64(e[k]);
         }
     }
     for (; x < n; x += st) {
         unsigned i;
         const int j = (int)dv.divmod(x, &i);
+        const size_t at = (size_t)j * L.pitch + i;
         float e;
         if ((((int)i + j) & 1) == c) {
             e = op.relaxed(f, u, (int)i, j, false);
-            u[x] = e;
+            u[at] = e;
         } else {
-            e = u[x];
+            e = u[at];
         }
         v[x] += f32_to_f64(e);
     }
@@ -209,7 +214,7 @@ __device__ void restrict_with(const Op& op, const LevelArgs& L, const LevelArgs&
 // u_l += P u_{l+1}, one item per coarse cell (its corner, edge and C points).
 template <typename T, typename W>
 __device__ void prolong_phase(const LevelArgs& L, const LevelArgs& C, size_t start, size_t stride) {
-    const int sc = L.sc, sf = L.side, nc1 = sc + 1;
+    const int sc = L.sc, sf = L.pitch, nc1 = sc + 1;
     const size_t ncell = (size_t)nc1 * nc1;
     const W* Pw = (const W*)L.P;
     auto P = [&](int k, size_t c) -> T { return (T)wval(Pw[k * ncell + c]); };
@@ -235,15 +240,15 @@ __device__ void prolong_phase(const LevelArgs& L, const LevelArgs& C, size_t sta
 template <typename T, typename W>
 __device__ void relax_level(const SolveArgs& a, const LevelArgs& L, int l, int c, bool zero,
                             size_t start, size_t stride) {
-    if (l == 0) relax_fine<T>(L0Op<T>{a.K, a.code, L.side}, L, c, zero, start, stride);
+    if (l == 0) relax_fine<T>(L0Op<T>{a.K, a.code, L.side, L.pitch}, L, c, zero, start, stride);
     else relax_coarse<T, W>(L, c, zero, start, stride);
 }
 
 template <typename T, typename W>
 __device__ void restrict_level(const SolveArgs& a, const LevelArgs& L, const LevelArgs& C, int l,
                                bool fuse, size_t start, size_t stride) {
-    if (l == 0 && a.nu1 > 0) restrict_with<T, W, true>(L0Op<T>{a.K, a.code, L.side}, L, C, fuse, start, stride);
-    else if (l == 0) restrict_with<T, W, false>(L0Op<T>{a.K, a.code, L.side}, L, C, fuse, start, stride);
+    if (l == 0 && a.nu1 > 0) restrict_with<T, W, true>(L0Op<T>{a.K, a.code, L.side, L.pitch}, L, C, fuse, start, stride);
+    else if (l == 0) restrict_with<T, W, false>(L0Op<T>{a.K, a.code, L.side, L.pitch}, L, C, fuse, start, stride);
     else restrict_with<T, W, false>(L9Op<T, W>{(const W*)L.A, L.n, L.side}, L, C, fuse, start, stride);
 }
 
@@ -265,12 +270,13 @@ __device__ void coarse_apply_block(const LevelArgs& L, const double* inv) {
     const int n = (int)L.n;
     const T* f = (const T*)L.f;
     T* u = (T*)L.u;
-    for (int k = threadIdx.x; k < n; k += blockDim.x) fs[k] = (double)f[k];
+    auto at = [&](int x) { return (x / L.side) * L.pitch + x % L.side; };
+    for (int k = threadIdx.x; k < n; k += blockDim.x) fs[k] = (double)f[at(k)];
     __syncthreads();
     for (int r = threadIdx.x; r < n; r += blockDim.x) {
         double acc = 0.0;
         for (int k = 0; k < n; ++k) acc += inv[(size_t)r * n + k] * fs[k];
-        u[r] = (T)acc;
+        u[at(r)] = (T)acc;
     }
     __syncthreads();
 }
@@ -364,7 +370,7 @@ __device__ bool grid_vcycle(const SolveArgs& a, const LevelArgs* tl, const doubl
             for (int c = 0; c < ncol; ++c) {
                 if constexpr (sizeof(T) == 4) {
                     if (l == 0 && k == sweeps_post(a, l) - 1 && c == ncol - 1) {
-                        relax_fine_update(L0Op<float>{a.K, a.code, a.L[0].side}, a.L[0], a.v, c, gt, gs);
+                        relax_fine_update(L0Op<float>{a.K, a.code, a.L[0].side, a.L[0].pitch}, a.L[0], a.v, c, gt, gs);
                         if (!G.sync()) return false;
                         prof_mark(1000 + 10 * l + c);
                         continue;
@@ -500,7 +506,7 @@ __device__ bool grid_wcycle(const SolveArgs& a, const LevelArgs* tl, const doubl
                 for (int c = 0; c < ncol; ++c) {
                     if constexpr (sizeof(T) == 4) {
                         if (l == 0 && k == sweeps_post(a, l) - 1 && c == ncol - 1) {
-                            relax_fine_update(L0Op<float>{a.K, a.code, a.L[0].side}, a.L[0], a.v, c,
+                            relax_fine_update(L0Op<float>{a.K, a.code, a.L[0].side, a.L[0].pitch}, a.L[0], a.v, c,
                                               gt, gs);
                             if (!G.sync()) return false;
                             continue;
@@ -526,13 +532,13 @@ __device__ __forceinline__ float* setup_P32(const SolveArgs& a, const LevelArgs&
 }
 
 // Mixed path set-up items (float32, exact leakage); delta(g) lives in the
-// level's float32 right-hand side vector, free during the set-up.
+// level's spare vector, free during the set-up.
 __device__ void setup_items_f(const SolveArgs& a, int l, int kind, size_t start, size_t stride) {
     const LevelArgs& L = a.L[l];
     const int sc = L.sc;
     float* P = setup_P32(a, L);
     __nv_bfloat16* P16 = a.wbf16 ? (__nv_bfloat16*)L.P32 : nullptr;
-    float* delta = (float*)L.f;
+    float* delta = (float*)L.u2;
     const Src5f s5{a.K, a.code, L.side};
     const Src9f s9{setup_A32(a, L), L.side, L.n};
     if (kind < 2) {
@@ -636,12 +642,10 @@ __device__ __forceinline__ unsigned long long abs_bits(double x) {
 }
 
 __device__ __forceinline__ unsigned long long warp_max_u64(unsigned long long v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const unsigned long long w = __shfl_xor_sync(0xffffffffu, v, o);
-        v = w > v ? w : v;
-    }
-    return v;
+    const unsigned hi = (unsigned)(v >> 32);
+    const unsigned mh = __reduce_max_sync(0xffffffffu, hi);
+    const unsigned ml = __reduce_max_sync(0xffffffffu, hi == mh ? (unsigned)v : 0u);
+    return (unsigned long long)mh << 32 | ml;
 }
 
 // The float64 residual r = rhs - A v of the fine level with |r|_inf and
@@ -649,10 +653,11 @@ __device__ __forceinline__ unsigned long long warp_max_u64(unsigned long long v)
 // right-hand side of the correction, and the correction's first relaxation
 // colour from the zero start (C points and cell corners: e = r / diag) is
 // done here; with no pre-relaxation the correction is zeroed instead.
-__device__ void check_phase(const SolveArgs& a, int slot, size_t gt, size_t gs) {
+__device__ __forceinline__ void check_rows(const SolveArgs& a, const IsaacsConsts* Kc, size_t gt, size_t gs,
+                                           unsigned long long* rmax, unsigned long long* vmax) {
     const LevelArgs& L = a.L[0];
-    const L0Op<double> op{a.K, a.code, L.side};
-    const L0Op<float> opf{a.K, a.code, L.side};
+    const L0Op<double> op{Kc, a.code, L.side, L.side};   // v and rhs: rows of `side` elements
+    const L0Op<float> opf{Kc, a.code, L.side, L.pitch};
     float* __restrict__ r32 = a.mixed ? (float*)L.f : nullptr;
     float* __restrict__ e32 = a.mixed ? (float*)L.u : nullptr;
     const bool relax0 = fine_colour0_in_check(a);
@@ -661,14 +666,15 @@ __device__ void check_phase(const SolveArgs& a, int slot, size_t gt, size_t gs) 
     const int side = L.side;
     const unsigned n = (unsigned)L.n, st = (unsigned)gs;
     const FastDiv dv(side);
-    auto finish = [&](unsigned x, int i, int j, double r) {
+    auto finish = [&](int i, int j, double r) {
         if (r32) {
             const float rf = f64_to_f32(r);
-            r32[x] = rf;
+            const size_t at = (size_t)j * L.pitch + i;
+            r32[at] = rf;
             if (relax0) {
-                if (((i + j) & 1) == 0) e32[x] = rf / opf.diag(i, j);
+                if (((i + j) & 1) == 0) e32[at] = rf / opf.diag(i, j);
             } else {
-                e32[x] = 0.0f;
+                e32[at] = 0.0f;
             }
         }
         rm = max(rm, abs_bits(r));
@@ -687,28 +693,58 @@ __device__ void check_phase(const SolveArgs& a, int slot, size_t gt, size_t gs) 
             vm = max(vm, abs_bits(v[x + k * st]));
         }
 #pragma unroll
-        for (int k = 0; k < K; ++k) finish(x + k * st, i[k], j[k], r[k]);
+        for (int k = 0; k < K; ++k) finish(i[k], j[k], r[k]);
     }
     for (; x < n; x += st) {
         unsigned iu;
         const int j = (int)dv.divmod(x, &iu);
-        finish(x, (int)iu, j, op.resid(a.rhs, v, (int)iu, j));
+        finish((int)iu, j, op.resid(a.rhs, v, (int)iu, j));
         vm = max(vm, abs_bits(v[x]));
     }
+    *rmax = rm;
+    *vmax = vm;
+}
+
+// The maxima of this block's points into the slot's.
+__device__ __forceinline__ void check_reduce(const SolveArgs& a, int slot, unsigned long long rm,
+                                             unsigned long long vm) {
+    __shared__ unsigned long long red[2][16];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
     rm = warp_max_u64(rm);
     vm = warp_max_u64(vm);
-    if ((threadIdx.x & 31) == 0) {
-        atomicMax(&a.out->rmax[slot], rm);
-        atomicMax(&a.out->vmax[slot], vm);
+    if (lane == 0) {
+        red[0][w] = rm;
+        red[1][w] = vm;
     }
+    __syncthreads();
+    if (w == 0) {
+        rm = warp_max_u64(lane < nw ? red[0][lane] : 0ull);
+        vm = warp_max_u64(lane < nw ? red[1][lane] : 0ull);
+        if (lane == 0) {
+            atomicMax(&a.out->rmax[slot], rm);
+            atomicMax(&a.out->vmax[slot], vm);
+        }
+    }
+}
+
+__device__ void check_phase(const SolveArgs& a, int slot, size_t gt, size_t gs) {
+    unsigned long long rm, vm;
+    check_rows(a, a.K, gt, gs, &rm, &vm);
+    check_reduce(a, slot, rm, vm);
 }
 
 __device__ void axpy_phase(const SolveArgs& a, size_t gt, size_t gs) {
     const float* __restrict__ e = (const float*)a.L[0].u;
     double* __restrict__ v = a.v;
+    const int side = a.L[0].side, pitch = a.L[0].pitch;
     const size_t n = a.L[0].n;
+    const FastDiv dv((unsigned)side);
 #pragma unroll 4
-    for (size_t x = gt; x < n; x += gs) v[x] += f32_to_f64(e[x]);
+    for (size_t x = gt; x < n; x += gs) {
+        unsigned i;
+        const unsigned j = dv.divmod((unsigned)x, &i);
+        v[x] += f32_to_f64(e[(size_t)j * pitch + i]);
+    }
 }
 
 // Copies the tail levels' operators and transfers (fixed during one launch)
@@ -1168,33 +1204,32 @@ __device__ __noinline__ void tile_up(const SolveArgs& a, int l, char* smem, int 
 }
 
 // First post-smoothing colour of the finest level fused with the
-// prolongation: a colour-0 point's Gauss-Seidel value needs only its four
-// neighbours (colour 1), taken as u + P u_c on the fly; the colour-0 points'
-// own prolonged values would be overwritten unread, and the colour-1 points'
-// are not needed by the next colour either (it reads only colour 0).
-template <typename T, typename W>
-__device__ __noinline__ void relax_fine_prolonged(const SolveArgs& a, const T* uc, size_t start,
-                                                  size_t stride) {
+// prolongation (float64): a colour-0 point's Gauss-Seidel value needs only its
+// four neighbours (colour 1), taken as u + P u_c on the fly; the colour-0
+// points' own prolonged values would be overwritten unread, and the colour-1
+// points' are not needed by the next colour either (it reads only colour 0).
+__device__ __noinline__ void relax_fine_prolonged(const SolveArgs& a, const IsaacsConsts* K, const double* uc,
+                                                  size_t start, size_t stride) {
     const LevelArgs& L = a.L[0];
-    const L0Op<T> op{a.K, a.code, L.side};
-    T* __restrict__ u = (T*)L.u;
-    const T* __restrict__ f = (const T*)L.f;
-    const W* P = (const W*)L.P;
+    const L0Op<double> op{K, a.code, L.side, L.pitch};
+    double* __restrict__ u = (double*)L.u;
+    const double* __restrict__ f = (const double*)L.f;
+    const double* P = (const double*)L.P;
     const int side = L.side, sc = L.sc, hs = (side + 1) / 2;
     const unsigned cnt = (unsigned)side * hs, st = (unsigned)stride;
     const FastDiv dv(hs);
-    auto nb = [&](int i, int j) -> T {
-        return u[(size_t)j * side + i] + prolonged<T, W>(P, uc, sc, i, j);
+    auto nb = [&](int i, int j) -> double {
+        return u[(size_t)j * L.pitch + i] + prolonged<double, double>(P, uc, sc, i, j);
     };
     for (unsigned t = (unsigned)start; t < cnt; t += st) {
         unsigned r;
         const int j = (int)dv.divmod(t, &r), i = (j & 1) + 2 * (int)r;
         if (i >= side) continue;
-        const T uW = i > 0 ? nb(i - 1, j) : T(0);
-        const T uE = i + 1 < side ? nb(i + 1, j) : T(0);
-        const T uS = j > 0 ? nb(i, j - 1) : T(0);
-        const T uN = j + 1 < side ? nb(i, j + 1) : T(0);
-        u[(size_t)j * side + i] = op.relaxed_nb(f, i, j, uW, uE, uS, uN);
+        const double uW = i > 0 ? nb(i - 1, j) : 0.0;
+        const double uE = i + 1 < side ? nb(i + 1, j) : 0.0;
+        const double uS = j > 0 ? nb(i, j - 1) : 0.0;
+        const double uN = j + 1 < side ? nb(i, j + 1) : 0.0;
+        u[(size_t)j * L.pitch + i] = op.relaxed_nb(f, i, j, uW, uE, uS, uN);
     }
 }
 
@@ -1218,16 +1253,16 @@ __device__ __noinline__ void prolong_colour1(const SolveArgs& a, const T* uc, si
             unsigned r;
             j[k] = (int)dv.divmod(t + k * st, &r);
             i[k] = ((j[k] + 1) & 1) + 2 * (int)r;
-            val[k] = i[k] < side ? u[(size_t)j[k] * side + i[k]] + prolonged<T, W>(P, uc, sc, i[k], j[k]) : T(0);
+            val[k] = i[k] < side ? u[(size_t)j[k] * L.pitch + i[k]] + prolonged<T, W>(P, uc, sc, i[k], j[k]) : T(0);
         }
 #pragma unroll
         for (int k = 0; k < K; ++k)
-            if (i[k] < side) u[(size_t)j[k] * side + i[k]] = val[k];
+            if (i[k] < side) u[(size_t)j[k] * L.pitch + i[k]] = val[k];
     }
     for (; t < cnt; t += st) {
         unsigned r;
         const int j = (int)dv.divmod(t, &r), i = ((j + 1) & 1) + 2 * (int)r;
-        if (i < side) u[(size_t)j * side + i] += prolonged<T, W>(P, uc, sc, i, j);
+        if (i < side) u[(size_t)j * L.pitch + i] += prolonged<T, W>(P, uc, sc, i, j);
     }
 }
 
@@ -1238,20 +1273,94 @@ __device__ __forceinline__ const void* final_u(const SolveArgs& a, int l) {
     return l == a.tail || l < a.tile_from ? a.L[l].u : a.L[l].u2;
 }
 
-// The tail's V-cycle and the grid-wide phases of the finest level as calls of
-// their own (the tiled kernel's register budget is that of two blocks per SM).
-template <typename T, typename W>
-__device__ __noinline__ void tail_vcycle(const SolveArgs& a, const LevelArgs* tl, const double* inv) {
-    block_vcycle<T, W>(a, tl, inv, a.tail, true);
-}
-template <typename T, typename W>
-__device__ __noinline__ void fine_relax(const SolveArgs& a, int c, bool zero, size_t gt, size_t gs) {
-    relax_level<T, W>(a, a.L[0], 0, c, zero, gt, gs);
-}
-template <typename T, typename W>
-__device__ __noinline__ void fine_restrict(const SolveArgs& a, size_t gt, size_t gs) {
-    restrict_level<T, W>(a, a.L[0], a.L[1], 0, 1 < a.tail && 1 < a.nlev - 1 && sweeps_pre(a, 1) > 0, gt, gs);
-}
+// The grid-wide phases of the finest level in the tiled kernel: wide accesses in
+// the mixed path (grids of side 7 and more), one point per step otherwise.  K
+// and tab are copies in shared memory; the scalar forms are calls of their own
+// (registers).
+template <typename T>
+struct FinePhases {
+    const SolveArgs& a;
+    const IsaacsConsts* K;
+    const FineTab& tab;
+    float* stage;            // kFineStage floats of dynamic shared memory
+    size_t gt, gs;
+    bool wide;
+    __device__ void relax(int c, bool zero) const {
+        if constexpr (sizeof(T) == 4) {
+            if (wide && !zero) {
+                fine_relax_wide(a, tab, c);
+                return;
+            }
+        }
+        relax_scalar(c, zero);
+    }
+    __device__ __noinline__ void relax_scalar(int c, bool zero) const {
+        relax_fine<T>(L0Op<T>{K, a.code, a.L[0].side, a.L[0].pitch}, a.L[0], c, zero, gt, gs);
+    }
+    template <typename W>
+    __device__ void restrict_down() const {
+        // a tiled level 1 forms its first colour itself; the tail starts from zero
+        const bool tiled1 = a.tail > 1 && a.tile_from <= 1;
+        const bool first = a.tail > 1 && !tiled1 && sweeps_pre(a, 1) > 0;
+        if constexpr (sizeof(T) == 4) {
+            if (wide && a.nu1 > 0) {
+                fine_restrict_wide<W>(a, tab, first, !tiled1, stage);
+                return;
+            }
+        }
+        restrict_scalar<W>(first);
+    }
+    template <typename W>
+    __device__ __noinline__ void restrict_scalar(bool first) const {
+        const L0Op<T> op{K, a.code, a.L[0].side, a.L[0].pitch};
+        if (a.nu1 > 0) restrict_with<T, W, true>(op, a.L[0], a.L[1], first, gt, gs);
+        else restrict_with<T, W, false>(op, a.L[0], a.L[1], first, gt, gs);
+    }
+    __device__ void update(int c) const {
+        if constexpr (sizeof(T) == 4) {
+            if (wide) fine_update_wide(a, tab, c, stage);
+            else update_scalar(c);
+        }
+    }
+    __device__ __noinline__ void update_scalar(int c) const {
+        relax_fine_update(L0Op<float>{K, a.code, a.L[0].side, a.L[0].pitch}, a.L[0], a.v, c, gt, gs);
+    }
+    template <typename W>
+    __device__ void prolong_edges(const T* uc) const {
+        if constexpr (sizeof(T) == 4) {
+            if (wide) {
+                fine_prolong_wide<W>(a, uc);
+                return;
+            }
+        }
+        prolong_colour1<T, W>(a, uc, gt, gs);
+    }
+    // skip: this block takes no part (it stages the tail while the others check)
+    __device__ __noinline__ void check(int slot, bool first_check) const {
+        unsigned long long rm = 0, vm = 0;
+        bool done = false;
+        if constexpr (sizeof(T) == 4) {
+            if (wide) {
+                int r0, r1;
+                if (first_check && gridDim.x > 1) {   // blocks 1 .. take all the rows
+                    const int nb = gridDim.x - 1, b = blockIdx.x - 1;
+                    r0 = (int)((long long)a.L[0].side * b / nb);
+                    r1 = (int)((long long)a.L[0].side * (b + 1) / nb);
+                } else {
+                    block_rows(a.L[0].side, &r0, &r1);
+                }
+                fine_check_rows(a, *K, tab, fine_colour0_in_check(a), r0, r1, &rm, &vm);
+                done = true;
+            }
+        }
+        if (!done) {
+            const bool part = first_check && gridDim.x > 1;
+            check_rows(a, K, part ? gt - blockDim.x : gt, part ? gs - blockDim.x : gs, &rm, &vm);
+        }
+        check_reduce(a, slot, rm, vm);
+    }
+};
+
 // One colour of a large coarse level l (first sweep's first colour excluded:
 // the restriction into l did it), its restriction into l + 1, and the
 // prolongation into it from l + 1.
@@ -1270,29 +1379,27 @@ __device__ __noinline__ void coarse_prolong(const SolveArgs& a, int l, size_t gt
     C.u = (void*)final_u(a, l + 1);
     prolong_phase<T, W>(a.L[l], C, gt, gs);
 }
-__device__ __noinline__ void fine_check(const SolveArgs& a, int slot, size_t gt, size_t gs) {
-    check_phase(a, slot, gt, gs);
-}
-__device__ __noinline__ void fine_update(const SolveArgs& a, int c, size_t gt, size_t gs) {
-    relax_fine_update(L0Op<float>{a.K, a.code, a.L[0].side}, a.L[0], a.v, c, gt, gs);
-}
-
 // V-cycles with tiled grid-wide levels; block 0 stages and runs the tail.
 template <typename T, typename W>
-__global__ void __launch_bounds__(kMGThreads, 2) k_mg_cycles_tiled(const __grid_constant__ SolveArgs a) {
+__global__ void __launch_bounds__(kTiledThreads, 1) k_mg_cycles_tiled(const __grid_constant__ SolveArgs a) {
     extern __shared__ __align__(16) char smem_t[];
-    __shared__ LevelArgs tl[kMaxLevels];
+    __shared__ IsaacsConsts sK;
+    __shared__ FineTab tab;
+    TailBase tail{};
     const GridSync G{a.bar, gridDim.x};
     const int worker = (int)blockIdx.x - 1, nworkers = (int)gridDim.x - 1;
     const size_t gt = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     const size_t gs = (size_t)gridDim.x * blockDim.x;
+    for (int k = threadIdx.x; k < (int)(sizeof(IsaacsConsts) / 4); k += blockDim.x)
+        ((unsigned*)&sK)[k] = ((const unsigned*)a.K)[k];
+    fine_tab_fill(tab, a.K);
+    const FinePhases<T> F{a, &sK, tab, (float*)(smem_t + a.stage_at), gt, gs, a.mixed && fine_wide(a.L[0].side)};
     if (!G.sync()) return;   // set-up complete (and error state shared)
     prof_mark(8000);
-    double* inv = a.inv;
     int slot = 0;
     // block 0 stages the tail while the others take the first residual check
-    if (blockIdx.x == 0) stage_tail<T, W>(a, smem_t, tl, &inv);
-    else fine_check(a, slot, gt - blockDim.x, gs - blockDim.x);
+    if (blockIdx.x == 0) tail = tail_stage<T, W>(a, a.tail);
+    if (gridDim.x == 1 || blockIdx.x > 0) F.check(slot, true);
     prof_done(6000);
     if (!G.sync()) return;
     prof_mark(6000);
@@ -1335,12 +1442,12 @@ __global__ void __launch_bounds__(kMGThreads, 2) k_mg_cycles_tiled(const __grid_
             for (int k = 0; k < a.nu1; ++k)
                 for (int c = 0; c < 2; ++c) {
                     if (done0 && k == 0 && c == 0) continue;
-                    fine_relax<T, W>(a, c, z && k == 0 && c == 0, gt, gs);
+                    F.relax(c, z && k == 0 && c == 0);
                     prof_done(1000 + c);
                     if (!G.sync()) return;
                     prof_mark(1000 + c);
                 }
-            fine_restrict<T, W>(a, gt, gs);
+            F.template restrict_down<W>();
             prof_done(2000);
             if (!G.sync()) return;
             prof_mark(2000);
@@ -1364,7 +1471,7 @@ __global__ void __launch_bounds__(kMGThreads, 2) k_mg_cycles_tiled(const __grid_
             if (!G.sync()) return;
             prof_mark(2000 + 10 * l);
         }
-        if (blockIdx.x == 0) tail_vcycle<T, W>(a, tl, inv);
+        if (blockIdx.x == 0) tail_cycle<T>(tail, (const T*)a.L[a.tail].f, (T*)a.L[a.tail].u, a.nu1c, a.nu2c);
         prof_done(4000);
         if (!G.sync()) return;
         prof_mark(4000);
@@ -1403,31 +1510,26 @@ __global__ void __launch_bounds__(kMGThreads, 2) k_mg_cycles_tiled(const __grid_
         }
         for (int k = 0; k < a.nu2; ++k)
             for (int c = 0; c < 2; ++c) {
-                if (k == 0 && c == 0 && a.tile_from > 1) {
-                    // large grids: the colour-1 points' prolongation in a phase
-                    // of its own (each is added once, not once per neighbour),
-                    // then a plain colour-0 relaxation
-                    prolong_colour1<T, W>(a, uc, gt, gs);
+                if (k == 0 && c == 0 && (sizeof(T) == 4 || a.tile_from > 1)) {
+                    // the colour-1 points' prolongation in a phase of its own (each
+                    // is added once, not once per neighbour), then a plain colour-0
+                    // relaxation
+                    F.template prolong_edges<W>(uc);
                     if (!G.sync()) return;
                     prof_mark(1090);
-                    fine_relax<T, W>(a, 0, false, gt, gs);
+                    F.relax(0, false);
                 } else if (k == 0 && c == 0) {
-                    relax_fine_prolonged<T, W>(a, uc, gt, gs);
+                    if constexpr (sizeof(T) == 8) relax_fine_prolonged(a, &sK, (const double*)uc, gt, gs);
+                } else if (sizeof(T) == 4 && k == a.nu2 - 1 && c == 1) {
+                    F.update(c);
                 } else {
-                    bool done = false;
-                    if constexpr (sizeof(T) == 4) {
-                        if (k == a.nu2 - 1 && c == 1) {
-                            fine_update(a, c, gt, gs);
-                            done = true;
-                        }
-                    }
-                    if (!done) fine_relax<T, W>(a, c, false, gt, gs);
+                    F.relax(c, false);
                 }
                 prof_done(1100 + 10 * k + c);
                 if (!G.sync()) return;
                 prof_mark(1100 + 10 * k + c);
             }
-        fine_check(a, slot, gt, gs);
+        F.check(slot, false);
         prof_done(6000);
         if (!G.sync()) return;
         prof_mark(6000);
@@ -1508,7 +1610,8 @@ size_t tiled_smem_bytes(const SolveArgs& a) {
     auto side = [](int tc, int sc, int sf, int H) {
         return (size_t)std::min(sf, 2 * std::min(tc, sc) + 1 + 2 * H);
     };
-    size_t need = tail_smem_bytes(a);
+    // the tail's levels, the finest level's staging, the largest tile
+    size_t need = (size_t)a.stage_at + (a.mixed ? kFineStage * sizeof(float) : 0);
     for (int l = std::max(1, a.tile_from); l < a.tail; ++l) {
         const LevelArgs& L = a.L[l];
         const int K1 = a.nu1c > 0 ? 4 * a.nu1c - 1 : 0;
@@ -1524,10 +1627,10 @@ size_t tiled_smem_bytes(const SolveArgs& a) {
 void set_tile_sides(SolveArgs& a, int workers) {
     a.tc[0] = 0;   // the finest level is not tiled (one grid-wide phase per colour)
     // coarse levels: about one tile per worker block, at least 2 x 2 points
-    // of the next level, at most 16 x 16 (8 x 8 in float64: shared memory)
+    // of the next level, at most 22 x 22 (11 x 11 in float64: shared memory)
     int root = 1;
     while ((root + 1) * (root + 1) <= std::max(1, workers)) ++root;
-    const int cap = a.mixed ? 16 : 8;
+    const int cap = a.mixed ? 22 : 11;
     for (int l = 1; l < kMaxLevels; ++l) {
         const int sc = l < a.nlev ? a.L[l].sc : 1;
         a.tc[l] = std::max(2, std::min(cap, (sc + root - 1) / root));
@@ -1583,16 +1686,15 @@ void launch_mg_cycles(const SolveArgs& a, cudaStream_t st) {
     if (a.tiled) {
         const int kind = !a.mixed ? 1 : a.wbf16 ? 2 : 0;
         const size_t smem = tiled_smem_bytes(a);
-        int per_sm = 0;
-        GS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, tiled_kernel(kind), kMGThreads,
-                                                              smem));
-        // one block per tile of the largest tiled level (plus block 0), the
-        // whole GPU when a large coarse level runs grid-wide phases
-        int nb = std::max(1, per_sm) * o.sms;
-        if (a.tile_from <= 1) nb = std::min(nb, 1 + tiled_max_tiles(a));
+        // one block per SM at most; enough for the tiles of the largest tiled
+        // level (plus block 0) and for the finest level's points: a float64
+        // point keeps its SM's float64 pipe busy far longer than a float32 one
+        const size_t per_block = a.mixed ? 512 : 128;
+        int nb = (int)std::min<size_t>((a.L[0].n + per_block - 1) / per_block, (size_t)o.sms);
+        nb = std::min(std::max(nb, 1 + tiled_max_tiles(a)), o.sms);
+        if (a.L[0].side <= 31) nb = 1;
         if (a.max_blocks > 0) nb = std::min(nb, a.max_blocks);
-        nb = std::max(nb, 2);
-        GS_CUDA(cudaLaunchCooperativeKernel(tiled_kernel(kind), dim3(nb), dim3(kMGThreads), args, smem,
+        GS_CUDA(cudaLaunchCooperativeKernel(tiled_kernel(kind), dim3(nb), dim3(kTiledThreads), args, smem,
                                             st));
         note_launches(1);
         return;

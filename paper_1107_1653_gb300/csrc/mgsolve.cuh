@@ -9,6 +9,7 @@ namespace gs {
 
 constexpr int kMaxLevels = 14;
 constexpr int kMGThreads = 256;
+constexpr int kTiledThreads = 512;   // the tiled cycle kernel: one block per SM
 // Largest shared-memory footprint of the tail levels staged by block 0.
 constexpr int kTailSmemMax = 100 * 1024;
 
@@ -16,6 +17,8 @@ constexpr int kTailSmemMax = 100 * 1024;
 struct LevelArgs {
     int side;            // grid side of the level
     int sc;              // side of the next coarser level, (side - 1) / 2
+    int pitch;           // elements per row of u and f (side, or side + 1 between zeros on
+                         // the finest level of the mixed path)
     size_t n;
     void* u;             // V-cycle unknown (float32 in the mixed path, else float64)
     void* f;             // V-cycle right-hand side
@@ -44,6 +47,8 @@ struct SolveArgs {
     const uint8_t* code;
     double* v;
     const double* rhs;
+    int lg0;         // log2(side + 1) of the finest level
+    int stage_at;    // tiled cycles: byte offset of the finest level's staging in shared memory
     int nlev;        // levels; nlev - 1 is the coarsest (explicit inverse)
     int tail;        // levels >= tail are relaxed by thread block 0 alone
     int smem_from;   // levels >= smem_from (>= max(tail, 1)) live in block 0's shared memory
@@ -78,7 +83,7 @@ size_t tail_smem_bytes(const SolveArgs& a);
 
 // Largest dynamic shared memory a tiled cycle launch may take, and what one
 // needs (the tail's and the largest tile's, whichever is more).
-constexpr int kTiledSmemMax = 110 * 1024;
+constexpr int kTiledSmemMax = 220 * 1024;
 // Largest coarse level side the tiled kernel tiles: a 1023 x 1023 coarse level
 // (the 2047 x 2047 grid's first) measured faster one phase per colour; in
 // float64 (tiles of at most 8 x 8 next-level points: shared memory) already a

@@ -10,6 +10,7 @@
 #include <mutex>
 
 #include "solver.cuh"
+#include "stencil.cuh"
 
 namespace gs {
 
@@ -122,7 +123,8 @@ gs_status static_solve(int32_t side, int32_t variant, uint64_t seed, const doubl
     g.v = w;                                   // the caller's output holds the iterate
     g.rhs = cv.take<double>(n);
     g.alpha = cv.take<uint8_t>(n);
-    g.code = cv.take<uint8_t>(n);
+    g.code = cv.take<uint8_t>(code_bytes(side));
+    GS_CUDA(cudaMemsetAsync(g.code, kStopCode, code_bytes(side), st));
     g.beta = cv.take<uint32_t>(n);
     g.beta4 = cv.take<uint8_t>(n);
     g.dstatus = cv.take<int>(4);
@@ -146,8 +148,12 @@ gs_status static_solve(int32_t side, int32_t variant, uint64_t seed, const doubl
             L.f64 = cv.take<double>(L.n);
         }
         L.r64 = cv.take<double>(L.n);
-        L.u32 = cv.take<float>(L.n);
-        L.f32 = cv.take<float>(L.n);
+        if (l == 0) {
+            set_fine_planes(L, cv.take<float>(2 * fine_plane_elems(side)), st);
+        } else {
+            L.u32 = cv.take<float>(L.n);
+            L.f32 = cv.take<float>(L.n);
+        }
         L.r32 = cv.take<float>(L.n);
         if (l + 1 < g.lv.size()) {
             const size_t sc = (size_t)(L.side - 1) / 2;

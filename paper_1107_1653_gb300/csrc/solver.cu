@@ -7,6 +7,8 @@
 #include <cstring>
 
 #include "mgsolve.cuh"
+#include "stencil.cuh"
+#include "tail.cuh"
 #include "solver.cuh"
 
 namespace gs {
@@ -180,8 +182,10 @@ IsaacsConsts make_isaacs_consts(int side, int variant, int mu_mode) {
             K.dr[a][b] = K.kappa * (0.1 * (a - b));
         }
     K.am[kStopCode][0] = 1.0;
-    for (int c = 0; c < kCodes; ++c)
+    for (int c = 0; c < kCodes; ++c) {
+        K.am0inv[c] = 1.0 / K.am[c][0];
         for (int d = 0; d < 5; ++d) K.amf[c][d] = (float)K.am[c][d];
+    }
     K.kappa_f = (float)K.kappa;
     K.w0mu = K.mu * (0.5 / c0);
     K.gmu = K.mu * (h / (2.0 * c0));
@@ -193,6 +197,13 @@ IsaacsConsts make_isaacs_consts(int side, int variant, int mu_mode) {
     return K;
 }
 
+void set_fine_planes(Level& L, float* p, cudaStream_t st) {
+    const size_t plane = fine_plane_elems(L.side);
+    GS_CUDA(cudaMemsetAsync(p, 0, 2 * plane * sizeof(float), st));
+    L.u32 = p + fine_plane_origin(L.side);
+    L.f32 = p + plane + fine_plane_origin(L.side);
+}
+
 static void alloc_grid(gs_solver* s, Arena& ar, IsaacsGrid& g) {
     const size_t n = g.n;
     g.Kd = ar.alloc<IsaacsConsts>(1);
@@ -202,7 +213,8 @@ static void alloc_grid(gs_solver* s, Arena& ar, IsaacsGrid& g) {
     g.rhs = ar.alloc<double>(n);
     g.fv = ar.alloc<double>(n);
     g.alpha = ar.alloc<uint8_t>(n);
-    g.code = ar.alloc<uint8_t>(n);
+    g.code = ar.alloc<uint8_t>(code_bytes(g.side));
+    GS_CUDA(cudaMemsetAsync(g.code, kStopCode, code_bytes(g.side), s->st));
     g.beta = ar.alloc<uint32_t>(n);
     g.beta4 = ar.alloc<uint8_t>(n);
     g.dstatus = ar.alloc<int>(4);
@@ -227,8 +239,13 @@ static void alloc_grid(gs_solver* s, Arena& ar, IsaacsGrid& g) {
             L.f64 = ar.alloc<double>(L.n);
         }
         L.r64 = ar.alloc<double>(L.n);
-        L.u32 = ar.alloc<float>(L.n);
-        L.f32 = ar.alloc<float>(L.n);
+        if (l == 0) {
+            float* p = ar.alloc<float>(2 * fine_plane_elems(L.side));
+            set_fine_planes(L, p, s->st);
+        } else {
+            L.u32 = ar.alloc<float>(L.n);
+            L.f32 = ar.alloc<float>(L.n);
+        }
         L.r32 = ar.alloc<float>(L.n);
         if (l + 1 < g.lv.size()) {
             const size_t sc = (size_t)(L.side - 1) / 2;
@@ -325,6 +342,7 @@ int linear_solve(gs_solver* s, IsaacsGrid& g, Counters& cnt, double rel_tol, boo
     a.v = g.v;
     a.rhs = g.rhs;
     a.nlev = (int)g.lv.size();
+    while ((2 << a.lg0) <= g.side + 1) ++a.lg0;
     a.tail = tail_level(s, g);
     a.nu1 = s->opt.nu1;
     a.nu2 = s->opt.nu2;
@@ -348,6 +366,7 @@ int linear_solve(gs_solver* s, IsaacsGrid& g, Counters& cnt, double rel_tol, boo
         L.side = Lv.side;
         L.sc = (Lv.side - 1) / 2;
         L.n = Lv.n;
+        L.pitch = l == 0 && mixed ? Lv.side + 1 : Lv.side;
         if (l == 0) {
             L.u = mixed ? (void*)Lv.u32 : (void*)g.v;
             L.f = mixed ? (void*)Lv.f32 : (void*)g.rhs;
@@ -363,27 +382,37 @@ int linear_solve(gs_solver* s, IsaacsGrid& g, Counters& cnt, double rel_tol, boo
         L.P32 = Lv.P32;
         L.u2 = mixed ? (void*)Lv.r32 : (void*)Lv.r64;
     }
-    // about two blocks per SM in a tiled launch; tile sides for that many workers
+    // tiled V-cycles where they apply: V-cycles, a grid with a coarse level (the
+    // tail takes at least one), shared memory within the launch's limit
+    const size_t elem = a.mixed ? sizeof(float) : sizeof(double);
+    a.tiled = s->opt.cycle_kernel == 0 && a.gamma == 1 && a.nlev >= 2;
+    const int tail_colour_kernel = a.tail;
+    if (a.tiled) {
+        a.tail = std::max(a.tail, 1);
+        while (a.tail < a.nlev - 1 && tail_set_bytes(a, a.tail, elem) > (size_t)kTiledSmemMax) ++a.tail;
+    }
+    if (a.tiled) a.stage_at = (int)((tail_set_bytes(a, a.tail, elem) + 127) / 128 * 128);
+    // one block per SM in a tiled launch; tile sides for that many workers
     {
         int dev = 0, sms = 0;
         GS_CUDA(cudaGetDevice(&dev));
         GS_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-        int blocks = 2 * sms;
+        int blocks = sms;
         if (a.max_blocks > 0) blocks = std::min(blocks, a.max_blocks);
         set_tile_sides(a, std::max(1, blocks - 1));
     }
     a.tile_from = 1;
     const int tile_max = a.mixed ? kTiledMaxSide : kTiledMaxSideF64;
     while (a.tile_from < a.tail && a.L[a.tile_from].side > tile_max) ++a.tile_from;
+    // (block 0 takes no tiles: grid-wide coarse levels need a second block)
+    if (a.tiled && (tiled_smem_bytes(a) > (size_t)kTiledSmemMax || (a.max_blocks == 1 && a.tail > 1))) {
+        a.tiled = 0;
+        a.tail = tail_colour_kernel;
+    }
     // levels from smem_from on are staged in block 0's shared memory, as many as fit
     a.smem_from = std::max(a.tail, 1);
     while (a.smem_from < a.nlev && tail_smem_bytes(a) > (size_t)kTailSmemMax)
         ++a.smem_from;
-    // tiled V-cycles where they apply: V-cycles with at least one grid-wide
-    // level, shared memory within the launch's limit
-    a.tiled = s->opt.cycle_kernel == 0 && a.gamma == 1 && a.tail >= 1 &&
-              (a.max_blocks == 0 || a.max_blocks >= 2) &&
-              tiled_smem_bytes(a) <= (size_t)kTiledSmemMax;
     GS_CUDA(cudaMemsetAsync(s->mgd, 0, sizeof(MGState), s->st));
     if (do_setup) {
         KScope ks(s, GS_K_MG_SETUP);

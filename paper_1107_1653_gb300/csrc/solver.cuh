@@ -49,6 +49,15 @@ struct Level {
     float *u32 = nullptr, *f32 = nullptr, *r32 = nullptr;
 };
 
+// The finest level's float32 u and f: rows of side + 1 elements (aligned, since
+// side = 2^k - 1) between a row and a column of zeros on every side, so that
+// neighbours of boundary points read zeros without bounds tests.  Elements of
+// one such plane and the position of grid point (0, 0) in it.
+inline size_t fine_plane_origin(int side) { return (size_t)(side + 1) + 32; }
+inline size_t fine_plane_elems(int side) {
+    return (fine_plane_origin(side) + (size_t)(side + 1) * (side + 1) + 32 + 63) / 64 * 64;
+}
+
 // An Isaacs grid with its policies, value and multigrid hierarchy.
 struct IsaacsGrid {
     int side = 0, variant = 0;
@@ -168,6 +177,8 @@ struct gs_solver {
 
 namespace gs {
 
+// Points L.u32 and L.f32 into 2 * fine_plane_elems floats at p, cleared on st.
+void set_fine_planes(Level& L, float* p, cudaStream_t st);
 IsaacsConsts make_isaacs_consts(int side, int variant, int mu_mode);
 std::unique_ptr<Problem> build_isaacs_problem(gs_solver* s, int side, int variant, uint64_t seed,
                                               const double* xi);

@@ -50,6 +50,13 @@ struct Src9 {
     }
 };
 
+// Policy codes are stored with side + 1 bytes per grid row, so that every row
+// of 2^k - 1 points starts aligned; the last byte of a row holds the stop code.
+__host__ __device__ __forceinline__ size_t code_at(int side, int i, int j) {
+    return (size_t)j * (side + 1) + i;
+}
+__host__ __device__ __forceinline__ size_t code_bytes(int side) { return (size_t)side * (side + 1); }
+
 // Implicit 5-point rows of the fine Isaacs level: the row of A = I - mu M for
 // the policy code at the point, couplings to boundary points dropped.
 struct Src5 {
@@ -58,7 +65,7 @@ struct Src5 {
     const uint8_t* code;
     int side;
     __device__ __forceinline__ void row(int i, int j, double a[9]) const {
-        int c = code[(size_t)j * side + i];
+        int c = code[code_at(side, i, j)];
         const double* am = K->am[c];
         a[DC] = am[0];
         a[DW] = i > 0 ? am[1] : 0.0;
@@ -95,44 +102,48 @@ template <>
 struct L0Op<double> {
     const IsaacsConsts* K;
     const uint8_t* code;
-    int side;
+    int side, pitch;     // pitch: elements per row of u and f
     // Couplings to the boundary multiply +0 instead of being skipped: no
     // branch or select on doubles (both would take the float64 pipe).
     // Five fused multiply-adds from f (each float64 operation costs 64 cycles).
     __device__ __forceinline__ double resid(const double* f, const double* u, int i, int j) const {
-        const size_t x = (size_t)j * side + i;
-        const double* am = K->am[code[x]];
+        const size_t x = (size_t)j * pitch + i;
+        const double* am = K->am[code[code_at(side, i, j)]];
         double r = fma(-am[0], u[x], f[x]);
         r = fma(-am[1], load_or_zero(u, x - 1, i > 0), r);
         r = fma(-am[2], load_or_zero(u, x + 1, i + 1 < side), r);
-        r = fma(-am[3], load_or_zero(u, x - side, j > 0), r);
-        return fma(-am[4], load_or_zero(u, x + side, j + 1 < side), r);
+        r = fma(-am[3], load_or_zero(u, x - pitch, j > 0), r);
+        return fma(-am[4], load_or_zero(u, x + pitch, j + 1 < side), r);
     }
     // Gauss-Seidel value of u at (i, j) (neighbours from u; zero: u == 0).
     __device__ __forceinline__ double relaxed(const double* f, const double* u, int i, int j,
                                               bool zero) const {
-        const size_t x = (size_t)j * side + i;
-        const double* am = K->am[code[x]];
-        double s = f[x];
-        if (!zero) {
-            if (i > 0) s -= am[1] * u[x - 1];
-            if (i + 1 < side) s -= am[2] * u[x + 1];
-            if (j > 0) s -= am[3] * u[x - side];
-            if (j + 1 < side) s -= am[4] * u[x + side];
-        }
-        return s / am[0];
+        const size_t x = (size_t)j * pitch + i;
+        if (zero) return over_diag(f[x], code[code_at(side, i, j)]);
+        return relaxed_nb(f, i, j, load_or_zero(u, x - 1, i > 0), load_or_zero(u, x + 1, i + 1 < side),
+                          load_or_zero(u, x - pitch, j > 0), load_or_zero(u, x + pitch, j + 1 < side));
     }
-    // The same update with the four neighbours' values given (W, E, S, N).
+    // The same update with the four neighbours' values given (W, E, S, N; zero
+    // outside the grid).
     __device__ __forceinline__ double relaxed_nb(const double* f, int i, int j, double uW, double uE,
                                                  double uS, double uN) const {
-        const size_t x = (size_t)j * side + i;
-        const double* am = K->am[code[x]];
-        double s = f[x];
-        if (i > 0) s -= am[1] * uW;
-        if (i + 1 < side) s -= am[2] * uE;
-        if (j > 0) s -= am[3] * uS;
-        if (j + 1 < side) s -= am[4] * uN;
-        return s / am[0];
+        const size_t x = (size_t)j * pitch + i;
+        const int c = code[code_at(side, i, j)];
+        const double* am = K->am[c];
+        double s = fma(-am[1], uW, f[x]);
+        s = fma(-am[2], uE, s);
+        s = fma(-am[3], uS, s);
+        s = fma(-am[4], uN, s);
+        return over_diag(s, c);
+    }
+    // s / am[c][0] by the stored inverse and one correction of the quotient: three
+    // float64 operations where a division is a chain of some ten.  The bare
+    // product with the rounded inverse errs to the same side at every point of a
+    // code, which the smallest eigenvalue of A (about 1e-5 at 1023^2) turns into
+    // a relative error of 2e-12 in v.
+    __device__ __forceinline__ double over_diag(double s, int c) const {
+        const double q = s * K->am0inv[c];
+        return fma(fma(-K->am[c][0], q, s), K->am0inv[c], q);
     }
 };
 
@@ -140,22 +151,22 @@ template <>
 struct L0Op<float> {
     const IsaacsConsts* K;
     const uint8_t* code;
-    int side;
+    int side, pitch;     // pitch: elements per row of u and f
     __device__ __forceinline__ float resid(const float* f, const float* u, int i, int j) const {
-        const size_t x = (size_t)j * side + i;
-        const int c = code[x];
+        const size_t x = (size_t)j * pitch + i;
+        const int c = code[code_at(side, i, j)];
         const float* am = K->amf[c];
         const float ux = u[x];
         float Au = l0_rowsum_f(K, c, i, j, side) * ux;
         if (i > 0) Au += am[1] * (u[x - 1] - ux);
         if (i + 1 < side) Au += am[2] * (u[x + 1] - ux);
-        if (j > 0) Au += am[3] * (u[x - side] - ux);
-        if (j + 1 < side) Au += am[4] * (u[x + side] - ux);
+        if (j > 0) Au += am[3] * (u[x - pitch] - ux);
+        if (j + 1 < side) Au += am[4] * (u[x + pitch] - ux);
         return f[x] - Au;
     }
     // Diagonal of the row in the leakage form, as relaxed() forms it.
     __device__ __forceinline__ float diag(int i, int j) const {
-        const int c = code[(size_t)j * side + i];
+        const int c = code[code_at(side, i, j)];
         const float* am = K->amf[c];
         float d = l0_rowsum_f(K, c, i, j, side);
         if (i > 0) d -= am[1];
@@ -166,26 +177,14 @@ struct L0Op<float> {
     }
     __device__ __forceinline__ float relaxed(const float* f, const float* u, int i, int j,
                                              bool zero) const {
-        const size_t x = (size_t)j * side + i;
-        const int c = code[x];
+        const size_t x = (size_t)j * pitch + i;
+        const int c = code[code_at(side, i, j)];
         const float* am = K->amf[c];
         float diag = l0_rowsum_f(K, c, i, j, side), s = f[x];
         if (i > 0) { diag -= am[1]; if (!zero) s -= am[1] * u[x - 1]; }
         if (i + 1 < side) { diag -= am[2]; if (!zero) s -= am[2] * u[x + 1]; }
-        if (j > 0) { diag -= am[3]; if (!zero) s -= am[3] * u[x - side]; }
-        if (j + 1 < side) { diag -= am[4]; if (!zero) s -= am[4] * u[x + side]; }
-        return s / diag;
-    }
-    __device__ __forceinline__ float relaxed_nb(const float* f, int i, int j, float uW, float uE,
-                                                float uS, float uN) const {
-        const size_t x = (size_t)j * side + i;
-        const int c = code[x];
-        const float* am = K->amf[c];
-        float diag = l0_rowsum_f(K, c, i, j, side), s = f[x];
-        if (i > 0) { diag -= am[1]; s -= am[1] * uW; }
-        if (i + 1 < side) { diag -= am[2]; s -= am[2] * uE; }
-        if (j > 0) { diag -= am[3]; s -= am[3] * uS; }
-        if (j + 1 < side) { diag -= am[4]; s -= am[4] * uN; }
+        if (j > 0) { diag -= am[3]; if (!zero) s -= am[3] * u[x - pitch]; }
+        if (j + 1 < side) { diag -= am[4]; if (!zero) s -= am[4] * u[x + pitch]; }
         return s / diag;
     }
 };
@@ -447,7 +446,7 @@ struct Src5f {
     const uint8_t* code;
     int side;
     __device__ __forceinline__ void row(int i, int j, float a[9], float* s) const {
-        const int c = code[(size_t)j * side + i];
+        const int c = code[code_at(side, i, j)];
         const float* am = K->amf[c];
         a[DC] = am[0];
         a[DW] = i > 0 ? am[1] : 0.0f;
