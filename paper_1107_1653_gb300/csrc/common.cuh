@@ -174,10 +174,6 @@ __device__ __forceinline__ double f32_to_f64(float v) {
 // Largest Isaacs grid side: keeps every level index below 2^28 (FastDiv).
 constexpr int kIsaacsMaxSide = 16383;
 
-__device__ __forceinline__ void atomic_max_nonneg(unsigned long long* dst, double v) {
-    atomicMax(dst, (unsigned long long)__double_as_longlong(v));
-}
-
 inline double bits_to_double(unsigned long long b) {
     double d;
     static_assert(sizeof(d) == sizeof(b), "");

@@ -16,20 +16,34 @@ struct NoiseSrc {
     int step;
 };
 
-void launch_isaacs_r0(const IsaacsConsts* K, int side, double kappa, NoiseSrc ns,
-                      double* r0, cudaStream_t st);
+// scratch: at least `side` doubles (the sines of the grid lines).
+void launch_isaacs_r0(int side, double kappa, NoiseSrc ns, double* scratch, double* r0, cudaStream_t st);
 
 enum ImproveMode { IMP_OUTER = 0, IMP_INNER = 1, IMP_REPLY = 2 };
 
 // Policy improvement at v (Eq. (eq1)/(ILPI)).  alpha, beta (packed 4 x 8 bits
-// per state: beta(x, a) for a = 0..3) are read and updated in place according
-// to the mode; code/rhs receive the policy-fixed row codes and right-hand
-// side r^{alpha beta} (assembly, Eq. (LSPI)); fv (may be null) receives F(v).
+// per state: beta(x, a) for a = 0..3) are read, alpha_out and beta_out (which may
+// be the same arrays, or null) receive the new ones according to the mode;
+// code/rhs (both or neither) receive the policy-fixed row codes and right-hand
+// side r^{alpha beta} (assembly, Eq. (LSPI)); fv (may be null) receives F(v);
+// beta5 (may be null) the replies as five bytes per state, the fifth from beta4.
 // tau >= 0 is the keep-current tolerance; tau < 0 takes 1e-13 max(1, sc->vmax).
-void launch_isaacs_improve(ImproveMode mode, const IsaacsConsts* K, int side, int variant,
-                           const double* v, const double* r0, uint8_t* alpha, uint32_t* beta,
-                           uint8_t* code, double* rhs, double* fv, DevScalars* sc, double tau,
-                           cudaStream_t st);
+struct ImproveArgs {
+    const IsaacsConsts* K;
+    int side, variant;
+    const double *v, *r0;
+    const uint8_t* alpha;
+    const uint32_t* beta;
+    uint8_t* alpha_out;
+    uint32_t* beta_out;
+    uint8_t* code;
+    double *rhs, *fv;
+    uint8_t* beta5;
+    const uint8_t* beta4;
+    DevScalars* sc;
+    double tau;
+};
+void launch_isaacs_improve(ImproveMode mode, const ImproveArgs& a, cudaStream_t st);
 
 // Assembly only: code/rhs from alpha and beta.
 void launch_isaacs_assemble(const IsaacsConsts* K, int side, const uint8_t* alpha,

@@ -169,7 +169,7 @@ gs_status static_solve(int32_t side, int32_t variant, uint64_t seed, const doubl
     GS_CUDA(cudaMemsetAsync(bad, 0, 2 * sizeof(int), st));
     GS_CUDA(cudaMemsetAsync(g.beta4, 0, n, st));
     NoiseSrc ns{xi, seed, side, 1};
-    launch_isaacs_r0(g.Kd, side, g.Kh.kappa, ns, g.r0, st);
+    launch_isaacs_r0(side, g.Kh.kappa, ns, g.rhs, g.r0, st);   // rhs: scratch until assembled
     GS_CUDA(cudaMemcpyAsync(g.alpha, alpha, n, cudaMemcpyDeviceToDevice, st));
     GS_CUDA(cudaMemcpyAsync(beta_stage, beta, n * m1, cudaMemcpyDeviceToDevice, st));
     launch_check_actions(g.alpha, n, m1, bad, st);

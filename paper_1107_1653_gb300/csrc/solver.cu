@@ -279,7 +279,7 @@ std::unique_ptr<Problem> build_isaacs_problem(gs_solver* s, int side, int varian
         g->Kh = make_isaacs_consts(sd, variant, s->opt.mu_mode);
         alloc_grid(s, P->arena, *g);
         NoiseSrc ns{P->xi, seed, side, (side + 1) / (sd + 1)};
-        launch_isaacs_r0(g->Kd, sd, g->Kh.kappa, ns, g->r0, s->st);
+        launch_isaacs_r0(sd, g->Kh.kappa, ns, g->fv, g->r0, s->st);
         P->grids.push_back(std::move(g));
     }
     sync(s);
@@ -460,6 +460,12 @@ void vmax_to_device(gs_solver* s, IsaacsGrid& g) {
     launch_absmax(g.v, g.n, &s->dsc->vmax, s->st);
 }
 
+// Improvement arguments on the grid's own arrays.
+ImproveArgs improve_args(gs_solver* s, IsaacsGrid& g, double* fv, double tau) {
+    return {g.Kd,   g.side, g.variant, g.v, g.r0,    g.alpha, g.beta, g.alpha,
+            g.beta, g.code, g.rhs,     fv,  nullptr, g.beta4, s->dsc, tau};
+}
+
 // AMGpi (Sec. 5.1): Algorithm 2 with Algorithm 1 inside, every linear system
 // solved by multigrid.  Starts from g.v, g.alpha and (if beta_given) g.beta.
 bool amgpi(gs_solver* s, IsaacsGrid& g, double eps, bool beta_given, Counters& cnt) {
@@ -468,8 +474,7 @@ bool amgpi(gs_solver* s, IsaacsGrid& g, double eps, bool beta_given, Counters& c
     if (!beta_given) {
         vmax_to_device(s, g);
         KScope ks(s, GS_K_IMPROVE);
-        launch_isaacs_improve(IMP_REPLY, g.Kd, g.side, g.variant, g.v, g.r0, g.alpha, g.beta,
-                              g.code, g.rhs, nullptr, s->dsc, -1.0, st);
+        launch_isaacs_improve(IMP_REPLY, improve_args(s, g, nullptr, -1.0), st);
     } else {
         launch_isaacs_assemble(g.Kd, g.side, g.alpha, g.beta, g.r0, g.code, g.rhs, st);
     }
@@ -479,8 +484,7 @@ bool amgpi(gs_solver* s, IsaacsGrid& g, double eps, bool beta_given, Counters& c
         auto inner_improve = [&]() {
             clear_scalars(s);
             KScope ks(s, GS_K_IMPROVE);
-            launch_isaacs_improve(IMP_INNER, g.Kd, g.side, g.variant, g.v, g.r0, g.alpha, g.beta,
-                                  g.code, g.rhs, nullptr, s->dsc, tie_tol(s), st);
+            launch_isaacs_improve(IMP_INNER, improve_args(s, g, nullptr, tie_tol(s)), st);
             const DevScalars& h = read_scalars(s);
             g.stale_rows += h.code_changed;
             return h.changed;
@@ -502,8 +506,7 @@ bool amgpi(gs_solver* s, IsaacsGrid& g, double eps, bool beta_given, Counters& c
         clear_scalars(s);
         {
             KScope ks(s, GS_K_IMPROVE);
-            launch_isaacs_improve(IMP_OUTER, g.Kd, g.side, g.variant, g.v, g.r0, g.alpha, g.beta,
-                                  g.code, g.rhs, g.fv, s->dsc, tie_tol(s), st);
+            launch_isaacs_improve(IMP_OUTER, improve_args(s, g, nullptr, tie_tol(s)), st);
         }
         const DevScalars& h = read_scalars(s);
         g.stale_rows += h.code_changed;
@@ -617,38 +620,61 @@ gs_status run_solve(gs_solver* s, gs_solve_stats* stats) {
     return converged ? GS_OK : GS_ENOTCONV;
 }
 
+namespace {
+
+// Whether a kernel may use p itself: memory of the current device, aligned.
+bool usable_on_device(const void* p, size_t align) {
+    if (!p || reinterpret_cast<uintptr_t>(p) % align) return false;
+    cudaPointerAttributes at{};
+    int dev = -1;
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return at.type == cudaMemoryTypeDevice && at.device == dev;
+}
+
+bool overlap(const void* a, size_t na, const void* b, size_t nb) {
+    const uintptr_t x = reinterpret_cast<uintptr_t>(a), y = reinterpret_cast<uintptr_t>(b);
+    return a && b && x < y + nb && y < x + na;
+}
+
+}  // namespace
+
+// The kernel reads v and writes the results where the caller has them on the
+// device (no copies through scratch: six of 8 MB and less at 1023^2); host
+// arrays, unaligned ones and results laid over v or each other go through
+// scratch.  The solver's own policies are only read.
 gs_status run_improve(gs_solver* s, const double* v, uint8_t* alpha_out, uint8_t* beta_out,
                       double* fv_out) {
     Problem& P = *s->prob;
     IsaacsGrid& g = *P.grids.back();
-    // work on copies so that the solver's state is untouched
+    const int m1 = g.variant == 1 ? 5 : 4;
+    const size_t n = g.n, nv = n * sizeof(double), nb = n * m1;
+    const bool apart = !overlap(v, nv, alpha_out, n) && !overlap(v, nv, beta_out, nb) &&
+                       !overlap(v, nv, fv_out, nv) && !overlap(alpha_out, n, beta_out, nb) &&
+                       !overlap(alpha_out, n, fv_out, nv) && !overlap(beta_out, nb, fv_out, nv);
+    const bool dv = apart && usable_on_device(v, 8), da = apart && usable_on_device(alpha_out, 1),
+               db = apart && usable_on_device(beta_out, m1 == 4 ? 4 : 1), df = apart && usable_on_device(fv_out, 8);
     Arena scratch(0, 0, s->st);
-    double* vd = scratch.alloc<double>(g.n);
-    uint8_t* a = scratch.alloc<uint8_t>(g.n);
-    uint32_t* b = scratch.alloc<uint32_t>(g.n);
-    uint8_t* code = scratch.alloc<uint8_t>(g.n);
-    double* rhs = scratch.alloc<double>(g.n);
-    double* fv = scratch.alloc<double>(g.n);
-    GS_CUDA(cudaMemcpyAsync(vd, v, g.n * sizeof(double), cudaMemcpyDefault, s->st));
-    GS_CUDA(cudaMemcpyAsync(a, g.alpha, g.n, cudaMemcpyDeviceToDevice, s->st));
-    GS_CUDA(cudaMemcpyAsync(b, g.beta, g.n * 4, cudaMemcpyDeviceToDevice, s->st));
-    clear_scalars(s);
-    launch_absmax(vd, g.n, &s->dsc->vmax, s->st);
-    launch_isaacs_improve(IMP_OUTER, g.Kd, g.side, g.variant, vd, g.r0, a, b, code, rhs, fv, s->dsc,
-                          -1.0, s->st);
-    if (alpha_out) GS_CUDA(cudaMemcpyAsync(alpha_out, a, g.n, cudaMemcpyDefault, s->st));
-    if (fv_out) GS_CUDA(cudaMemcpyAsync(fv_out, fv, g.n * sizeof(double), cudaMemcpyDefault, s->st));
-    if (beta_out) {
-        const int m1 = g.variant == 1 ? 5 : 4;
-        if (m1 == 4) {
-            GS_CUDA(cudaMemcpyAsync(beta_out, b, g.n * 4, cudaMemcpyDefault, s->st));
-        } else {
-            uint8_t* stage = scratch.alloc<uint8_t>(g.n * m1);
-            k_unpack_beta<<<div_up(g.n, 256), 256, 0, s->st>>>(b, g.beta4, m1, g.n, stage);
-            GS_CHECK_LAUNCH();
-            GS_CUDA(cudaMemcpyAsync(beta_out, stage, g.n * m1, cudaMemcpyDefault, s->st));
-        }
+    const double* vd = v;
+    if (!dv) {
+        double* t = scratch.alloc<double>(n);
+        GS_CUDA(cudaMemcpyAsync(t, v, nv, cudaMemcpyDefault, s->st));
+        vd = t;
     }
+    uint8_t* a = !alpha_out ? nullptr : da ? alpha_out : scratch.alloc<uint8_t>(n);
+    uint8_t* b = !beta_out ? nullptr : db ? beta_out : scratch.alloc<uint8_t>(nb);
+    double* fv = !fv_out ? nullptr : df ? fv_out : scratch.alloc<double>(n);
+    clear_scalars(s);
+    launch_absmax(vd, n, &s->dsc->vmax, s->st);
+    const ImproveArgs A{g.Kd, g.side, g.variant, vd, g.r0, g.alpha, g.beta, a,
+                        m1 == 4 ? reinterpret_cast<uint32_t*>(b) : nullptr, nullptr, nullptr, fv,
+                        m1 == 5 ? b : nullptr, g.beta4, s->dsc, -1.0};
+    launch_isaacs_improve(IMP_OUTER, A, s->st);
+    if (a && !da) GS_CUDA(cudaMemcpyAsync(alpha_out, a, n, cudaMemcpyDefault, s->st));
+    if (fv && !df) GS_CUDA(cudaMemcpyAsync(fv_out, fv, nv, cudaMemcpyDefault, s->st));
+    if (b && !db) GS_CUDA(cudaMemcpyAsync(beta_out, b, nb, cudaMemcpyDefault, s->st));
     sync(s);
     return GS_OK;
 }
