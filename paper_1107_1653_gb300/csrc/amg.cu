@@ -39,7 +39,8 @@ namespace gs {
 
 namespace {
 
-constexpr int kAmgThreads = 256;
+constexpr int kAmgThreads = 1024;   // the cycle kernel: one block per SM
+constexpr int kLoopThreads = 512;   // the set-up's cooperative loops
 
 // ------------------------------------------------------------------ set-up kernels
 // Rows of A = I - mu M for the selected rows (ELL, diagonal first, duplicate
@@ -109,45 +110,51 @@ __global__ void k_pmis_init(int n, const unsigned long long* __restrict__ S, con
     }
 }
 
-// Along every strong edge between two undecided points, the one of smaller
-// weight is not a local maximum.
-__global__ void k_pmis_mark(int n, int W, const int* __restrict__ col, const unsigned long long* __restrict__ S,
-                            const int8_t* __restrict__ state, const double* __restrict__ w,
-                            int* __restrict__ notmax) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        if (state[i] != 0) continue;
-        const unsigned long long m = S[i];
-        for (int s = 1; s < W; ++s) {
-            if (!(m >> s & 1ull)) continue;
-            const int j = col[(size_t)i * W + s];
-            if (state[j] != 0) continue;
-            if (w[j] > w[i]) notmax[i] = 1;
-            else notmax[j] = 1;
+// Independent sets until every point is decided (at most kPmisRounds rounds), in
+// one cooperative launch: along every strong edge between two undecided points
+// the one of smaller weight is not a local maximum; local maxima become C;
+// undecided points that strongly depend on a C point become F.  The three steps
+// of a round as launches of their own with a read-back of the points left cost
+// a host round trip per round.  B: zeroed; B->left counts in turn.
+constexpr int kPmisRounds = 200;
+__global__ void __launch_bounds__(kLoopThreads) k_pmis(int n, int W, const int* __restrict__ col,
+                                                       const unsigned long long* __restrict__ S, int8_t* state,
+                                                       const double* __restrict__ w, int* notmax, AmgLoop* B) {
+    const GridSync G{&B->bar, gridDim.x};
+    const int first = blockIdx.x * blockDim.x + threadIdx.x, step = gridDim.x * blockDim.x;
+    for (int round = 0; round < kPmisRounds; ++round) {
+        for (int i = first; i < n; i += step) {
+            if (state[i] != 0) continue;
+            const unsigned long long m = S[i];
+            for (int s = 1; s < W; ++s) {
+                if (!(m >> s & 1ull)) continue;
+                const int j = col[(size_t)i * W + s];
+                if (state[j] != 0) continue;
+                if (w[j] > w[i]) notmax[i] = 1;
+                else notmax[j] = 1;
+            }
         }
+        if (first == 0) B->left[(round + 1) % 3] = 0;
+        if (!G.sync()) return;
+        for (int i = first; i < n; i += step) {
+            if (state[i] == 0 && !notmax[i]) state[i] = 1;
+            notmax[i] = 0;
+        }
+        if (!G.sync()) return;
+        int cnt = 0;
+        for (int i = first; i < n; i += step) {
+            if (state[i] != 0) continue;
+            const unsigned long long m = S[i];
+            bool f = false;
+            for (int s = 1; s < W && !f; ++s)
+                if ((m >> s & 1ull) && state[col[(size_t)i * W + s]] == 1) f = true;
+            if (f) state[i] = 2;
+            else ++cnt;
+        }
+        if (cnt) atomicAdd(&B->left[round % 3], cnt);
+        if (!G.sync()) return;
+        if (__ldcg(&B->left[round % 3]) == 0) return;
     }
-}
-
-__global__ void k_pmis_select(int n, int8_t* __restrict__ state, int* __restrict__ notmax) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        if (state[i] == 0 && !notmax[i]) state[i] = 1;
-        notmax[i] = 0;
-    }
-}
-
-// Undecided points that strongly depend on a C point become F; counts the rest.
-__global__ void k_pmis_fpass(int n, int W, const int* __restrict__ col, const unsigned long long* __restrict__ S,
-                             int8_t* __restrict__ state, int* __restrict__ left) {
-    int cnt = 0;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        if (state[i] != 0) continue;
-        const unsigned long long m = S[i];
-        bool f = false;
-        for (int s = 1; s < W && !f; ++s)
-            if ((m >> s & 1ull) && state[col[(size_t)i * W + s]] == 1) f = true;
-        if (f) state[i] = 2;
-        else ++cnt;
-    }
-    if (cnt) atomicAdd(left, cnt);
 }
 
 // Ruge-Stueben second pass: an F point i with a strong F neighbour j that
@@ -186,12 +193,14 @@ __global__ void k_rs_apply(int n, int8_t* __restrict__ state, int* __restrict__ 
     }
 }
 
-// Colouring of the matrix graph for the Gauss-Seidel smoother (greedy
-// independent sets, Jones-Plassmann): in round k every uncoloured point whose
-// hashed weight beats all its uncoloured neighbours' (along either direction
-// of a coupling) takes colour k.  Points of one colour are mutually
-// uncoupled, so relaxing them together is exactly Gauss-Seidel in colour
-// order.
+// Colouring of the matrix graph for the Gauss-Seidel smoother (Jones-Plassmann):
+// in each round every uncoloured point whose hashed weight beats all its
+// uncoloured neighbours' (along either direction of a coupling) takes the
+// smallest colour none of its coloured neighbours has.  Points of one colour are
+// mutually uncoupled, so relaxing them together is exactly Gauss-Seidel in
+// colour order.  (Taking the round's number as the colour needed 28 colours per
+// level on the tables of a 127^2 grid, and as many phases per half sweep; the
+// smallest free colour needs 5 to 14.)
 __device__ __forceinline__ unsigned colour_weight(int i) {
     unsigned z = (unsigned)i * 0x9e3779b9u + 0x7f4a7c15u;
     z = (z ^ (z >> 16)) * 0x85ebca6bu;
@@ -204,53 +213,84 @@ __device__ __forceinline__ bool colour_beats(int i, int j) {   // strict total o
     return wi != wj ? wi > wj : i > j;
 }
 
-__global__ void k_colour_mark(int n, int W, const int* __restrict__ col, const int16_t* __restrict__ colour,
-                              int* __restrict__ notmax) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        if (colour[i] >= 0) continue;
-        for (int s = 1; s < W; ++s) {
-            const int j = col[(size_t)i * W + s];
-            if (j < 0 || j == i || colour[j] >= 0) continue;
-            if (colour_beats(j, i)) notmax[i] = 1;
-            else notmax[j] = 1;
-        }
-    }
-}
-
-// Round k: local maxima take colour k; counts per (colour, C/F) class and the
-// points left uncoloured.
-// The points of each smoother class (C or F, colour k) counted, then listed
-// (class order: C colours, then F colours; order within a class is free: its
-// points are mutually uncoupled).
-__global__ void k_class_count(int n, int ncolour, const int16_t* __restrict__ colour,
-                              const int8_t* __restrict__ cf, int* __restrict__ cnt) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-        atomicAdd(&cnt[(cf[i] == 1 ? 0 : ncolour) + colour[i]], 1);
-}
-__global__ void k_class_scatter(int n, int ncolour, const int16_t* __restrict__ colour,
-                                const int8_t* __restrict__ cf, int* __restrict__ cursor, int* __restrict__ ord) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-        ord[atomicAdd(&cursor[(cf[i] == 1 ? 0 : ncolour) + colour[i]], 1)] = i;
-}
-
-__global__ void k_colour_select(int n, int k, int16_t* __restrict__ colour, int* __restrict__ notmax,
-                                const int8_t* __restrict__ cf, int* __restrict__ cls, int* __restrict__ left) {
-    int lc = 0, nC = 0, nF = 0;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        if (colour[i] < 0) {
-            if (!notmax[i]) {
-                colour[i] = (int16_t)k;
-                if (cf[i] == 1) ++nC;
-                else ++nF;
-            } else {
-                ++lc;
+// used[2 i ..]: the colours of the coloured points whose rows hold i; cls->over is
+// set when a point finds no colour free.
+__global__ void __launch_bounds__(kLoopThreads) k_colour(int n, int W, const int* __restrict__ col, int16_t* colour,
+                                                         int* notmax, unsigned long long* used, AmgClasses* cls,
+                                                         AmgLoop* B) {
+    const GridSync G{&B->bar, gridDim.x};
+    const int first = blockIdx.x * blockDim.x + threadIdx.x, step = gridDim.x * blockDim.x;
+    for (int round = 0; round < n; ++round) {
+        for (int i = first; i < n; i += step) {
+            if (colour[i] >= 0) continue;
+            for (int s = 1; s < W; ++s) {
+                const int j = col[(size_t)i * W + s];
+                if (j < 0 || j == i || colour[j] >= 0) continue;
+                if (colour_beats(j, i)) notmax[i] = 1;
+                else notmax[j] = 1;
             }
         }
-        notmax[i] = 0;
+        if (first == 0) B->left[(round + 1) % 3] = 0;
+        if (!G.sync()) return;
+        int cnt = 0;
+        for (int i = first; i < n; i += step) {
+            if (colour[i] < 0) {
+                if (!notmax[i]) {
+                    unsigned long long u0 = used[2 * i], u1 = used[2 * i + 1];
+                    for (int s = 1; s < W; ++s) {
+                        const int j = col[(size_t)i * W + s];
+                        const int c = j < 0 || j == i ? -1 : colour[j];
+                        if (c >= 64) u1 |= 1ull << (c - 64);
+                        else if (c >= 0) u0 |= 1ull << c;
+                    }
+                    int c = u0 != ~0ull ? __ffsll((long long)~u0) - 1 : u1 != ~0ull ? 63 + __ffsll((long long)~u1) : -1;
+                    if (c < 0) {
+                        cls->over = 1;
+                        c = 0;
+                    }
+                    colour[i] = (int16_t)c;
+                    for (int s = 1; s < W; ++s) {
+                        const int j = col[(size_t)i * W + s];
+                        if (j >= 0 && j != i) atomicOr(&used[2 * (size_t)j + (c >> 6)], 1ull << (c & 63));
+                    }
+                } else {
+                    ++cnt;
+                }
+            }
+            notmax[i] = 0;
+        }
+        if (cnt) atomicAdd(&B->left[round % 3], cnt);
+        if (!G.sync()) return;
+        if (__ldcg(&B->left[round % 3]) == 0) return;
     }
-    if (lc) atomicAdd(left, lc);
-    if (nC) atomicAdd(&cls[0], nC);
-    if (nF) atomicAdd(&cls[1], nF);
+}
+
+// The points of each smoother class (C or F, colour k) counted, the non-empty
+// classes listed (C colours, then F colours), the points listed by class (order
+// within a class is free: its points are mutually uncoupled).
+__device__ __forceinline__ int class_key(int8_t cf, int16_t colour) { return (cf == 1 ? 0 : kAmgMaxColours) + colour; }
+__global__ void k_class_count(int n, const int16_t* __restrict__ colour, const int8_t* __restrict__ cf,
+                              int* __restrict__ cnt) {
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
+        atomicAdd(&cnt[class_key(cf[i], colour[i])], 1);
+}
+__global__ void k_class_list(int* __restrict__ cnt, AmgClasses* __restrict__ cls) {   // cnt becomes the cursors
+    if (threadIdx.x != 0) return;
+    int acc = 0, m = 0;
+    for (int key = 0; key < 2 * kAmgMaxColours; ++key) {
+        if (key == kAmgMaxColours) cls->nC = m;
+        const int c = cnt[key];
+        cnt[key] = acc;
+        if (c) cls->ofs[m++] = acc;
+        acc += c;
+    }
+    cls->ofs[m] = acc;
+    cls->count = m;
+}
+__global__ void k_class_scatter(int n, const int16_t* __restrict__ colour, const int8_t* __restrict__ cf,
+                                int* __restrict__ cursor, int* __restrict__ ord) {
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
+        ord[atomicAdd(&cursor[class_key(cf[i], colour[i])], 1)] = i;
 }
 
 // Exclusive prefix sum of (state == C) in blocks of 1024, then over the blocks.
@@ -290,6 +330,13 @@ __global__ void k_scan_add(int n, const int8_t* __restrict__ state, const int* _
     if (i < n) idx[i] = state[i] == 1 ? idx[i] + sums[blockIdx.x] : -1;
 }
 
+// Sum over a warp in a fixed order; every lane gets it.
+__device__ __forceinline__ double warp_tree(double v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+
 // Interpolation rows keep at most this many weights: the largest, rescaled
 // to the row's full sum (truncation keeps the coarse operators sparse).
 constexpr int kPMax = 4;
@@ -302,152 +349,162 @@ constexpr int kInterpCap = 64;   // candidate C points of one F row
 //   w_ij = -(a_ij + sum_k a_ik abar_kj / d_k) / a~_ii,
 //   a~_ii = a_ii + sum_{weak, non-candidate m} a_im + sum_k a_ik abar_ki / d_k,
 //   d_k = sum_{l candidate} abar_kl + abar_ki
-// (a strong F neighbour with d_k = 0 is lumped into the diagonal).  Returns
-// the number of candidates (keys/w hold them), -1 if they overflow.
-__device__ int ext_interp_row(int i, int W, const int* __restrict__ col, const double* __restrict__ a,
-                              const unsigned long long* __restrict__ S, const int8_t* __restrict__ state,
-                              int* keys, double* w) {
-    const int* ci = col + (size_t)i * W;
-    const double* ai = a + (size_t)i * W;
-    const unsigned long long mi = S[i];
-    int m = 0;
-    auto add = [&](int j) {
-        for (int q = 0; q < m; ++q)
-            if (keys[q] == j) return true;
-        if (m == kInterpCap) return false;
-        keys[m] = j;
-        w[m] = 0.0;
-        ++m;
-        return true;
-    };
-    for (int s = 1; s < W; ++s) {
-        const int j = ci[s];
-        if (j < 0 || !(mi >> s & 1ull)) continue;
-        if (state[j] == 1) {
-            if (!add(j)) return -1;
-        } else {
-            const unsigned long long mk = S[j];
-            for (int t = 1; t < W; ++t) {
-                const int l = col[(size_t)j * W + t];
-                if (l >= 0 && (mk >> t & 1ull) && state[l] == 1 && !add(l)) return -1;
+// (a strong F neighbour with d_k = 0 is lumped into the diagonal).
+//
+// One warp per point: its strong neighbours are taken in turn, the lanes hold a
+// neighbour's row, candidates and weights are in shared memory, and every sum
+// is a fixed tree.  Bound by the latency of those rows; one thread per point
+// (its candidates in local memory, each coupling a dependent load, once to count
+// and once to fill) took 1040 us per level on average on the tables of a 127^2
+// grid.  Rows keep the kPMax largest weights (ties: the earlier candidate),
+// rescaled to the row's full sum.
+constexpr int kInterpWarps = 8;
+__global__ void __launch_bounds__(32 * kInterpWarps) k_interp(
+    int n, int W, const int* __restrict__ col, const double* __restrict__ a, const unsigned long long* __restrict__ S,
+    const int8_t* __restrict__ state, const int* __restrict__ cidx, int* __restrict__ pcol, double* __restrict__ p64,
+    float* __restrict__ p32, int* __restrict__ rcount, int* __restrict__ overflow) {
+    __shared__ int s_key[kInterpWarps][kInterpCap];
+    __shared__ double s_w[kInterpWarps][kInterpCap];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    int* key = s_key[wid];
+    double* w = s_w[wid];
+    constexpr unsigned kAll = 0xffffffffu;
+    for (int i = blockIdx.x * kInterpWarps + wid; i < n; i += gridDim.x * kInterpWarps) {
+        int* pc = pcol + (size_t)i * kPMax;
+        double* pv = p64 + (size_t)i * kPMax;
+        float* pf = p32 + (size_t)i * kPMax;
+        if (state[i] == 1) {
+            if (lane < kPMax) {
+                pc[lane] = lane == 0 ? cidx[i] : -1;
+                pv[lane] = lane == 0 ? 1.0 : 0.0;
+                pf[lane] = lane == 0 ? 1.0f : 0.0f;
+                if (lane == 0) atomicAdd(&rcount[cidx[i]], 1);
             }
-        }
-    }
-    if (m == 0) return 0;
-    auto find = [&](int j) {
-        for (int q = 0; q < m; ++q)
-            if (keys[q] == j) return q;
-        return -1;
-    };
-    double diag = ai[0];
-    for (int s = 1; s < W; ++s) {
-        const int j = ci[s];
-        if (j < 0) continue;
-        const int q = find(j);
-        if (q >= 0) {
-            w[q] += ai[s];
-        } else if (!((mi >> s & 1ull) && state[j] != 1)) {
-            diag += ai[s];   // weak coupling outside the candidates: lumped
-        }
-    }
-    for (int s = 1; s < W; ++s) {
-        const int k = ci[s];
-        if (k < 0 || !(mi >> s & 1ull) || state[k] == 1) continue;
-        const int* ck = col + (size_t)k * W;
-        const double* ak = a + (size_t)k * W;
-        double den = 0.0, aki = 0.0;
-        for (int t = 1; t < W; ++t) {
-            const int l = ck[t];
-            if (l < 0) continue;
-            const double ab = fmin(ak[t], 0.0);
-            if (l == i) aki = ab;
-            else if (find(l) >= 0) den += ab;
-        }
-        den += aki;
-        if (den == 0.0) {
-            diag += ai[s];
             continue;
         }
-        for (int t = 1; t < W; ++t) {
-            const int l = ck[t];
-            if (l < 0 || l == i) continue;
-            const int q = find(l);
-            if (q >= 0) w[q] += ai[s] * fmin(ak[t], 0.0) / den;
-        }
-        diag += ai[s] * aki / den;
-    }
-    for (int q = 0; q < m; ++q) w[q] = -w[q] / diag;
-    return m;
-}
-
-// Interpolation: count pass (entries per row after truncation; widest in
-// *wmax; candidate overflow counted in *overflow).
-__global__ void k_interp_count(int n, int W, const int* __restrict__ col, const double* __restrict__ a,
-                               const unsigned long long* __restrict__ S, const int8_t* __restrict__ state,
-                               int* __restrict__ wmax, int* __restrict__ overflow) {
-    int mx = 0;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        int c = 1;
-        if (state[i] != 1) {
-            int keys[kInterpCap];
-            double w[kInterpCap];
-            c = ext_interp_row(i, W, col, a, S, state, keys, w);
-            if (c < 0) {
-                atomicAdd(overflow, 1);
-                c = 0;
-            }
-        }
-        mx = max(mx, min(c, kPMax));
-    }
-    if (mx) atomicMax(wmax, mx);
-}
-
-__global__ void k_interp_fill(int n, int W, const int* __restrict__ col, const double* __restrict__ a,
-                              const unsigned long long* __restrict__ S, const int8_t* __restrict__ state,
-                              const int* __restrict__ cidx, int WP, int* __restrict__ pcol,
-                              double* __restrict__ p64, float* __restrict__ p32, int* __restrict__ rcount) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        int* pc = pcol + (size_t)i * WP;
-        double* pv = p64 + (size_t)i * WP;
+        const unsigned long long mi = S[i];
         int m = 0;
-        if (state[i] == 1) {
-            pc[0] = cidx[i];
-            pv[0] = 1.0;
-            m = 1;
-            atomicAdd(&rcount[cidx[i]], 1);
-        } else {
-            int keys[kInterpCap];
-            double w[kInterpCap];
-            const int c = ext_interp_row(i, W, col, a, S, state, keys, w);
-            if (c > 0) {
-                // the kPMax largest weights (ties: first candidate), rescaled to the full sum
-                int keep[kPMax];
-                int nk = 0;
-                double total = 0.0;
-                for (int q = 0; q < c; ++q) {
-                    total += w[q];
-                    if (nk < kPMax) {
-                        keep[nk++] = q;
-                    } else {
-                        int lo = 0;
-                        for (int t = 1; t < kPMax; ++t)
-                            if (w[keep[t]] < w[keep[lo]]) lo = t;
-                        if (w[q] > w[keep[lo]]) keep[lo] = q;
-                    }
-                }
-                double kept = 0.0;
-                for (int t = 0; t < nk; ++t) kept += w[keep[t]];
-                const double scale = kept != 0.0 ? total / kept : 1.0;
-                for (int t = 0; t < nk; ++t) {
-                    pc[m] = cidx[keys[keep[t]]];
-                    pv[m] = scale * w[keep[t]];
-                    atomicAdd(&rcount[pc[m]], 1);
-                    ++m;
+        bool over = false;
+        auto find = [&](int j) {   // position of column j among the candidates
+            for (int q = 0; q < m; ++q)
+                if (key[q] == j) return q;
+            return -1;
+        };
+        // lanes with `want` add their (distinct) column j unless it is there
+        auto add = [&](bool want, int j) {
+            const bool fresh = want && find(j) < 0;
+            const unsigned b = __ballot_sync(kAll, fresh);
+            const int at = m + __popc(b & ((1u << lane) - 1u)), end = m + __popc(b);
+            __syncwarp();
+            if (end > kInterpCap) {
+                over = true;
+                return;
+            }
+            if (fresh) {
+                key[at] = j;
+                w[at] = 0.0;
+            }
+            m = end;
+            __syncwarp();
+        };
+        for (unsigned long long rest = mi; rest && !over; rest &= rest - 1) {
+            const int s = __ffsll((long long)rest) - 1;
+            const int j = col[(size_t)i * W + s];
+            if (state[j] == 1) {
+                add(lane == 0, j);
+            } else {
+                const unsigned long long mk = S[j];
+                for (int t0 = 0; t0 < W && !over; t0 += 32) {
+                    const int t = t0 + lane;
+                    const bool strong = t < W && (mk >> t & 1ull);
+                    const int l = strong ? col[(size_t)j * W + t] : -1;
+                    add(strong && state[l] == 1, l);
                 }
             }
         }
-        for (int s = m; s < WP; ++s) { pc[s] = -1; pv[s] = 0.0; }
-        for (int s = 0; s < WP; ++s) p32[(size_t)i * WP + s] = (float)pv[s];
+        if (over && lane == 0) atomicAdd(overflow, 1);
+        if (over || m == 0) {
+            if (lane < kPMax) {
+                pc[lane] = -1;
+                pv[lane] = 0.0;
+                pf[lane] = 0.0f;
+            }
+            __syncwarp();
+            continue;
+        }
+        // own couplings: candidates' weights; weak couplings outside are lumped
+        double lump = 0.0;
+        for (int s = 1 + lane; s < W; s += 32) {
+            const int j = col[(size_t)i * W + s];
+            if (j < 0) continue;
+            const double v = a[(size_t)i * W + s];
+            const int q = find(j);
+            if (q >= 0) w[q] += v;
+            else if (!((mi >> s & 1ull) && state[j] != 1)) lump += v;
+        }
+        double diag = a[(size_t)i * W] + warp_tree(lump);
+        __syncwarp();
+        // strong F neighbours' couplings distributed over the candidates
+        for (unsigned long long rest = mi; rest; rest &= rest - 1) {
+            const int s = __ffsll((long long)rest) - 1;
+            const int k = col[(size_t)i * W + s];
+            if (state[k] == 1) continue;
+            const double aik = a[(size_t)i * W + s];
+            double den = 0.0, ab[2];
+            int q[2];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int t = 1 + lane + 32 * h;
+                const int l = t < W ? col[(size_t)k * W + t] : -1;
+                ab[h] = l >= 0 ? fmin(a[(size_t)k * W + t], 0.0) : 0.0;
+                q[h] = l < 0 ? -1 : l == i ? -2 : find(l);
+                if (q[h] != -1) den += ab[h];   // -2: the coupling back to i
+            }
+            den = warp_tree(den);
+            if (den == 0.0) {
+                diag += aik;
+                continue;
+            }
+            const double scale = aik / den;
+            double back = 0.0;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                if (q[h] >= 0) w[q[h]] += scale * ab[h];
+                else if (q[h] == -2) back = scale * ab[h];
+            }
+            diag += warp_tree(back);
+            __syncwarp();
+        }
+        double total = 0.0;
+        for (int q = lane; q < m; q += 32) {
+            w[q] = -w[q] / diag;
+            total += w[q];
+        }
+        total = warp_tree(total);
+        __syncwarp();
+        // rank of each candidate; the first kPMax are kept, in that order
+        for (int q = lane; q < m; q += 32) {
+            int rank = 0;
+            for (int t = 0; t < m; ++t) rank += w[t] > w[q] || (w[t] == w[q] && t < q);
+            if (rank < kPMax) {
+                pc[rank] = cidx[key[q]];
+                pv[rank] = w[q];
+                atomicAdd(&rcount[cidx[key[q]]], 1);
+            }
+        }
+        __syncwarp();
+        if (lane == 0) {
+            const int kept = m < kPMax ? m : kPMax;
+            double sum = 0.0;
+            for (int t = 0; t < kept; ++t) sum += pv[t];
+            const double scale = sum != 0.0 ? total / sum : 1.0;
+            for (int t = 0; t < kPMax; ++t) {
+                if (t >= kept) pc[t] = -1;
+                pv[t] = t < kept ? scale * pv[t] : 0.0;
+                pf[t] = (float)pv[t];
+            }
+        }
+        __syncwarp();
     }
 }
 
@@ -491,92 +548,126 @@ __global__ void k_transpose_sort(int nc, int WR, const int* __restrict__ cnt, in
     }
 }
 
-// Galerkin row I of A_c = R A P, accumulated in float64 in a fixed order:
-// fine points of R's row ascending, then A's slots, then P's slots.  count
-// pass (write == false): distinct columns only; fill pass: the row in ELL
-// form with the diagonal first and the rest in order of first appearance.
-// Threads per block of the Galerkin product and the size of each thread's
-// hash table over its coarse row's columns (a power of two above the row cap).
-constexpr int kRapThreads = 16;
-constexpr int kRapHash = 128;
+// Galerkin row I of A_c = R A P, accumulated in float64 in a fixed order: fine
+// points of R's row ascending, then P's slots, then A's slots.  count pass (write
+// == false): distinct columns only; fill pass: the row in ELL form with the
+// diagonal first and the rest by ascending column.
+//
+// One warp per coarse row: the lanes hold the slots of a fine row, lanes with
+// the same target column add up in lane order and the first of them adds the sum
+// to the row, kept in shared memory with a hash table from column to position.
+// Bound by the latency of the fine rows; one thread per row, every product a
+// chain of dependent loads, took 600 us per pass on average on the tables of a
+// 127^2 grid.
+constexpr int kRapWarps = 4;
+constexpr int kRapHash = 128;          // a power of two above the row cap
 static_assert(kRapHash > kAmgRowCap, "hash table must exceed the row cap");
 
-__global__ void __launch_bounds__(kRapThreads) k_rap(int nc, const AmgLevelArgs F, int Wc, bool write,
-                                                     int* __restrict__ wmax, int* __restrict__ overflow,
-                                                     int* __restrict__ ccol, double* __restrict__ c64,
-                                                     float* __restrict__ c32) {
-    // each thread's row lives in shared memory: its columns in order of first
-    // appearance (keys, vals) and a hash table column -> position, so that
-    // adding a product costs one probe instead of a scan of the row (the sums
-    // are formed in the same order as by a scan: the same values)
-    __shared__ int s_keys[kRapThreads][kAmgRowCap];
-    __shared__ double s_vals[kRapThreads][kAmgRowCap];
-    __shared__ int s_hk[kRapThreads][kRapHash];            // column + 1, 0 = empty
-    __shared__ unsigned char s_hq[kRapThreads][kRapHash];  // its position in keys/vals
-    int* keys = s_keys[threadIdx.x];
-    double* vals = s_vals[threadIdx.x];
-    int* hk = s_hk[threadIdx.x];
-    unsigned char* hq = s_hq[threadIdx.x];
-    auto slot = [&](int J) {
-        unsigned h = ((unsigned)J * 2654435761u) >> (32 - 7);
-        while (hk[h] != 0 && hk[h] != J + 1) h = (h + 1) & (kRapHash - 1);
-        return h;
-    };
-    for (int I = blockIdx.x * blockDim.x + threadIdx.x; I < nc; I += gridDim.x * blockDim.x) {
-        for (int h = 0; h < kRapHash; ++h) hk[h] = 0;
-        int m = 1;
-        keys[0] = I;
-        vals[0] = 0.0;
-        {
-            const unsigned h = slot(I);
-            hk[h] = I + 1;
-            hq[h] = 0;
+__global__ void __launch_bounds__(32 * kRapWarps) k_rap(int nc, const AmgLevelArgs F, int Wc, bool write,
+                                                        int* __restrict__ wmax, int* __restrict__ overflow,
+                                                        int* __restrict__ ccol, double* __restrict__ c64,
+                                                        float* __restrict__ c32) {
+    __shared__ int s_key[kRapWarps][kAmgRowCap];
+    __shared__ double s_val[kRapWarps][kAmgRowCap], s_sorted[kRapWarps][kAmgRowCap];
+    __shared__ int s_hk[kRapWarps][kRapHash];    // column + 1, 0 = empty
+    __shared__ int s_hq[kRapWarps][kRapHash];    // its position in key / val
+    __shared__ int s_m[kRapWarps];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    int *key = s_key[wid], *hk = s_hk[wid], *hq = s_hq[wid], *cnt = &s_m[wid];
+    double *val = s_val[wid], *sorted = s_sorted[wid];
+    constexpr unsigned kAll = 0xffffffffu;
+    auto hash = [](int J) { return ((unsigned)J * 2654435761u) >> (32 - 7); };
+    for (int I = blockIdx.x * kRapWarps + wid; I < nc; I += gridDim.x * kRapWarps) {
+        for (int h = lane; h < kRapHash; h += 32) hk[h] = 0;
+        for (int q = lane; q < kAmgRowCap; q += 32) val[q] = 0.0;
+        __syncwarp();
+        if (lane == 0) {
+            *cnt = 1;
+            key[0] = I;
+            hk[hash(I)] = I + 1;
+            hq[hash(I)] = 0;
         }
+        __syncwarp();
         bool over = false;
         for (int r = 0; r < F.WR; ++r) {
             const int i = F.rcol[(size_t)I * F.WR + r];
             if (i < 0) break;
             const double wi = F.r64[(size_t)I * F.WR + r];
-            for (int s = 0; s < F.W; ++s) {
-                const int k = F.col[(size_t)i * F.W + s];
-                if (k < 0) continue;
-                const double wa = wi * F.a64[(size_t)i * F.W + s];
+            for (int s0 = 0; s0 < F.W; s0 += 32) {
+                const int s = s0 + lane;
+                const int k = s < F.W ? F.col[(size_t)i * F.W + s] : -1;
+                const double wa = k >= 0 ? wi * F.a64[(size_t)i * F.W + s] : 0.0;
                 for (int p = 0; p < F.WP; ++p) {
-                    const int J = F.pcol[(size_t)k * F.WP + p];
-                    if (J < 0) break;
-                    const double add = wa * F.p64[(size_t)k * F.WP + p];
-                    const unsigned h = slot(J);
-                    int q;
-                    if (hk[h] == 0) {
-                        if (m == kAmgRowCap) {
-                            over = true;
-                            continue;
-                        }
-                        q = m++;
-                        keys[q] = J;
-                        vals[q] = 0.0;
-                        hk[h] = J + 1;
-                        hq[h] = (unsigned char)q;
-                    } else {
-                        q = hq[h];
+                    const int J = k >= 0 ? F.pcol[(size_t)k * F.WP + p] : -1;
+                    const double v = J >= 0 ? wa * F.p64[(size_t)k * F.WP + p] : 0.0;
+                    const unsigned same = __match_any_sync(kAll, J);
+                    const int lead = __ffs(same) - 1;
+                    double sum = v;
+                    unsigned rest = same & (same - 1);   // the group's lanes after the first
+                    while (__any_sync(kAll, J >= 0 && rest)) {
+                        const int src = rest ? __ffs(rest) - 1 : lane;
+                        const double o = __shfl_sync(kAll, v, src);
+                        if (rest) sum += o;
+                        rest &= rest - 1;
                     }
-                    vals[q] += add;
+                    if (J >= 0 && lane == lead) {
+                        unsigned h = hash(J);
+                        int q = -1;
+                        while (true) {
+                            const int old = atomicCAS(&hk[h], 0, J + 1);
+                            if (old == J + 1) {
+                                q = hq[h];
+                                break;
+                            }
+                            if (old == 0) {
+                                q = atomicAdd(cnt, 1);
+                                hq[h] = q;
+                                if (q < kAmgRowCap) key[q] = J;
+                                break;
+                            }
+                            h = (h + 1) & (kRapHash - 1);
+                        }
+                        if (q < kAmgRowCap) val[q] += sum;
+                        else over = true;
+                    }
+                    __syncwarp();
+                    // a full row: no further insertions (the table must keep an empty slot)
+                    if (*cnt > kAmgRowCap) over = true;
+                    if (__any_sync(kAll, over)) break;
                 }
+                if (__any_sync(kAll, over)) break;
+            }
+            if (__any_sync(kAll, over)) break;
+        }
+        over = __any_sync(kAll, over);
+        const int m = min(*cnt, kAmgRowCap);
+        if (lane == 0) {
+            if (over) atomicAdd(overflow, 1);
+            if (!write) atomicMax(wmax, m);
+        }
+        if (write) {
+            // the diagonal first, then ascending columns
+            for (int q = lane; q < m; q += 32) {
+                int at = 0;
+                if (q > 0) {
+                    at = 1;
+                    for (int t = 1; t < m; ++t) at += key[t] < key[q];
+                }
+                sorted[at] = val[q];
+                ccol[(size_t)I * Wc + at] = key[q];
+            }
+            __syncwarp();
+            double part = 0.0;
+            for (int q = lane; q < m; q += 32) part += sorted[q];
+            const double rowsum = warp_tree(part);
+            for (int q = lane; q < Wc; q += 32) {
+                const double v = q < m ? sorted[q] : 0.0;
+                if (q >= m) ccol[(size_t)I * Wc + q] = -1;
+                c64[(size_t)I * Wc + q] = v;
+                c32[(size_t)I * Wc + q] = q == 0 ? (float)rowsum : (float)v;
             }
         }
-        if (over) atomicAdd(overflow, 1);
-        if (!write) {
-            atomicMax(wmax, m);
-            continue;
-        }
-        double rowsum = 0.0;
-        for (int q = 0; q < m; ++q) rowsum += vals[q];
-        for (int q = 0; q < Wc; ++q) {
-            const bool in = q < m;
-            ccol[(size_t)I * Wc + q] = in ? keys[q] : -1;
-            c64[(size_t)I * Wc + q] = in ? vals[q] : 0.0;
-            c32[(size_t)I * Wc + q] = q == 0 ? (float)rowsum : (in ? (float)vals[q] : 0.0f);
-        }
+        __syncwarp();
     }
 }
 
@@ -639,33 +730,41 @@ __global__ void k_amg_coarse_inv(int n, int W, const int* __restrict__ col, cons
             if (r != k) M(r, k) = 0.0;
         __syncthreads();
     }
-    for (int k = threadIdx.x; k < n * n; k += blockDim.x) inv[k] = M(k / n, n + k % n);
+    // by columns: the cycles' threads, one per row, read consecutive entries
+    for (int k = threadIdx.x; k < n * n; k += blockDim.x) inv[k] = M(k % n, n + k / n);
 }
 
 // ------------------------------------------------------------------ cycles
 // (A u)_i and the diagonal: float64 rows hold the entries, float32 rows the
-// row sum in slot 0 and the off-diagonals (leakage form).
+// row sum in slot 0 and the off-diagonals (leakage form).  The row's slots are
+// shared by `g` neighbouring lanes (this one is number `sub`), which all get the
+// results; every lane of the warp must call it.
 template <typename T>
-__device__ __forceinline__ void amg_row(const AmgLevelArgs& L, int i, const T* u, T* Au, T* d) {
+__device__ __forceinline__ void amg_row(const AmgLevelArgs& L, int i, const T* u, int sub, int g, T* Au, T* d) {
     const int* c = L.col + (size_t)i * L.W;
     if constexpr (sizeof(T) == 8) {
         const double* a = L.a64 + (size_t)i * L.W;
         double s = 0.0;
-        for (int k = 0; k < L.W; ++k)
+        for (int k = sub; k < L.W; k += g)
             if (c[k] >= 0) s = fma(a[k], u[c[k]], s);
+        for (int o = 1; o < g; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
         *Au = s;
         *d = a[0];
     } else {
         const float* a = L.a32 + (size_t)i * L.W;
-        const float ui = u[i];
-        float s = a[0] * ui, dg = a[0];
-        for (int k = 1; k < L.W; ++k) {
+        const float ui = u[i], lead = a[0];
+        float s = 0.0f, dg = 0.0f;
+        for (int k = 1 + sub; k < L.W; k += g) {
             if (c[k] < 0) continue;
             s = fmaf(a[k], u[c[k]] - ui, s);
-            dg -= a[k];
+            dg += a[k];
         }
-        *Au = s;
-        *d = dg;
+        for (int o = 1; o < g; o <<= 1) {
+            s += __shfl_xor_sync(0xffffffffu, s, o);
+            dg += __shfl_xor_sync(0xffffffffu, dg, o);
+        }
+        *Au = fmaf(lead, ui, s);
+        *d = lead - dg;
     }
 }
 
@@ -680,64 +779,62 @@ __device__ __forceinline__ T rw(const AmgLevelArgs& L, size_t k) {
     else return L.r32[k];
 }
 
-// Jacobi relaxation of the C points (which = 1), of the F points (which = 0)
-// or of all points (which = 2) (u -> t, the others copied; the splitting
-// marks C points 1, F points 2).
-template <typename T>
-__device__ void amg_relax(const AmgLevelArgs& L, const T* u, T* t, const T* f, int which, size_t gt, size_t gs) {
-    for (size_t i = gt; i < (size_t)L.n; i += gs) {
-        if (which != 2 && (L.cf[i] == 1) != (which == 1)) {
-            t[i] = u[i];
-            continue;
-        }
-        T Au, d;
-        amg_row<T>(L, (int)i, u, &Au, &d);
-        t[i] = u[i] + (f[i] - Au) / d;
-    }
-}
-
-// Gauss-Seidel on the points of colour k in the C (which = 1) or F (which =
-// 0) set, in place: they are mutually uncoupled.  The class's points are read
-// from its list (thread index gt of gs).
-template <typename T>
-__device__ void amg_gs(const AmgLevelArgs& L, T* u, const T* f, int k, int which, size_t gt, size_t gs) {
-    const int key = (which == 1 ? 0 : L.ncolour) + k;
-    const size_t b = (size_t)L.kofs[key], e = (size_t)L.kofs[key + 1];
-    for (size_t x = b + gt; x < e; x += gs) {
-        const int i = L.ord[x];
-        T Au, d;
-        amg_row<T>(L, i, u, &Au, &d);
-        u[i] += (f[i] - Au) / d;
-    }
-}
-
-// One C/F Gauss-Seidel sweep, colour by colour (C points first when c_first).
 // Who runs a phase and how it ends: the whole grid with a grid barrier, or
-// thread block 0 alone with a block barrier (small levels).
-// gx numbers the threads block-minor (thread t of block b is t * blocks + b),
-// so that a short list is spread over all the blocks, not packed into the
-// first few.
+// thread block 0 alone with a block barrier (small levels).  rows(g, f) calls
+// f(x, sub, in) for x = 0, 1, .. < count by groups of g lanes, numbered block-minor
+// (group t of block b is t * blocks + b) so that a short list is spread over all
+// the blocks; in is false for the lanes past the end that only join the lane
+// exchanges (x is then the last entry).
 struct GridPh {
     const GridSync* G;
-    size_t gt, gs, gx;
+    size_t gt, gs;
+    unsigned block, blocks;
     __device__ bool sync() const { return G->sync(); }
 };
 struct BlockPh {
-    size_t gt, gs, gx;
+    size_t gt, gs;
+    unsigned block, blocks;   // 0, 1
     __device__ bool sync() const {
         __syncthreads();
         return true;
     }
 };
+template <class Ph, class F>
+__device__ __forceinline__ void amg_rows(const Ph& ph, int count, int g, F&& f) {
+    const int lg = __popc(g - 1), t = threadIdx.x >> lg, groups = (int)(blockDim.x >> lg) * (int)ph.blocks;
+    const int lane_group = (int)(threadIdx.x & 31) >> lg;
+    const int x0 = (t - lane_group) * (int)ph.blocks + (int)ph.block;   // the warp's first group
+    for (int b = x0; b < count; b += groups) {
+        const int x = b + lane_group * (int)ph.blocks;
+        f(min(x, count - 1), (int)threadIdx.x & (g - 1), x < count);
+    }
+}
 
+// Jacobi relaxation of all points (u -> t).
 template <typename T, class Ph>
-__device__ bool amg_sweep(const AmgLevelArgs& L, T* u, const T* f, bool c_first, const Ph& ph) {
+__device__ void amg_jacobi(const AmgLevelArgs& L, const T* u, T* t, const T* f, const Ph& ph) {
+    amg_rows(ph, L.n, 1, [&](int i, int sub, bool in) {
+        T Au, d;
+        amg_row<T>(L, i, u, sub, 1, &Au, &d);
+        if (in) t[i] = u[i] + (f[i] - Au) / d;
+    });
+}
+
+// One C/F Gauss-Seidel sweep, class by class (C points first when c_first): a
+// class's points are mutually uncoupled and relaxed together, in place.
+template <typename T, class Ph>
+__device__ bool amg_sweep(const AmgLevelArgs& L, const AmgLists& S, T* u, const T* f, bool c_first, const Ph& ph) {
     for (int half = 0; half < 2; ++half) {
-        const int which = (half == 0) == c_first ? 1 : 0;
-        for (int k = 0; k < L.ncolour; ++k) {
-            const unsigned long long m = which ? L.cmaskC[k >> 6] : L.cmaskF[k >> 6];
-            if (!(m >> (k & 63) & 1ull)) continue;   // no point of this set has colour k
-            amg_gs<T>(L, u, f, k, which, ph.gx, ph.gs);
+        const bool isC = (half == 0) == c_first;
+        for (int k = isC ? 0 : S.nC; k < (isC ? S.nC : S.count); ++k) {
+            const int b = S.ofs[k], e = S.ofs[k + 1];
+            amg_rows(ph, e - b, L.g, [&](int x, int sub, bool in) {
+                const int i = S.ord[b + x];
+                T Au, d;
+                amg_row<T>(L, i, u, sub, L.g, &Au, &d);
+                __syncwarp();
+                if (in && sub == 0) u[i] += (f[i] - Au) / d;
+            });
             if (!ph.sync()) return false;
         }
     }
@@ -747,19 +844,18 @@ __device__ bool amg_sweep(const AmgLevelArgs& L, T* u, const T* f, bool c_first,
 // Down leg of level l: C/F relaxation, residual, restriction f_{l+1} = R r_l,
 // u_{l+1} = 0.
 template <typename T, class Ph>
-__device__ bool amg_down(const AmgSolveArgs& a, int l, T* const* u, T* const* t, const Ph& ph) {
+__device__ bool amg_down(const AmgSolveArgs& a, int l, const AmgLists* S, T* const* u, T* const* t, T* const* f,
+                         const Ph& ph) {
     const AmgLevelArgs& L = a.L[l];
-    const T* f = (const T*)L.f;
     for (int s = 0; s < a.nu1; ++s)
-        if (!amg_sweep<T>(L, u[l], f, true, ph)) return false;
-    for (size_t i = ph.gt; i < (size_t)L.n; i += ph.gs) {
+        if (!amg_sweep<T>(L, S[l], u[l], f[l], true, ph)) return false;
+    amg_rows(ph, L.n, L.g, [&](int i, int sub, bool in) {
         T Au, d;
-        amg_row<T>(L, (int)i, u[l], &Au, &d);
-        t[l][i] = f[i] - Au;
-    }
+        amg_row<T>(L, i, u[l], sub, L.g, &Au, &d);
+        if (in && sub == 0) t[l][i] = f[l][i] - Au;
+    });
     if (!ph.sync()) return false;
     const AmgLevelArgs& C = a.L[l + 1];
-    T* fc = (T*)C.f;
     for (size_t I = ph.gt; I < (size_t)C.n; I += ph.gs) {
         T acc = 0;
         for (int r = 0; r < L.WR; ++r) {
@@ -767,7 +863,7 @@ __device__ bool amg_down(const AmgSolveArgs& a, int l, T* const* u, T* const* t,
             if (i < 0) break;
             acc += rw<T>(L, I * L.WR + r) * t[l][i];
         }
-        fc[I] = acc;
+        f[l + 1][I] = acc;
         u[l + 1][I] = T(0);
     }
     return ph.sync();
@@ -775,9 +871,8 @@ __device__ bool amg_down(const AmgSolveArgs& a, int l, T* const* u, T* const* t,
 
 // Up leg of level l: u_l += P u_{l+1}, then F/C relaxation.
 template <typename T, class Ph>
-__device__ bool amg_up(const AmgSolveArgs& a, int l, T* const* u, const Ph& ph) {
+__device__ bool amg_up(const AmgSolveArgs& a, int l, const AmgLists* S, T* const* u, T* const* f, const Ph& ph) {
     const AmgLevelArgs& L = a.L[l];
-    const T* f = (const T*)L.f;
     for (size_t i = ph.gt; i < (size_t)L.n; i += ph.gs) {
         T acc = 0;
         for (int p = 0; p < L.WP; ++p) {
@@ -789,7 +884,7 @@ __device__ bool amg_up(const AmgSolveArgs& a, int l, T* const* u, const Ph& ph) 
     }
     if (!ph.sync()) return false;
     for (int s = 0; s < a.nu2; ++s)
-        if (!amg_sweep<T>(L, u[l], f, false, ph)) return false;
+        if (!amg_sweep<T>(L, S[l], u[l], f[l], false, ph)) return false;
     return true;
 }
 
@@ -831,14 +926,15 @@ __device__ void amg_check(const AmgSolveArgs& a, int slot, T* f0, T* u0, size_t 
 // `inverse_block` set (block 0), or (coarsening stopped early) Jacobi sweeps
 // over the phase's threads.
 template <typename T, class Ph>
-__device__ bool amg_coarsest(const AmgSolveArgs& a, T** u, T** t, double* fs, const Ph& ph, bool inverse_block) {
+__device__ bool amg_coarsest(const AmgSolveArgs& a, T** u, T** t, T* const* f, double* fs, const Ph& ph,
+                             bool inverse_block) {
     const int Lc = a.nlev - 1;
     const AmgLevelArgs& C = a.L[Lc];
     if (a.coarse_sweeps > 0) {
         for (size_t i = ph.gt; i < (size_t)C.n; i += ph.gs) u[Lc][i] = T(0);
         if (!ph.sync()) return false;
         for (int k = 0; k < a.coarse_sweeps; ++k) {
-            amg_relax<T>(C, u[Lc], t[Lc], (const T*)C.f, 2, ph.gt, ph.gs);
+            amg_jacobi<T>(C, u[Lc], t[Lc], f[Lc], ph);
             T* sw = u[Lc];
             u[Lc] = t[Lc];
             t[Lc] = sw;
@@ -847,12 +943,12 @@ __device__ bool amg_coarsest(const AmgSolveArgs& a, T** u, T** t, double* fs, co
         return true;
     }
     if (inverse_block) {
-        const T* f = (const T*)C.f;
-        for (int k = threadIdx.x; k < C.n; k += blockDim.x) fs[k] = (double)f[k];
+        for (int k = threadIdx.x; k < C.n; k += blockDim.x) fs[k] = (double)f[Lc][k];
         __syncthreads();
         for (int r = threadIdx.x; r < C.n; r += blockDim.x) {
             double acc = 0.0;
-            for (int k = 0; k < C.n; ++k) acc += a.inv[(size_t)r * C.n + k] * fs[k];
+#pragma unroll 8
+            for (int k = 0; k < C.n; ++k) acc = fma(a.inv[(size_t)k * C.n + r], fs[k], acc);
             u[Lc][r] = (T)acc;
         }
         __syncthreads();
@@ -860,21 +956,50 @@ __device__ bool amg_coarsest(const AmgSolveArgs& a, T** u, T** t, double* fs, co
     return true;
 }
 
+// V-cycles on the correction of a.v in one cooperative launch.  The levels from
+// a.tail on are cycled by thread block 0 alone: their phases are too short for a
+// grid barrier each; their vectors and point lists live in its shared memory.
 template <typename T>
 __global__ void __launch_bounds__(kAmgThreads) k_amg_cycles(const __grid_constant__ AmgSolveArgs a) {
+    extern __shared__ __align__(16) char smem[];
     __shared__ double fs[kAmgCoarsest];
+    __shared__ AmgLists S[kAmgMaxLevels];
     const GridSync G{a.bar, gridDim.x};
     const size_t gt = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     const size_t gs = (size_t)gridDim.x * blockDim.x;
-    T* u[kAmgMaxLevels];
-    T* t[kAmgMaxLevels];
-    for (int l = 0; l < a.nlev; ++l) {
-        u[l] = (T*)a.L[l].u;
-        t[l] = (T*)a.L[l].t;
-    }
     const int Lc = a.nlev - 1;
+    T *u[kAmgMaxLevels], *t[kAmgMaxLevels], *f[kAmgMaxLevels];
+    size_t off = 0;
+    auto take = [&](size_t bytes) {
+        char* p = smem + off;
+        off += (bytes + 15) & ~size_t(15);
+        return p;
+    };
+    for (int l = 0; l < a.nlev; ++l) {
+        const AmgLevelArgs& L = a.L[l];
+        u[l] = (T*)L.u;
+        t[l] = (T*)L.t;
+        f[l] = (T*)L.f;
+        const int* ord = L.ord;
+        if (l < Lc) {   // the classes of the smoother
+            int* ofs = (int*)take(sizeof(int) * (2 * kAmgMaxColours + 1));
+            for (int k = threadIdx.x; k <= L.cls->count; k += blockDim.x) ofs[k] = L.cls->ofs[k];
+            if (l >= a.tail && blockIdx.x == 0) {
+                int* o = (int*)take(sizeof(int) * L.n);
+                for (int k = threadIdx.x; k < L.n; k += blockDim.x) o[k] = L.ord[k];
+                ord = o;
+            }
+            if (threadIdx.x == 0) S[l] = AmgLists{L.cls->nC, L.cls->count, ofs, ord};
+        }
+        if (l >= a.tail && l > 0 && blockIdx.x == 0) {
+            u[l] = (T*)take(sizeof(T) * L.n);
+            t[l] = (T*)take(sizeof(T) * L.n);
+            f[l] = (T*)take(sizeof(T) * L.n);
+        }
+    }
+    __syncthreads();
     int slot = 0;
-    amg_check<T>(a, slot, (T*)a.L[0].f, u[0], gt, gs);
+    amg_check<T>(a, slot, (T*)a.L[0].f, (T*)a.L[0].u, gt, gs);
     if (!G.sync()) return;
     double prev = 0.0, res0 = 0.0;
     int slow = 0;
@@ -908,24 +1033,49 @@ __global__ void __launch_bounds__(kAmgThreads) k_amg_cycles(const __grid_constan
         }
         // down legs of the grid-wide levels, then the small levels (a.tail
         // and below) by thread block 0 alone, then the up legs
-        const GridPh gp{&G, gt, gs, (size_t)threadIdx.x * gridDim.x + blockIdx.x};
+        const GridPh gp{&G, gt, gs, blockIdx.x, gridDim.x};
         const int tl = a.tail < Lc ? a.tail : Lc;
-        for (int l = 0; l < tl; ++l)
-            if (!amg_down<T>(a, l, u, t, gp)) return;
+        // (the restriction into the tail writes its global vectors)
+        for (int l = 0; l < tl; ++l) {
+            T* const uc = u[l + 1];
+            T* const fc = f[l + 1];
+            u[l + 1] = (T*)a.L[l + 1].u;
+            f[l + 1] = (T*)a.L[l + 1].f;
+            const bool ok = amg_down<T>(a, l, S, u, t, f, gp);
+            u[l + 1] = uc;
+            f[l + 1] = fc;
+            if (!ok) return;
+        }
         if (a.tail <= Lc) {
             if (blockIdx.x == 0) {
-                const BlockPh bp{threadIdx.x, blockDim.x, threadIdx.x};
-                for (int l = a.tail; l < Lc; ++l) amg_down<T>(a, l, u, t, bp);
-                amg_coarsest<T>(a, u, t, fs, bp, true);
-                for (int l = Lc - 1; l >= a.tail; --l) amg_up<T>(a, l, u, bp);
+                const BlockPh bp{threadIdx.x, blockDim.x, 0, 1};
+                const int n = a.L[a.tail].n;
+                const bool staged = a.tail > 0;
+                if (staged) {
+                    for (int k = threadIdx.x; k < n; k += blockDim.x) {
+                        f[a.tail][k] = __ldcg((const T*)a.L[a.tail].f + k);
+                        u[a.tail][k] = T(0);
+                    }
+                    __syncthreads();
+                }
+                for (int l = a.tail; l < Lc; ++l) amg_down<T>(a, l, S, u, t, f, bp);
+                amg_coarsest<T>(a, u, t, f, fs, bp, true);
+                for (int l = Lc - 1; l >= a.tail; --l) amg_up<T>(a, l, S, u, f, bp);
+                if (staged)
+                    for (int k = threadIdx.x; k < n; k += blockDim.x) ((T*)a.L[a.tail].u)[k] = u[a.tail][k];
             }
             if (!G.sync()) return;
         } else {
-            if (!amg_coarsest<T>(a, u, t, fs, gp, blockIdx.x == 0)) return;
+            if (!amg_coarsest<T>(a, u, t, f, fs, gp, blockIdx.x == 0)) return;
             if (!G.sync()) return;
         }
-        for (int l = tl - 1; l >= 0; --l)
-            if (!amg_up<T>(a, l, u, gp)) return;
+        for (int l = tl - 1; l >= 0; --l) {
+            T* const uc = u[l + 1];
+            if (l + 1 == a.tail) u[l + 1] = (T*)a.L[l + 1].u;
+            const bool ok = amg_up<T>(a, l, S, u, f, gp);
+            u[l + 1] = uc;
+            if (!ok) return;
+        }
         // v += e and the next residual check
         for (size_t i = gt; i < (size_t)a.L[0].n; i += gs) a.v[i] += (double)u[0][i];
         if (!G.sync()) return;
@@ -968,6 +1118,26 @@ __global__ void k_game_assemble(int64_t n, int m1, int m2, const uint8_t* __rest
         sel[x] = row;
         rhs[x] = rew[row];
     }
+}
+
+// Blocks of the set-up's cooperative loops.
+int loop_blocks(int n, int cap) {
+    int dev = 0, sms = 0;
+    GS_CUDA(cudaGetDevice(&dev));
+    GS_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    int nb = std::min(sms, (n + kLoopThreads - 1) / kLoopThreads);
+    if (cap > 0) nb = std::min(nb, cap);
+    return std::max(1, nb);
+}
+
+// The C/F splitting's rounds; clears the loop state first.
+void launch_pmis(int n, int W, const int* col, const unsigned long long* S, int8_t* state, const double* w,
+                 int* notmax, AmgLoop* loop, int max_blocks, cudaStream_t st) {
+    GS_CUDA(cudaMemsetAsync(loop, 0, sizeof(AmgLoop), st));
+    void* args[] = {&n, &W, &col, &S, &state, &w, &notmax, &loop};
+    GS_CUDA(cudaLaunchCooperativeKernel((const void*)k_pmis, dim3(loop_blocks(n, max_blocks)), dim3(kLoopThreads),
+                                        args, 0, st));
+    GS_CHECK_LAUNCH();
 }
 
 unsigned grid_for(int64_t n) {
@@ -1380,15 +1550,8 @@ gs_status run_game_fmg(gs_solver* s, gs_solve_stats* stats) {
         k_amg_strength<<<g, 256, 0, st>>>((int)n, W, col, a, theta, S, lam);
         k_pmis_init<<<g, 256, 0, st>>>((int)n, S, lam, cf, w);
         GS_CHECK_LAUNCH_N(3);
-        for (int it = 0; it < 200; ++it) {
-            GS_CUDA(cudaMemsetAsync(scal, 0, sizeof(int) * 8, st));
-            k_pmis_mark<<<g, 256, 0, st>>>((int)n, W, col, S, cf, w, flag);
-            k_pmis_select<<<g, 256, 0, st>>>((int)n, cf, flag);
-            k_pmis_fpass<<<g, 256, 0, st>>>((int)n, W, col, S, cf, scal + 2);
-            GS_CHECK_LAUNCH_N(3);
-            read_scal();
-            if (hs[2] == 0) break;
-        }
+        AmgLoop* loop = tmp.alloc<AmgLoop>(1);
+        launch_pmis((int)n, W, col, S, cf, w, flag, loop, s->opt.grid_blocks, st);
         k_rs_second<<<g, 256, 0, st>>>((int)n, W, col, S, cf, flag);
         k_rs_apply<<<g, 256, 0, st>>>((int)n, cf, flag);
         k_promote_lonely<<<g, 256, 0, st>>>((int)n, W, col, S, cf);
@@ -1399,7 +1562,12 @@ gs_status run_game_fmg(gs_solver* s, gs_solve_stats* stats) {
         k_scan_sums<<<1, 32, 0, st>>>(nblk, sums, scal + 3);
         k_scan_add<<<nblk, kScanBlock, 0, st>>>((int)n, cf, sums, cidx);
         GS_CHECK_LAUNCH_N(6);
+        GS_CUDA(cudaMemcpyAsync(scal + 6, &loop->bar.error, sizeof(int), cudaMemcpyDeviceToDevice, st));
         read_scal();
+        if (hs[6]) {
+            set_last_error("FAMGpi set-up: a grid barrier wait timed out");
+            throw Error{GS_ETIMEOUT};
+        }
         const int nc = hs[3];
         if (nc == 0 || nc > n - n / 8) break;   // no useful coarsening
         int* agg = tmp.alloc<int>(n);
@@ -1542,22 +1710,15 @@ void AmgHierarchy::build(const GameTables& T, const int64_t* sel, double mu, int
         k_amg_strength<<<grid(nf), 256, 0, st>>>(nf, F.W, F.col, F.a64, theta, S, lam);
         k_pmis_init<<<grid(nf), 256, 0, st>>>(nf, S, lam, F.cf, w);
         GS_CHECK_LAUNCH_N(2);
-        for (int it = 0; it < 200; ++it) {
-            GS_CUDA(cudaMemsetAsync(scal, 0, sizeof(int) * 8, st));
-            k_pmis_mark<<<grid(nf), 256, 0, st>>>(nf, F.W, F.col, S, F.cf, w, flag);
-            k_pmis_select<<<grid(nf), 256, 0, st>>>(nf, F.cf, flag);
-            k_pmis_fpass<<<grid(nf), 256, 0, st>>>(nf, F.W, F.col, S, F.cf, scal + 2);
-            GS_CHECK_LAUNCH_N(3);
-            read_scal();
-            if (hs[2] == 0) break;
-        }
+        AmgLoop* loop = ar->alloc<AmgLoop>(1);
+        launch_pmis(nf, F.W, F.col, S, F.cf, w, flag, loop, opt.grid_blocks, st);
         if (opt.amg_coarsening == 1) {
             k_rs_second<<<grid(nf), 256, 0, st>>>(nf, F.W, F.col, S, F.cf, flag);
             k_rs_apply<<<grid(nf), 256, 0, st>>>(nf, F.cf, flag);
             GS_CHECK_LAUNCH_N(2);
         }
         // colouring for the Gauss-Seidel smoother, with the (colour, C/F) classes used
-        colour_level(F, flag, scal, hs, read_scal, grid(nf), st);
+        colour_level(F, flag, loop, grid(nf), opt.grid_blocks, st);
         // coarse numbering and the interpolation's width
         const int nblk = (nf + kScanBlock - 1) / kScanBlock;
         int* sums = ar->alloc<int>(nblk);
@@ -1565,24 +1726,33 @@ void AmgHierarchy::build(const GameTables& T, const int64_t* sel, double mu, int
         k_scan_local<<<nblk, kScanBlock, 0, st>>>(nf, F.cf, cidx, sums);
         k_scan_sums<<<1, 32, 0, st>>>(nblk, sums, scal + 3);
         k_scan_add<<<nblk, kScanBlock, 0, st>>>(nf, F.cf, sums, cidx);
-        k_interp_count<<<grid(nf), 256, 0, st>>>(nf, F.W, F.col, F.a64, S, F.cf, scal, scal + 1);
-        GS_CHECK_LAUNCH_N(4);
+        GS_CHECK_LAUNCH_N(3);
+        GS_CUDA(cudaMemcpyAsync(scal + 5, &F.cls->over, sizeof(int), cudaMemcpyDeviceToDevice, st));
+        GS_CUDA(cudaMemcpyAsync(scal + 6, &loop->bar.error, sizeof(int), cudaMemcpyDeviceToDevice, st));
         read_scal();
+        if (hs[6]) {
+            set_last_error("AMG set-up: a grid barrier wait timed out");
+            throw Error{GS_ETIMEOUT};
+        }
+        if (hs[5]) {
+            set_last_error("AMG: more than %d colours needed for the smoother", kAmgMaxColours);
+            throw Error{GS_EINVAL};
+        }
         const int nc = hs[3];
-        if (hs[1]) break;                      // interpolation candidates overflow: coarsest here
         if (nc == 0 || nc > nf - nf / 8) break;  // no useful coarser level: this one is the coarsest
-        F.WP = std::max(1, hs[0]);
+        F.WP = kPMax;
         F.pcol = ar->alloc<int>((size_t)nf * F.WP);
         F.p64 = ar->alloc<double>((size_t)nf * F.WP);
         F.p32 = ar->alloc<float>((size_t)nf * F.WP);
         int* rcount = ar->alloc<int>(nc);
         GS_CUDA(cudaMemsetAsync(rcount, 0, sizeof(int) * nc, st));
-        k_interp_fill<<<grid(nf), 256, 0, st>>>(nf, F.W, F.col, F.a64, S, F.cf, cidx, F.WP, F.pcol,
-                                                F.p64, F.p32, rcount);
         GS_CUDA(cudaMemsetAsync(scal, 0, sizeof(int) * 8, st));
+        k_interp<<<(unsigned)std::min((nf + kInterpWarps - 1) / kInterpWarps, 152 * 64), 32 * kInterpWarps, 0, st>>>(
+            nf, F.W, F.col, F.a64, S, F.cf, cidx, F.pcol, F.p64, F.p32, rcount, scal + 1);
         k_max_int<<<grid(nc), 256, 0, st>>>(nc, rcount, scal);
         GS_CHECK_LAUNCH_N(2);
         read_scal();
+        if (hs[1]) break;   // interpolation candidates overflow: this level is the coarsest
         F.WR = std::max(1, hs[0]);
         F.rcol = ar->alloc<int>((size_t)nc * F.WR);
         F.r64 = ar->alloc<double>((size_t)nc * F.WR);
@@ -1594,8 +1764,8 @@ void AmgHierarchy::build(const GameTables& T, const int64_t* sel, double mu, int
         // Galerkin coarse operator: count pass, then fill
         const AmgLevelArgs FA = args_of(F);
         GS_CUDA(cudaMemsetAsync(scal, 0, sizeof(int) * 8, st));
-        const unsigned rap_blocks = (unsigned)std::max(1, std::min((nc + kRapThreads - 1) / kRapThreads, 152 * 64));
-        k_rap<<<rap_blocks, kRapThreads, 0, st>>>(nc, FA, 0, false, scal, scal + 1, nullptr, nullptr, nullptr);
+        const unsigned rap_blocks = (unsigned)std::max(1, std::min((nc + kRapWarps - 1) / kRapWarps, 152 * 64));
+        k_rap<<<rap_blocks, 32 * kRapWarps, 0, st>>>(nc, FA, 0, false, scal, scal + 1, nullptr, nullptr, nullptr);
         GS_CHECK_LAUNCH();
         read_scal();
         if (hs[1]) break;   // a Galerkin row too wide: relax this level as the coarsest
@@ -1605,7 +1775,7 @@ void AmgHierarchy::build(const GameTables& T, const int64_t* sel, double mu, int
         C.col = ar->alloc<int>((size_t)nc * C.W);
         C.a64 = ar->alloc<double>((size_t)nc * C.W);
         C.a32 = ar->alloc<float>((size_t)nc * C.W);
-        k_rap<<<rap_blocks, kRapThreads, 0, st>>>(nc, FA, C.W, true, scal, scal + 1, C.col, C.a64, C.a32);
+        k_rap<<<rap_blocks, 32 * kRapWarps, 0, st>>>(nc, FA, C.W, true, scal, scal + 1, C.col, C.a64, C.a32);
         GS_CHECK_LAUNCH();
         lv.push_back(C);
     }
@@ -1638,48 +1808,30 @@ void AmgHierarchy::build(const GameTables& T, const int64_t* sel, double mu, int
     }
 }
 
-template <class Read>
-void AmgHierarchy::colour_level(AmgLevelMem& F, int* flag, int* scal, int* hs, Read&& read_scal, unsigned g,
+void AmgHierarchy::colour_level(AmgLevelMem& F, int* flag, AmgLoop* loop, unsigned g, int max_blocks,
                                 cudaStream_t st) {
     const int nf = F.n;
-    F.colour = ar->alloc<int16_t>(nf);
-    GS_CUDA(cudaMemsetAsync(F.colour, 0xff, sizeof(int16_t) * nf, st));   // -1: uncoloured
-    GS_CUDA(cudaMemsetAsync(flag, 0, sizeof(int) * nf, st));
-    std::memset(F.cmaskC, 0, sizeof F.cmaskC);
-    std::memset(F.cmaskF, 0, sizeof F.cmaskF);
-    F.ncolour = 0;
-    for (int k = 0; k < kAmgMaxColours; ++k) {
-        GS_CUDA(cudaMemsetAsync(scal, 0, sizeof(int) * 8, st));
-        k_colour_mark<<<g, 256, 0, st>>>(nf, F.W, F.col, F.colour, flag);
-        k_colour_select<<<g, 256, 0, st>>>(nf, k, F.colour, flag, F.cf, scal + 5, scal + 2);
-        GS_CHECK_LAUNCH_N(2);
-        read_scal();
-        if (hs[5]) F.cmaskC[k >> 6] |= 1ull << (k & 63);
-        if (hs[6]) F.cmaskF[k >> 6] |= 1ull << (k & 63);
-        F.ncolour = k + 1;
-        if (hs[2] == 0) break;
-    }
-    if (hs[2] != 0) {
-        set_last_error("AMG: more than %d colours needed for the smoother", kAmgMaxColours);
-        throw Error{GS_EINVAL};
-    }
-    // the points listed by class, so that a colour phase visits only its own
-    const int nk = 2 * F.ncolour;
-    int* cnt = ar->alloc<int>(nk);
-    GS_CUDA(cudaMemsetAsync(cnt, 0, sizeof(int) * nk, st));
-    k_class_count<<<g, 256, 0, st>>>(nf, F.ncolour, F.colour, F.cf, cnt);
-    GS_CHECK_LAUNCH();
-    std::vector<int> hc(nk), ofs(nk + 1, 0);
-    GS_CUDA(cudaMemcpyAsync(hc.data(), cnt, sizeof(int) * nk, cudaMemcpyDeviceToHost, st));
-    GS_CUDA(cudaStreamSynchronize(st));
-    for (int k = 0; k < nk; ++k) ofs[k + 1] = ofs[k] + hc[k];
-    F.kofs = ar->alloc<int>(nk + 1);
+    int16_t* colour = ar->alloc<int16_t>(nf);
+    unsigned long long* used = ar->alloc<unsigned long long>(2 * (size_t)nf);
+    int* cnt = ar->alloc<int>(2 * kAmgMaxColours);
+    F.cls = ar->alloc<AmgClasses>(1);
     F.ord = ar->alloc<int>(std::max(1, nf));
-    GS_CUDA(cudaMemcpyAsync(F.kofs, ofs.data(), sizeof(int) * (nk + 1), cudaMemcpyHostToDevice, st));
-    GS_CUDA(cudaMemcpyAsync(cnt, ofs.data(), sizeof(int) * nk, cudaMemcpyHostToDevice, st));
-    k_class_scatter<<<g, 256, 0, st>>>(nf, F.ncolour, F.colour, F.cf, cnt, F.ord);
-    GS_CHECK_LAUNCH();
-    GS_CUDA(cudaStreamSynchronize(st));   // the host offsets' buffer is released on return
+    GS_CUDA(cudaMemsetAsync(colour, 0xff, sizeof(int16_t) * nf, st));   // -1: uncoloured
+    GS_CUDA(cudaMemsetAsync(flag, 0, sizeof(int) * nf, st));
+    GS_CUDA(cudaMemsetAsync(used, 0, 2 * sizeof(unsigned long long) * nf, st));
+    GS_CUDA(cudaMemsetAsync(cnt, 0, 2 * kAmgMaxColours * sizeof(int), st));
+    GS_CUDA(cudaMemsetAsync(F.cls, 0, sizeof(AmgClasses), st));
+    GS_CUDA(cudaMemsetAsync(loop->left, 0, sizeof loop->left, st));
+    int n = nf, W = F.W;
+    const int* col = F.col;
+    AmgClasses* cls = F.cls;
+    void* args[] = {&n, &W, &col, &colour, &flag, &used, &cls, &loop};
+    GS_CUDA(cudaLaunchCooperativeKernel((const void*)k_colour, dim3(loop_blocks(nf, max_blocks)), dim3(kLoopThreads),
+                                        args, 0, st));
+    k_class_count<<<g, 256, 0, st>>>(nf, colour, F.cf, cnt);
+    k_class_list<<<1, 32, 0, st>>>(cnt, F.cls);
+    k_class_scatter<<<g, 256, 0, st>>>(nf, colour, F.cf, cnt, F.ord);
+    GS_CHECK_LAUNCH_N(4);
 }
 
 AmgLevelArgs AmgHierarchy::args_of(const AmgLevelMem& m) {
@@ -1699,12 +1851,8 @@ AmgLevelArgs AmgHierarchy::args_of(const AmgLevelMem& m) {
     A.r32 = m.r32;
     A.cf = m.cf;
     A.ord = m.ord;
-    A.kofs = m.kofs;
-    A.ncolour = m.ncolour;
-    A.cmaskC[0] = m.cmaskC[0];
-    A.cmaskC[1] = m.cmaskC[1];
-    A.cmaskF[0] = m.cmaskF[0];
-    A.cmaskF[1] = m.cmaskF[1];
+    A.cls = m.cls;
+    A.g = m.W <= 8 ? 1 : m.W <= 16 ? 4 : 8;
     A.u = m.u;
     A.f = m.f;
     A.t = m.t;
@@ -1728,24 +1876,32 @@ int AmgHierarchy::solve(double* v, const double* rhs, const gs_options& opt, dou
     a.inv = inv;
     a.coarse_sweeps = coarse_sweeps;
     // the small levels' phases are short: one block with block barriers beats
-    // the grid barrier there (needs the coarsest inverse: the Jacobi sweeps
-    // swap their vectors per thread)
+    // the grid barrier there, up to the rows and the shared memory one block
+    // takes (needs the coarsest inverse: the Jacobi sweeps swap their vectors
+    // per thread)
+    const size_t lists = sizeof(int) * (2 * kAmgMaxColours + 1) + 16;
+    size_t smem = lists * a.nlev;
     a.tail = a.nlev;
     if (coarse_sweeps == 0)
-        while (a.tail > 0 && lv[a.tail - 1].n <= kAmgTailN) --a.tail;
+        while (a.tail > 0) {
+            const AmgLevelMem& L = lv[a.tail - 1];
+            const size_t more = (size_t)L.n * (sizeof(int) + 3 * (mixed ? sizeof(float) : sizeof(double))) + 64;
+            if (L.n > (mixed ? kAmgTailN : kAmgTailNF64) || smem + more > (size_t)kAmgSmemMax) break;
+            smem += more;
+            --a.tail;
+        }
     a.bar = bar_state;
     a.out = dout;
     for (int l = 0; l < a.nlev; ++l) a.L[l] = args_of(lv[l]);
-    static int per_sm[2] = {0, 0}, sms = 0;
+    static int sms = 0;
     if (!sms) {
         int dev = 0;
         GS_CUDA(cudaGetDevice(&dev));
         GS_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-        GS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm[0], k_amg_cycles<float>, kAmgThreads, 0));
-        GS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm[1], k_amg_cycles<double>, kAmgThreads, 0));
+        GS_CUDA(cudaFuncSetAttribute(k_amg_cycles<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAmgSmemMax));
+        GS_CUDA(cudaFuncSetAttribute(k_amg_cycles<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAmgSmemMax));
     }
-    const int ps = std::max(1, per_sm[mixed ? 0 : 1]);
-    int nb = (int)std::min<size_t>((size_t)ps * sms, ((size_t)lv[0].n + kAmgThreads - 1) / kAmgThreads);
+    int nb = (int)std::min<size_t>((size_t)sms, ((size_t)lv[0].n + 127) / 128);
     if (opt.grid_blocks > 0) nb = std::min(nb, opt.grid_blocks);
     if (a.tail == 0) nb = 1;   // the whole hierarchy is small
     nb = std::max(1, nb);
@@ -1753,7 +1909,7 @@ int AmgHierarchy::solve(double* v, const double* rhs, const gs_options& opt, dou
     GS_CUDA(cudaMemsetAsync(dout, 0, sizeof(AmgOut), st));
     void* args[] = {(void*)&a};
     const void* fn = mixed ? (const void*)k_amg_cycles<float> : (const void*)k_amg_cycles<double>;
-    GS_CUDA(cudaLaunchCooperativeKernel(fn, dim3(nb), dim3(kAmgThreads), args, 0, st));
+    GS_CUDA(cudaLaunchCooperativeKernel(fn, dim3(nb), dim3(kAmgThreads), args, smem, st));
     note_launches(1);
     GridBarrier hb{};
     GS_CUDA(cudaMemcpyAsync(&hb, bar_state, sizeof hb, cudaMemcpyDeviceToHost, st));

@@ -18,8 +18,24 @@ constexpr int kAmgInvSmem = 64;         // inverted in shared memory up to this 
 constexpr int kAmgRowCap = 96;          // entries of a coarse row the set-up accumulates
 constexpr int kAmgCoarseSweeps = 30;    // Jacobi sweeps on a coarsest level too large to invert
 constexpr int kAmgMaxColours = 128;     // colours of the Gauss-Seidel smoother's colouring
-constexpr int kAmgTailN = 2048;         // levels this small run in one thread block, with
-                                        // block barriers instead of grid barriers
+constexpr int kAmgTailN = 6144;         // levels this small run in one thread block, with
+constexpr int kAmgTailNF64 = 2048;      // block barriers instead of grid barriers (in float64
+                                        // one SM's float64 pipe is the bound sooner)
+constexpr int kAmgSmemMax = 200 * 1024; // shared memory of a cycle launch
+
+// The smoother's classes of one level: C points by colour, then F points by
+// colour, empty classes left out; class k is ord[ofs[k], ofs[k + 1]).
+struct AmgClasses {
+    int nC, count;          // classes of C points, of all
+    int over;               // a point found no free colour
+    int ofs[2 * kAmgMaxColours + 1];
+};
+
+// The same as the cycle kernel holds it.
+struct AmgLists {
+    int nC, count;
+    const int *ofs, *ord;
+};
 
 // One level of the hierarchy, rows in ELL form (slot 0 holds the diagonal;
 // unused slots have column -1 and value 0).
@@ -38,10 +54,9 @@ struct AmgLevelArgs {
     const double* r64;
     const float* r32;
     const int8_t* cf;       // 1 C point, 2 F point (this level's splitting)
-    const int* ord;         // the points ordered by class: C points by colour, then F points
-    const int* kofs;        // class k (C: colour k, F: ncolour + colour k) is ord[kofs[k], kofs[k+1])
-    int ncolour;
-    unsigned long long cmaskC[2], cmaskF[2];   // colours that hold C (F) points
+    const int* ord;         // the points ordered by smoother class
+    const AmgClasses* cls;  // the classes (levels above the coarsest)
+    int g;                  // lanes that share a row (1, 4 or 8)
     void* u;                // V-cycle unknown (float32 in the mixed path, else float64)
     void* f;                // V-cycle right-hand side
     void* t;                // relaxation's second buffer
@@ -81,15 +96,19 @@ struct AmgLevelMem {
     double* r64 = nullptr;
     float* r32 = nullptr;
     int8_t* cf = nullptr;
-    int16_t* colour = nullptr;
     int* ord = nullptr;
-    int* kofs = nullptr;
-    int ncolour = 0;
-    unsigned long long cmaskC[2] = {0, 0}, cmaskF[2] = {0, 0};
+    AmgClasses* cls = nullptr;
     void *u = nullptr, *f = nullptr, *t = nullptr;
 };
 
 class Arena;
+
+// State of one cooperative set-up loop (zeroed before the launch).
+struct AmgLoop {
+    GridBarrier bar;
+    int left[3];
+    int pad;
+};
 
 // A hierarchy for one policy-fixed system, built on the device.
 struct AmgHierarchy {
@@ -109,9 +128,7 @@ struct AmgHierarchy {
               GridBarrier* bar_state, AmgOut* dout, AmgOut* hout, int* cycles, double* res,
               double* vmax, cudaStream_t st);
     static AmgLevelArgs args_of(const AmgLevelMem& m);
-    template <class Read>
-    void colour_level(AmgLevelMem& F, int* flag, int* scal, int* hs, Read&& read_scal, unsigned g,
-                      cudaStream_t st);
+    void colour_level(AmgLevelMem& F, int* flag, AmgLoop* loop, unsigned g, int max_blocks, cudaStream_t st);
 };
 
 }  // namespace gs
