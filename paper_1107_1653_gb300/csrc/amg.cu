@@ -110,6 +110,23 @@ __global__ void k_pmis_init(int n, const unsigned long long* __restrict__ S, con
     }
 }
 
+// f(j, s) for the slots s, s + 1, .. of a row (after the diagonal), kAhead at a
+// time: j holds their columns, -1 past the end, for empty slots and for slots
+// outside `mask`.  The columns of a step are loaded together, and so are the
+// values f looks up: walked one by one, every coupling waits for two dependent
+// loads.
+constexpr int kAhead = 8;
+template <class F>
+__device__ __forceinline__ void for_neighbours(const int* __restrict__ row, int W, F&& f,
+                                               unsigned long long mask = ~0ull) {
+    for (int s = 1; s < W; s += kAhead) {
+        int j[kAhead];
+#pragma unroll
+        for (int k = 0; k < kAhead; ++k) j[k] = s + k < W && (s + k >= 64 || (mask >> (s + k) & 1ull)) ? row[s + k] : -1;
+        f(j, s);
+    }
+}
+
 // Independent sets until every point is decided (at most kPmisRounds rounds), in
 // one cooperative launch: along every strong edge between two undecided points
 // the one of smaller weight is not a local maximum; local maxima become C;
@@ -126,13 +143,22 @@ __global__ void __launch_bounds__(kLoopThreads) k_pmis(int n, int W, const int* 
         for (int i = first; i < n; i += step) {
             if (state[i] != 0) continue;
             const unsigned long long m = S[i];
-            for (int s = 1; s < W; ++s) {
-                if (!(m >> s & 1ull)) continue;
-                const int j = col[(size_t)i * W + s];
-                if (state[j] != 0) continue;
-                if (w[j] > w[i]) notmax[i] = 1;
-                else notmax[j] = 1;
-            }
+            const double wi = w[i];
+            for_neighbours(col + (size_t)i * W, W, [&](const int* j, unsigned) {
+                int8_t sj[kAhead];
+                double wj[kAhead];
+#pragma unroll
+                for (int k = 0; k < kAhead; ++k) {
+                    sj[k] = j[k] >= 0 ? state[j[k]] : 1;
+                    wj[k] = j[k] >= 0 ? w[j[k]] : 0.0;
+                }
+#pragma unroll
+                for (int k = 0; k < kAhead; ++k) {
+                    if (sj[k] != 0) continue;
+                    if (wj[k] > wi) notmax[i] = 1;
+                    else notmax[j[k]] = 1;
+                }
+            }, m);
         }
         if (first == 0) B->left[(round + 1) % 3] = 0;
         if (!G.sync()) return;
@@ -144,10 +170,11 @@ __global__ void __launch_bounds__(kLoopThreads) k_pmis(int n, int W, const int* 
         int cnt = 0;
         for (int i = first; i < n; i += step) {
             if (state[i] != 0) continue;
-            const unsigned long long m = S[i];
             bool f = false;
-            for (int s = 1; s < W && !f; ++s)
-                if ((m >> s & 1ull) && state[col[(size_t)i * W + s]] == 1) f = true;
+            for_neighbours(col + (size_t)i * W, W, [&](const int* j, unsigned) {
+#pragma unroll
+                for (int k = 0; k < kAhead; ++k) f |= j[k] >= 0 && state[j[k]] == 1;
+            }, S[i]);
             if (f) state[i] = 2;
             else ++cnt;
         }
@@ -223,12 +250,17 @@ __global__ void __launch_bounds__(kLoopThreads) k_colour(int n, int W, const int
     for (int round = 0; round < n; ++round) {
         for (int i = first; i < n; i += step) {
             if (colour[i] >= 0) continue;
-            for (int s = 1; s < W; ++s) {
-                const int j = col[(size_t)i * W + s];
-                if (j < 0 || j == i || colour[j] >= 0) continue;
-                if (colour_beats(j, i)) notmax[i] = 1;
-                else notmax[j] = 1;
-            }
+            for_neighbours(col + (size_t)i * W, W, [&](const int* j, unsigned) {
+                int16_t cj[kAhead];
+#pragma unroll
+                for (int k = 0; k < kAhead; ++k) cj[k] = j[k] >= 0 && j[k] != i ? colour[j[k]] : (int16_t)0;
+#pragma unroll
+                for (int k = 0; k < kAhead; ++k) {
+                    if (cj[k] >= 0) continue;
+                    if (colour_beats(j[k], i)) notmax[i] = 1;
+                    else notmax[j[k]] = 1;
+                }
+            });
         }
         if (first == 0) B->left[(round + 1) % 3] = 0;
         if (!G.sync()) return;
@@ -237,22 +269,27 @@ __global__ void __launch_bounds__(kLoopThreads) k_colour(int n, int W, const int
             if (colour[i] < 0) {
                 if (!notmax[i]) {
                     unsigned long long u0 = used[2 * i], u1 = used[2 * i + 1];
-                    for (int s = 1; s < W; ++s) {
-                        const int j = col[(size_t)i * W + s];
-                        const int c = j < 0 || j == i ? -1 : colour[j];
-                        if (c >= 64) u1 |= 1ull << (c - 64);
-                        else if (c >= 0) u0 |= 1ull << c;
-                    }
+                    for_neighbours(col + (size_t)i * W, W, [&](const int* j, unsigned) {
+                        int c[kAhead];
+#pragma unroll
+                        for (int k = 0; k < kAhead; ++k) c[k] = j[k] >= 0 && j[k] != i ? colour[j[k]] : -1;
+#pragma unroll
+                        for (int k = 0; k < kAhead; ++k) {
+                            if (c[k] >= 64) u1 |= 1ull << (c[k] - 64);
+                            else if (c[k] >= 0) u0 |= 1ull << c[k];
+                        }
+                    });
                     int c = u0 != ~0ull ? __ffsll((long long)~u0) - 1 : u1 != ~0ull ? 63 + __ffsll((long long)~u1) : -1;
                     if (c < 0) {
                         cls->over = 1;
                         c = 0;
                     }
                     colour[i] = (int16_t)c;
-                    for (int s = 1; s < W; ++s) {
-                        const int j = col[(size_t)i * W + s];
-                        if (j >= 0 && j != i) atomicOr(&used[2 * (size_t)j + (c >> 6)], 1ull << (c & 63));
-                    }
+                    for_neighbours(col + (size_t)i * W, W, [&](const int* j, unsigned) {
+#pragma unroll
+                        for (int k = 0; k < kAhead; ++k)
+                            if (j[k] >= 0 && j[k] != i) atomicOr(&used[2 * (size_t)j[k] + (c >> 6)], 1ull << (c & 63));
+                    });
                 } else {
                     ++cnt;
                 }
@@ -275,17 +312,23 @@ __global__ void k_class_count(int n, const int16_t* __restrict__ colour, const i
         atomicAdd(&cnt[class_key(cf[i], colour[i])], 1);
 }
 __global__ void k_class_list(int* __restrict__ cnt, AmgClasses* __restrict__ cls) {   // cnt becomes the cursors
-    if (threadIdx.x != 0) return;
-    int acc = 0, m = 0;
-    for (int key = 0; key < 2 * kAmgMaxColours; ++key) {
-        if (key == kAmgMaxColours) cls->nC = m;
-        const int c = cnt[key];
-        cnt[key] = acc;
-        if (c) cls->ofs[m++] = acc;
-        acc += c;
+    __shared__ int s_cnt[2 * kAmgMaxColours];
+    for (int key = threadIdx.x; key < 2 * kAmgMaxColours; key += blockDim.x) s_cnt[key] = cnt[key];
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        int acc = 0, m = 0;
+        for (int key = 0; key < 2 * kAmgMaxColours; ++key) {
+            if (key == kAmgMaxColours) cls->nC = m;
+            const int c = s_cnt[key];
+            s_cnt[key] = acc;
+            if (c) cls->ofs[m++] = acc;
+            acc += c;
+        }
+        cls->ofs[m] = acc;
+        cls->count = m;
     }
-    cls->ofs[m] = acc;
-    cls->count = m;
+    __syncthreads();
+    for (int key = threadIdx.x; key < 2 * kAmgMaxColours; key += blockDim.x) cnt[key] = s_cnt[key];
 }
 __global__ void k_class_scatter(int n, const int16_t* __restrict__ colour, const int8_t* __restrict__ cf,
                                 int* __restrict__ cursor, int* __restrict__ ord) {
@@ -738,15 +781,29 @@ __global__ void k_amg_coarse_inv(int n, int W, const int* __restrict__ col, cons
 // (A u)_i and the diagonal: float64 rows hold the entries, float32 rows the
 // row sum in slot 0 and the off-diagonals (leakage form).  The row's slots are
 // shared by `g` neighbouring lanes (this one is number `sub`), which all get the
-// results; every lane of the warp must call it.
+// results; every lane of the warp must call it.  kRowAhead slots are loaded
+// together: one by one, each slot's column and then its u are a chain of two
+// latencies.
+constexpr int kRowAhead = 4;
 template <typename T>
 __device__ __forceinline__ void amg_row(const AmgLevelArgs& L, int i, const T* u, int sub, int g, T* Au, T* d) {
     const int* c = L.col + (size_t)i * L.W;
     if constexpr (sizeof(T) == 8) {
         const double* a = L.a64 + (size_t)i * L.W;
         double s = 0.0;
-        for (int k = sub; k < L.W; k += g)
-            if (c[k] >= 0) s = fma(a[k], u[c[k]], s);
+        for (int k = sub; k < L.W; k += kRowAhead * g) {
+            int j[kRowAhead];
+            double v[kRowAhead];
+#pragma unroll
+            for (int q = 0; q < kRowAhead; ++q) {
+                const bool in = k + q * g < L.W;
+                j[q] = in ? c[k + q * g] : -1;
+                v[q] = in ? a[k + q * g] : 0.0;
+            }
+#pragma unroll
+            for (int q = 0; q < kRowAhead; ++q)
+                if (j[q] >= 0) s = fma(v[q], u[j[q]], s);
+        }
         for (int o = 1; o < g; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
         *Au = s;
         *d = a[0];
@@ -754,10 +811,22 @@ __device__ __forceinline__ void amg_row(const AmgLevelArgs& L, int i, const T* u
         const float* a = L.a32 + (size_t)i * L.W;
         const float ui = u[i], lead = a[0];
         float s = 0.0f, dg = 0.0f;
-        for (int k = 1 + sub; k < L.W; k += g) {
-            if (c[k] < 0) continue;
-            s = fmaf(a[k], u[c[k]] - ui, s);
-            dg += a[k];
+        for (int k = 1 + sub; k < L.W; k += kRowAhead * g) {
+            int j[kRowAhead];
+            float v[kRowAhead], w[kRowAhead];
+#pragma unroll
+            for (int q = 0; q < kRowAhead; ++q) {
+                const bool in = k + q * g < L.W;
+                j[q] = in ? c[k + q * g] : -1;
+                v[q] = in ? a[k + q * g] : 0.0f;
+            }
+#pragma unroll
+            for (int q = 0; q < kRowAhead; ++q) w[q] = j[q] >= 0 ? u[j[q]] : ui;   // empty slots hold 0
+#pragma unroll
+            for (int q = 0; q < kRowAhead; ++q) {
+                s = fmaf(v[q], w[q] - ui, s);
+                dg += v[q];
+            }
         }
         for (int o = 1; o < g; o <<= 1) {
             s += __shfl_xor_sync(0xffffffffu, s, o);
@@ -1829,7 +1898,7 @@ void AmgHierarchy::colour_level(AmgLevelMem& F, int* flag, AmgLoop* loop, unsign
     GS_CUDA(cudaLaunchCooperativeKernel((const void*)k_colour, dim3(loop_blocks(nf, max_blocks)), dim3(kLoopThreads),
                                         args, 0, st));
     k_class_count<<<g, 256, 0, st>>>(nf, colour, F.cf, cnt);
-    k_class_list<<<1, 32, 0, st>>>(cnt, F.cls);
+    k_class_list<<<1, 256, 0, st>>>(cnt, F.cls);
     k_class_scatter<<<g, 256, 0, st>>>(nf, colour, F.cf, cnt, F.ord);
     GS_CHECK_LAUNCH_N(4);
 }

@@ -285,7 +285,9 @@ void worker(gs_server* S, int slot) {
     if (o.grid_blocks == 0) {
         int sms = 152;
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, S->device);
-        o.grid_blocks = std::max(1, 2 * sms / S->slots);
+        // the cooperative kernels take one block per SM: slots that share the SMs
+        // run side by side, slots that each ask for all of them in turn
+        o.grid_blocks = std::max(1, sms / S->slots);
     }
     gs_solver* solver = nullptr;
     const gs_status created = gamesolve_create(&solver, &o);
