@@ -531,6 +531,41 @@ __device__ __forceinline__ float* setup_P32(const SolveArgs& a, const LevelArgs&
     return a.wbf16 ? (float*)L.P64 : L.P32;
 }
 
+// Galerkin rows 0 .. nc - 1: store(sum of the row's three parts, t).  A level with
+// at most two warps of rows per block gives the parts of 32 rows to three warps
+// (the chain of one row is what the phase takes there); larger levels a row to
+// a thread.  Either way a row is (part -1 + part 0) + part 1.
+template <typename V, class Part, class Store>
+__device__ __forceinline__ void rap_rows(unsigned nc, size_t start, size_t stride, Part&& part, Store&& store) {
+    __shared__ V parts[2][2][9][32];   // [slot][part 0, 1][entry][row]
+    if (nc <= 64u * gridDim.x) {
+        const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, slot = w / 3, oy = w % 3;
+        const unsigned t = (slot * gridDim.x + blockIdx.x) * 32 + lane;
+        const bool in = w < 6 && t < nc;
+        RapPart<V> R;
+        if (in) {
+            R = part(oy - 1, t);
+            if (oy > 0)
+#pragma unroll
+                for (int d = 0; d < 9; ++d) parts[slot][oy - 1][d][lane] = R.a[d];
+        }
+        __syncthreads();
+        if (in && oy == 0) {
+#pragma unroll
+            for (int d = 0; d < 9; ++d) R.a[d] = (R.a[d] + parts[slot][0][d][lane]) + parts[slot][1][d][lane];
+            store(R, t);
+        }
+        __syncthreads();
+        return;
+    }
+    for (unsigned t = (unsigned)start; t < nc; t += (unsigned)stride) {
+        RapPart<V> R = part(-1, t);
+        R.add(part(0, t));
+        R.add(part(1, t));
+        store(R, t);
+    }
+}
+
 // Mixed path set-up items (float32, exact leakage); delta(g) lives in the
 // level's spare vector, free during the set-up.
 __device__ void setup_items_f(const SolveArgs& a, int l, int kind, size_t start, size_t stride) {
@@ -557,10 +592,15 @@ __device__ void setup_items_f(const SolveArgs& a, int l, int kind, size_t start,
         float* Ac = setup_A32(a, C);
         __nv_bfloat16* A16 = a.wbf16 ? (__nv_bfloat16*)C.A32 : nullptr;
         const unsigned nc = (unsigned)sc * sc;
-        for (unsigned t = (unsigned)start; t < nc; t += (unsigned)stride) {
-            if (l == 0) rap_item_f(s5, sc, t, P, delta, Ac, A16);
-            else rap_item_f(s9, sc, t, P, delta, Ac, A16);
-        }
+        auto part = [&](int oy, unsigned t) {
+            if (l == 0)
+                return oy < 0 ? rap_part_f<-1>(s5, sc, t, P, delta)
+                              : oy == 0 ? rap_part_f<0>(s5, sc, t, P, delta) : rap_part_f<1>(s5, sc, t, P, delta);
+            return oy < 0 ? rap_part_f<-1>(s9, sc, t, P, delta)
+                          : oy == 0 ? rap_part_f<0>(s9, sc, t, P, delta) : rap_part_f<1>(s9, sc, t, P, delta);
+        };
+        rap_rows<float>(nc, start, stride, part,
+                        [&](const RapPart<float>& R, unsigned t) { rap_store_f(R, nc, t, Ac, A16); });
     }
 }
 
@@ -590,10 +630,16 @@ __device__ void setup_items(const SolveArgs& a, int l, int kind, size_t start, s
         const size_t nc = (size_t)sc * sc;
         const LevelArgs& C = a.L[l + 1];
         const WOut Aw{a.mixed && !a.wbf16 ? C.A32 : nullptr, a.wbf16 ? (__nv_bfloat16*)C.A32 : nullptr};
-        for (size_t t = start; t < nc; t += stride) {
-            if (l == 0) rap_item(Src5{a.K, a.code, L.side}, sc, t, L.P64, C.A64, Aw);
-            else rap_item(Src9{L.A64, L.side, L.n}, sc, t, L.P64, C.A64, Aw);
-        }
+        const Src5 s5{a.K, a.code, L.side};
+        const Src9 s9{L.A64, L.side, L.n};
+        const double* P = L.P64;
+        auto part = [&](int oy, unsigned t) {
+            if (l == 0)
+                return oy < 0 ? rap_part<-1>(s5, sc, t, P) : oy == 0 ? rap_part<0>(s5, sc, t, P) : rap_part<1>(s5, sc, t, P);
+            return oy < 0 ? rap_part<-1>(s9, sc, t, P) : oy == 0 ? rap_part<0>(s9, sc, t, P) : rap_part<1>(s9, sc, t, P);
+        };
+        rap_rows<double>((unsigned)nc, start, stride, part,
+                         [&](const RapPart<double>& R, unsigned t) { rap_store(R, nc, t, C.A64, Aw); });
     }
 }
 

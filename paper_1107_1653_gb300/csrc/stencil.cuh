@@ -374,49 +374,60 @@ __device__ __forceinline__ void rap_scatter(const V* P, int sc, int I, int J, in
     }
 }
 
-// Galerkin coarse row A_c(t, .) = (P^T A P)(t, .) for the coarse point t
-// (float64 accumulation); also its rounded leakage form (row sum, then the
-// off-diagonal entries) when Aw has a destination.
-template <class Src>
-__device__ __forceinline__ void rap_item(const Src& src, int sc, size_t t, const double* P,
-                                         double* Ac, const WOut& Aw) {
-    const size_t nc = (size_t)sc * sc;
-    const int I = (int)(t % sc), J = (int)(t / sc);
+// Part of the Galerkin coarse row A_c(t, .) = (P^T A P)(t, .) of the coarse point
+// t: the products of the fine rows 2 J + 1 + OY of its stencil (float64).  A row
+// is the sum of its three parts, formed in this order whether one thread
+// computes them in turn or three warps at once (small levels, where a part's
+// chain of operations is what a phase takes).
+template <class V>
+struct RapPart {
+    V a[9];
+    __device__ __forceinline__ void add(const RapPart& o) {
+#pragma unroll
+        for (int d = 0; d < 9; ++d) a[d] += o.a[d];
+    }
+};
+template <int OY, class Src>
+__device__ __noinline__ RapPart<double> rap_part(const Src src, int sc, unsigned t, const double* P) {
+    const int I = (int)(t % (unsigned)sc), J = (int)(t / (unsigned)sc);
     const int sf = 2 * sc + 1;
-    double acc[9];
+    RapPart<double> R;
 #pragma unroll
-    for (int d = 0; d < 9; ++d) acc[d] = 0.0;
+    for (int d = 0; d < 9; ++d) R.a[d] = 0.0;
 #pragma unroll
-    for (int oy = -1; oy <= 1; ++oy) {
+    for (int ox = -1; ox <= 1; ++ox) {
+        const double w = restrict_weight(P, sc, I, J, ox, OY);
+        double a[9];
+        src.row(2 * I + 1 + ox, 2 * J + 1 + OY, a);
 #pragma unroll
-        for (int ox = -1; ox <= 1; ++ox) {
-            const double R = restrict_weight(P, sc, I, J, ox, oy);
-            double a[9];
-            src.row(2 * I + 1 + ox, 2 * J + 1 + oy, a);
-#pragma unroll
-            for (int d = 0; d < 9; ++d) {
-                // The 5-point rows' diagonal entries are zero: skip them at
-                // compile time.  No test on loaded values: it would make each
-                // weight load below wait for the row's load.
-                if constexpr (Src::kFivePoint)
-                    if (d >= DSW) continue;
-                const int qx = ox + dir_di(d), qy = oy + dir_dj(d);
-                const int gi = 2 * I + 1 + qx, gj = 2 * J + 1 + qy;
-                if (gi < 0 || gj < 0 || gi >= sf || gj >= sf) continue;
-                rap_scatter(P, sc, I, J, qx, qy, R * a[d], acc);
-            }
+        for (int d = 0; d < 9; ++d) {
+            // The 5-point rows' diagonal entries are zero: skip them at
+            // compile time.  No test on loaded values: it would make each
+            // weight load below wait for the row's load.
+            if constexpr (Src::kFivePoint)
+                if (d >= DSW) continue;
+            const int qx = ox + dir_di(d), qy = OY + dir_dj(d);
+            const int gi = 2 * I + 1 + qx, gj = 2 * J + 1 + qy;
+            if (gi < 0 || gj < 0 || gi >= sf || gj >= sf) continue;
+            rap_scatter(P, sc, I, J, qx, qy, w * a[d], R.a);
         }
     }
+    return R;
+}
+
+// The row of coarse point t from its parts' sum: the entries, and their rounded
+// leakage form (row sum, then the off-diagonal entries) when Aw has a destination.
+__device__ __forceinline__ void rap_store(const RapPart<double>& R, size_t nc, unsigned t, double* Ac, const WOut& Aw) {
     double s = 0.0;
 #pragma unroll
     for (int d = 0; d < 9; ++d) {
-        Ac[d * nc + t] = acc[d];
-        s += acc[d];
+        Ac[d * nc + t] = R.a[d];
+        s += R.a[d];
     }
     if (Aw.any()) {
         Aw.put(t, s);
 #pragma unroll
-        for (int d = 1; d < 9; ++d) Aw.put(d * nc + t, acc[d]);
+        for (int d = 1; d < 9; ++d) Aw.put(d * nc + t, R.a[d]);
     }
 }
 
@@ -611,56 +622,58 @@ __device__ __forceinline__ float delta_at(const float* P, const float* delta, in
     return d;
 }
 
-// Galerkin coarse row t in float32 leakage form: Ac[t] = its row sum from
-// R (s + A delta), Ac[d * nc + t] = its off-diagonal entries (and A16 their
-// bfloat16 copy when given).
-template <class Src>
-__device__ __forceinline__ void rap_item_f(const Src& src, int sc, unsigned t, const float* P,
-                                           const float* delta, float* Ac, __nv_bfloat16* A16) {
-    const unsigned nc = (unsigned)sc * sc;
+// Part of the Galerkin coarse row t in float32 leakage form: slot 0 its row sum's
+// share from R (s + A delta), slots 1 .. 8 the off-diagonal entries' (as rap_part).
+template <int OY, class Src>
+__device__ __noinline__ RapPart<float> rap_part_f(const Src src, int sc, unsigned t, const float* P,
+                                                  const float* delta) {
     const int I = (int)(t % (unsigned)sc), J = (int)(t / (unsigned)sc);
     const int sf = 2 * sc + 1;
-    float dl[5][5];
+    float dl[3][5];
 #pragma unroll
-    for (int qy = -2; qy <= 2; ++qy)
+    for (int qy = -1; qy <= 1; ++qy)
 #pragma unroll
         for (int qx = -2; qx <= 2; ++qx) {
-            const int gi = 2 * I + 1 + qx, gj = 2 * J + 1 + qy;
+            const int gi = 2 * I + 1 + qx, gj = 2 * J + 1 + OY + qy;
             const bool in = gi >= 0 && gj >= 0 && gi < sf && gj < sf;
-            dl[qy + 2][qx + 2] = in ? delta_at(P, delta, sc, gi, gj) : 0.0f;
+            dl[qy + 1][qx + 2] = in ? delta_at(P, delta, sc, gi, gj) : 0.0f;
         }
     float acc[9];
 #pragma unroll
     for (int d = 0; d < 9; ++d) acc[d] = 0.0f;
     float rowsum = 0.0f;
 #pragma unroll
-    for (int oy = -1; oy <= 1; ++oy) {
+    for (int ox = -1; ox <= 1; ++ox) {
+        const float w = restrict_weight(P, sc, I, J, ox, OY);
+        float a[9], s;
+        src.row(2 * I + 1 + ox, 2 * J + 1 + OY, a, &s);
+        float inner = s;   // (A (P 1))(f) = s_f + sum_g A(f, g) delta(g)
 #pragma unroll
-        for (int ox = -1; ox <= 1; ++ox) {
-            const float R = restrict_weight(P, sc, I, J, ox, oy);
-            float a[9], s;
-            src.row(2 * I + 1 + ox, 2 * J + 1 + oy, a, &s);
-            float inner = s;   // (A (P 1))(f) = s_f + sum_g A(f, g) delta(g)
-#pragma unroll
-            for (int d = 0; d < 9; ++d) {
-                if constexpr (Src::kFivePoint)
-                    if (d >= DSW) continue;
-                const int qx = ox + dir_di(d), qy = oy + dir_dj(d);
-                inner += a[d] * dl[qy + 2][qx + 2];
-                const int gi = 2 * I + 1 + qx, gj = 2 * J + 1 + qy;
-                if (gi < 0 || gj < 0 || gi >= sf || gj >= sf) continue;
-                rap_scatter(P, sc, I, J, qx, qy, R * a[d], acc);
-            }
-            rowsum += R * inner;
+        for (int d = 0; d < 9; ++d) {
+            if constexpr (Src::kFivePoint)
+                if (d >= DSW) continue;
+            const int qx = ox + dir_di(d), qy = OY + dir_dj(d);
+            inner += a[d] * dl[dir_dj(d) + 1][qx + 2];
+            const int gi = 2 * I + 1 + qx, gj = 2 * J + 1 + qy;
+            if (gi < 0 || gj < 0 || gi >= sf || gj >= sf) continue;
+            rap_scatter(P, sc, I, J, qx, qy, w * a[d], acc);
         }
+        rowsum += w * inner;
     }
-    Ac[t] = rowsum;
+    RapPart<float> R;
+    R.a[0] = rowsum;
 #pragma unroll
-    for (int d = 1; d < 9; ++d) Ac[d * nc + t] = acc[d];
+    for (int d = 1; d < 9; ++d) R.a[d] = acc[d];
+    return R;
+}
+
+// The row of coarse point t from its parts' sum (and its bfloat16 copy).
+__device__ __forceinline__ void rap_store_f(const RapPart<float>& R, size_t nc, unsigned t, float* Ac, __nv_bfloat16* A16) {
+#pragma unroll
+    for (int d = 0; d < 9; ++d) Ac[d * nc + t] = R.a[d];
     if (A16) {
-        A16[t] = __float2bfloat16_rn(rowsum);
 #pragma unroll
-        for (int d = 1; d < 9; ++d) A16[d * nc + t] = __float2bfloat16_rn(acc[d]);
+        for (int d = 0; d < 9; ++d) A16[d * nc + t] = __float2bfloat16_rn(R.a[d]);
     }
 }
 
