@@ -217,9 +217,11 @@ struct ImprovePoint {
 template <int MODE>
 __global__ void __launch_bounds__(kBlock) k_isaacs_improve(const __grid_constant__ ImproveArgs A, double tau_host,
                                                            float tau_host_f, int tau_from_vmax) {
+    if (A.skip && *A.skip == A.skip_if) return;
     const IsaacsConsts* __restrict__ K = A.K;
     const int side = A.side, variant = A.variant;
-    const DevScalars* sc = A.sc;
+    const double tau = tau_from_vmax ? tau_of_vmax(A.sc) : tau_host;
+    const float tauf = tau_from_vmax ? f64_to_f32(tau) : tau_host_f;
     const unsigned n = (unsigned)side * side, stride = gridDim.x * blockDim.x;
     const FastDiv dv((unsigned)side);
     double wsq = 0.0;
@@ -248,7 +250,6 @@ __global__ void __launch_bounds__(kBlock) k_isaacs_improve(const __grid_constant
         // four in five to a few in a hundred).  The inner mode takes one decision
         // instead of five: there the four subtractions would cost what they save.
         const float gf = K->gmu_f, cf = K->c01_f;
-        const float tauf = tau_from_vmax ? f64_to_f32(tau_of_vmax(sc)) : tau_host_f;
         float fx, fE, fW, fN, fS, err;
         if (MODE == IMP_INNER) {
             fx = f64_to_f32(nb.vx);
@@ -348,7 +349,6 @@ __global__ void __launch_bounds__(kBlock) k_isaacs_improve(const __grid_constant
                     // near-tie: keep the current action unless beaten by more than
                     // tau (a current move other than the best one is: by its margin)
                     const double fcur = acur == 4 ? psi : fmax_, top = anew == 4 ? psi : fmax_;
-                    const double tau = tau_from_vmax ? tau_of_vmax(sc) : tau_host;
                     if ((acur == 4 || acur == amax) && !(top - fcur > tau)) anew = acur;
                     fmax_ = top;
                 } else if (stop) {
@@ -356,8 +356,7 @@ __global__ void __launch_bounds__(kBlock) k_isaacs_improve(const __grid_constant
                 }
             }
         } else {
-            improve_exact<MODE>(K, nb, rx, i, j, m1, acur, bw, tau_from_vmax ? tau_of_vmax(sc) : tau_host,
-                                &bnew, &anew, &fmax_);
+            improve_exact<MODE>(K, nb, rx, i, j, m1, acur, bw, tau, &bnew, &anew, &fmax_);
         }
         if (MODE == IMP_OUTER) {
             changed = anew != acur;

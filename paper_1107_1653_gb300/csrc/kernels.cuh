@@ -42,6 +42,8 @@ struct ImproveArgs {
     const uint8_t* beta4;
     DevScalars* sc;
     double tau;
+    const int* skip;   // where *skip is skip_if, nothing is done (null: never)
+    int skip_if;
 };
 void launch_isaacs_improve(ImproveMode mode, const ImproveArgs& a, cudaStream_t st);
 

@@ -877,6 +877,7 @@ __global__ void __launch_bounds__(kMGThreads) k_mg_cycles(const __grid_constant_
                 a.out->reason = reason;
                 a.out->res = res;
                 a.out->vmax_final = vm;
+                if (a.vmax_out) *a.vmax_out = abs_bits(vm);
             }
             return;
         }
@@ -1472,6 +1473,7 @@ __global__ void __launch_bounds__(kTiledThreads, 1) k_mg_cycles_tiled(const __gr
                 a.out->reason = reason;
                 a.out->res = res;
                 a.out->vmax_final = vm;
+                if (a.vmax_out) *a.vmax_out = abs_bits(vm);
             }
             return;
         }

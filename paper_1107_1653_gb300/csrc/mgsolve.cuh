@@ -65,6 +65,7 @@ struct SolveArgs {
     int tile_from;   // tiled cycles: coarse levels l >= tile_from are tiled, larger ones
                      // (1 <= l < tile_from) take one grid-wide phase per colour
     int tc[kMaxLevels];   // tile side of level l >= 1, in points of level l + 1
+    unsigned long long* vmax_out;   // |v|_inf at the end (bits) also goes here (null: nowhere)
     double* inv;     // inverse of the coarsest operator (n_L x n_L)
     int* inv_status;
     GridBarrier* bar;

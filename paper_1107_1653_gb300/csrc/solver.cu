@@ -20,6 +20,16 @@ Arena::~Arena() {
 
 void* Arena::raw(size_t bytes) {
     bytes = (bytes + 255) & ~size_t(255);
+    if (measuring_) {
+        measured_ += bytes;
+        return nullptr;
+    }
+    if (bytes <= left_) {
+        void* p = next_;
+        next_ += bytes;
+        left_ -= bytes;
+        return p;
+    }
     if (budget_ && base_ + held_ + bytes > budget_) {
         set_last_error("device memory budget exceeded: %zu + %zu > %zu bytes", base_ + held_, bytes,
                        budget_);
@@ -35,6 +45,11 @@ void* Arena::raw(size_t bytes) {
     ptrs_.push_back(p);
     held_ += bytes;
     return p;
+}
+
+void Arena::reserve(size_t bytes) {
+    next_ = static_cast<char*>(raw(bytes));
+    left_ = bytes;
 }
 
 // ------------------------------------------------------------------ tracing
@@ -204,22 +219,22 @@ void set_fine_planes(Level& L, float* p, cudaStream_t st) {
     L.f32 = p + plane + fine_plane_origin(L.side);
 }
 
-static void alloc_grid(gs_solver* s, Arena& ar, IsaacsGrid& g) {
+// The arrays of one grid, taken from the arena (which may be only measuring).
+// Returns the finest level's float32 planes.
+static float* take_grid(const gs_options& opt, Arena& ar, IsaacsGrid& g) {
     const size_t n = g.n;
     g.Kd = ar.alloc<IsaacsConsts>(1);
-    GS_CUDA(cudaMemcpyAsync(g.Kd, &g.Kh, sizeof(IsaacsConsts), cudaMemcpyHostToDevice, s->st));
     g.r0 = ar.alloc<double>(n);
     g.v = ar.alloc<double>(n);
     g.rhs = ar.alloc<double>(n);
     g.fv = ar.alloc<double>(n);
     g.alpha = ar.alloc<uint8_t>(n);
     g.code = ar.alloc<uint8_t>(code_bytes(g.side));
-    GS_CUDA(cudaMemsetAsync(g.code, kStopCode, code_bytes(g.side), s->st));
     g.beta = ar.alloc<uint32_t>(n);
     g.beta4 = ar.alloc<uint8_t>(n);
     g.dstatus = ar.alloc<int>(4);
     // multigrid levels
-    const int coarse_max = std::max(1, std::min<int>(s->opt.coarse_max, 64));
+    const int coarse_max = std::max(1, std::min<int>(opt.coarse_max, 64));
     int side = g.side;
     g.lv.clear();
     while (true) {
@@ -230,6 +245,7 @@ static void alloc_grid(gs_solver* s, Arena& ar, IsaacsGrid& g) {
         if ((int)L.n <= coarse_max || side < 3) break;
         side = (side - 1) / 2;
     }
+    float* planes = nullptr;
     for (size_t l = 0; l < g.lv.size(); ++l) {
         Level& L = g.lv[l];
         if (l > 0) {
@@ -237,15 +253,12 @@ static void alloc_grid(gs_solver* s, Arena& ar, IsaacsGrid& g) {
             L.A32 = ar.alloc<float>(9 * L.n);
             L.u64 = ar.alloc<double>(L.n);
             L.f64 = ar.alloc<double>(L.n);
-        }
-        L.r64 = ar.alloc<double>(L.n);
-        if (l == 0) {
-            float* p = ar.alloc<float>(2 * fine_plane_elems(L.side));
-            set_fine_planes(L, p, s->st);
-        } else {
             L.u32 = ar.alloc<float>(L.n);
             L.f32 = ar.alloc<float>(L.n);
+        } else {
+            planes = ar.alloc<float>(2 * fine_plane_elems(L.side));
         }
+        L.r64 = ar.alloc<double>(L.n);
         L.r32 = ar.alloc<float>(L.n);
         if (l + 1 < g.lv.size()) {
             const size_t sc = (size_t)(L.side - 1) / 2;
@@ -255,6 +268,19 @@ static void alloc_grid(gs_solver* s, Arena& ar, IsaacsGrid& g) {
     }
     const int nL = (int)g.lv.back().n;
     g.inv = ar.alloc<double>((size_t)nL * nL);
+    return planes;
+}
+
+// One allocation per grid instead of some 60 (a microsecond or two each, and as
+// many frees when the problem is replaced).
+static void alloc_grid(gs_solver* s, Arena& ar, IsaacsGrid& g) {
+    Arena size = Arena::measure();
+    take_grid(s->opt, size, g);
+    ar.reserve(size.measured());
+    float* planes = take_grid(s->opt, ar, g);
+    GS_CUDA(cudaMemcpyAsync(g.Kd, &g.Kh, sizeof(IsaacsConsts), cudaMemcpyHostToDevice, s->st));
+    GS_CUDA(cudaMemsetAsync(g.code, kStopCode, code_bytes(g.side), s->st));
+    set_fine_planes(g.lv[0], planes, s->st);
 }
 
 std::unique_ptr<Problem> build_isaacs_problem(gs_solver* s, int side, int variant, uint64_t seed,
@@ -325,6 +351,12 @@ int tail_level(const gs_solver* s, const IsaacsGrid& g) {
     return Lc;
 }
 
+// Improvement arguments on the grid's own arrays.
+ImproveArgs improve_args(gs_solver* s, IsaacsGrid& g, double* fv, double tau) {
+    return {g.Kd,   g.side, g.variant, g.v, g.r0,    g.alpha, g.beta, g.alpha,
+            g.beta, g.code, g.rhs,     fv,  nullptr, g.beta4, s->dsc, tau, nullptr, 0};
+}
+
 // Solves (I - mu M) v = r for the assembled codes/rhs of g, warm-started from
 // g.v, in one cooperative launch: Galerkin set-up for the current policies,
 // then float64 V-cycles, or float32 V-cycles on the float64 residual with
@@ -334,7 +366,10 @@ int tail_level(const gs_solver* s, const IsaacsGrid& g) {
 // call (valid when the policy codes are unchanged).  Returns why the solve
 // stopped: kLinExact (float64 floor or tolerance), kLinInexact (the residual
 // fell by rel_tol) or kLinCapped (max_cycles reached short of both).
-int linear_solve(gs_solver* s, IsaacsGrid& g, Counters& cnt, double rel_tol, bool do_setup) {
+// With `improve` MIN's replies at the solution are improved in the same go (one
+// read-back for both; not done where the solve was capped): the changed entries
+// are then in s->hsc.
+int linear_solve(gs_solver* s, IsaacsGrid& g, Counters& cnt, double rel_tol, bool do_setup, bool improve = false) {
     const bool mixed = s->opt.precision != GS_PREC_FP64;
     SolveArgs a{};
     a.K = g.Kd;
@@ -414,6 +449,10 @@ int linear_solve(gs_solver* s, IsaacsGrid& g, Counters& cnt, double rel_tol, boo
     while (a.smem_from < a.nlev && tail_smem_bytes(a) > (size_t)kTailSmemMax)
         ++a.smem_from;
     GS_CUDA(cudaMemsetAsync(s->mgd, 0, sizeof(MGState), s->st));
+    if (improve) {
+        clear_scalars(s);
+        a.vmax_out = &s->dsc->vmax;   // the improvement's keep-current tolerance
+    }
     if (do_setup) {
         KScope ks(s, GS_K_MG_SETUP);
         launch_mg_setup(a, s->st);
@@ -422,7 +461,15 @@ int linear_solve(gs_solver* s, IsaacsGrid& g, Counters& cnt, double rel_tol, boo
         KScope ks(s, GS_K_MG_CYCLES);
         launch_mg_cycles(a, s->st);
     }
+    if (improve) {
+        KScope ks(s, GS_K_IMPROVE);
+        ImproveArgs A = improve_args(s, g, nullptr, -1.0);
+        A.skip = &s->mgd->out.reason;
+        A.skip_if = kLinCapped;
+        launch_isaacs_improve(IMP_INNER, A, s->st);
+    }
     GS_CUDA(cudaMemcpyAsync(s->mgh, s->mgd, sizeof(MGState), cudaMemcpyDeviceToHost, s->st));
+    if (improve) GS_CUDA(cudaMemcpyAsync(s->hsc, s->dsc, sizeof(DevScalars), cudaMemcpyDeviceToHost, s->st));
     sync(s);
     if (s->mgh->bar.error) {
         set_last_error("multigrid solve: a grid barrier wait timed out");
@@ -441,6 +488,7 @@ int linear_solve(gs_solver* s, IsaacsGrid& g, Counters& cnt, double rel_tol, boo
     cnt.last_lin_res = s->mgh->out.res;
     const int why = s->mgh->out.reason;
     if (why == kLinCapped) cnt.lin_capped = true;
+    else if (improve) g.stale_rows += s->hsc->code_changed;
     return why;
 }
 
@@ -460,12 +508,6 @@ void vmax_to_device(gs_solver* s, IsaacsGrid& g) {
     launch_absmax(g.v, g.n, &s->dsc->vmax, s->st);
 }
 
-// Improvement arguments on the grid's own arrays.
-ImproveArgs improve_args(gs_solver* s, IsaacsGrid& g, double* fv, double tau) {
-    return {g.Kd,   g.side, g.variant, g.v, g.r0,    g.alpha, g.beta, g.alpha,
-            g.beta, g.code, g.rhs,     fv,  nullptr, g.beta4, s->dsc, tau};
-}
-
 // AMGpi (Sec. 5.1): Algorithm 2 with Algorithm 1 inside, every linear system
 // solved by multigrid.  Starts from g.v, g.alpha and (if beta_given) g.beta.
 bool amgpi(gs_solver* s, IsaacsGrid& g, double eps, bool beta_given, Counters& cnt) {
@@ -481,24 +523,17 @@ bool amgpi(gs_solver* s, IsaacsGrid& g, double eps, bool beta_given, Counters& c
     bool converged = false;
     int outer = 0;
     while (true) {
-        auto inner_improve = [&]() {
-            clear_scalars(s);
-            KScope ks(s, GS_K_IMPROVE);
-            launch_isaacs_improve(IMP_INNER, improve_args(s, g, nullptr, tie_tol(s)), st);
-            const DevScalars& h = read_scalars(s);
-            g.stale_rows += h.code_changed;
-            return h.changed;
-        };
         for (int j = 0; j < s->opt.max_inner; ++j) {
             // Algorithm 1 step 1: evaluate MIN's policy (inexactly inside the loop)
-            const int why = linear_solve(s, g, cnt, s->opt.pi_rtol, need_setup(s, g));
+            // and, in the same go, improve its replies
+            const int why = linear_solve(s, g, cnt, s->opt.pi_rtol, need_setup(s, g), true);
             ++cnt.systems;
             if (why == kLinCapped) break;   // not evaluated: no decision may rest on it
-            if (inner_improve() != 0) continue;
+            if (s->hsc->changed != 0) continue;
             if (why == kLinInexact) {
                 // confirm on the float64-floor solution of the same system before stopping
-                if (linear_solve(s, g, cnt, 0.0, need_setup(s, g)) == kLinCapped) break;
-                if (inner_improve() != 0) continue;
+                if (linear_solve(s, g, cnt, 0.0, need_setup(s, g), true) == kLinCapped) break;
+                if (s->hsc->changed != 0) continue;
             }
             break;
         }
@@ -670,7 +705,7 @@ gs_status run_improve(gs_solver* s, const double* v, uint8_t* alpha_out, uint8_t
     launch_absmax(vd, n, &s->dsc->vmax, s->st);
     const ImproveArgs A{g.Kd, g.side, g.variant, vd, g.r0, g.alpha, g.beta, a,
                         m1 == 4 ? reinterpret_cast<uint32_t*>(b) : nullptr, nullptr, nullptr, fv,
-                        m1 == 5 ? b : nullptr, g.beta4, s->dsc, -1.0};
+                        m1 == 5 ? b : nullptr, g.beta4, s->dsc, -1.0, nullptr, 0};
     launch_isaacs_improve(IMP_OUTER, A, s->st);
     if (a && !da) GS_CUDA(cudaMemcpyAsync(alpha_out, a, n, cudaMemcpyDefault, s->st));
     if (fv && !df) GS_CUDA(cudaMemcpyAsync(fv_out, fv, nv, cudaMemcpyDefault, s->st));

@@ -28,10 +28,18 @@ public:
     }
     void* raw_bytes(size_t bytes) { return raw(bytes); }
     size_t held() const { return held_; }
+    // One allocation of this size, which the next ones are cut from.
+    void reserve(size_t bytes);
+    // An arena that only adds up what it is asked for (alloc returns null).
+    static Arena measure() { return Arena(true); }
+    size_t measured() const { return measured_; }
 
 private:
+    explicit Arena(bool) : budget_(0), base_(0), measuring_(true), st_(nullptr) {}
     void* raw(size_t bytes);
-    size_t budget_, base_, held_ = 0;
+    size_t budget_, base_, held_ = 0, measured_ = 0, left_ = 0;
+    char* next_ = nullptr;
+    bool measuring_ = false;
     cudaStream_t st_;
     std::vector<void*> ptrs_;
 };
