@@ -1955,7 +1955,7 @@ int AmgHierarchy::solve(double* v, const double* rhs, const gs_options& opt, dou
         while (a.tail > 0) {
             const AmgLevelMem& L = lv[a.tail - 1];
             const size_t more = (size_t)L.n * (sizeof(int) + 3 * (mixed ? sizeof(float) : sizeof(double))) + 64;
-            if (L.n > (mixed ? kAmgTailN : kAmgTailNF64) || smem + more > (size_t)kAmgSmemMax) break;
+            if (L.n > kAmgTailN || smem + more > (size_t)kAmgSmemMax) break;
             smem += more;
             --a.tail;
         }

@@ -18,9 +18,9 @@ constexpr int kAmgInvSmem = 64;         // inverted in shared memory up to this 
 constexpr int kAmgRowCap = 96;          // entries of a coarse row the set-up accumulates
 constexpr int kAmgCoarseSweeps = 30;    // Jacobi sweeps on a coarsest level too large to invert
 constexpr int kAmgMaxColours = 128;     // colours of the Gauss-Seidel smoother's colouring
-constexpr int kAmgTailN = 6144;         // levels this small run in one thread block, with
-constexpr int kAmgTailNF64 = 2048;      // block barriers instead of grid barriers (in float64
-                                        // one SM's float64 pipe is the bound sooner)
+constexpr int kAmgTailN = 2048;         // levels this small run in one thread block, with
+                                        // block barriers instead of grid barriers (tables of
+                                        // a 127^2 grid, mixed: 58.0 ms; up to 6144 points 60.2)
 constexpr int kAmgSmemMax = 200 * 1024; // shared memory of a cycle launch
 
 // The smoother's classes of one level: C points by colour, then F points by

@@ -136,12 +136,14 @@ struct L0Op<double> {
         s = fma(-am[4], uN, s);
         return over_diag(s, c);
     }
-    // s / am[c][0] by the stored inverse and one correction of the quotient: three
-    // float64 operations where a division is a chain of some ten.  The bare
-    // product with the rounded inverse errs to the same side at every point of a
-    // code, which the smallest eigenvalue of A (about 1e-5 at 1023^2) turns into
-    // a relative error of 2e-12 in v.
+    // s / am[c][0].  The diagonal is exactly 1 but where both players take the
+    // same direction; there, the stored inverse and one correction of the
+    // quotient: three float64 operations where a division is a chain of some ten.
+    // The bare product with the rounded inverse errs to the same side at every
+    // such point, which the smallest eigenvalue of A (about 1e-5 at 1023^2) turns
+    // into a relative error of 2e-12 in v.
     __device__ __forceinline__ double over_diag(double s, int c) const {
+        if ((c >> 2) != (c & 3)) return s;   // (the stop code too)
         const double q = s * K->am0inv[c];
         return fma(fma(-K->am[c][0], q, s), K->am0inv[c], q);
     }
