@@ -108,7 +108,7 @@ typedef struct {
                               two grid-wide barriers per level and cycle; the finest level,
                               and coarse levels of side above 511 (255 in float64), keep one
                               phase per colour); 1 one grid-wide phase per
-                              relaxation colour.  Same arithmetic per point.  W-cycles always
+                              relaxation colour.  The same cycles up to rounding.  W-cycles always
                               take the latter. */
     int32_t game_solver;   /* policy evaluation of a single finite game (gamesolve_set_game):
                               0 (default) relaxation plus the constant-vector coarse

@@ -210,8 +210,8 @@ struct ImprovePoint {
 
 // Every thread walks points a grid apart and loads the next one while it works
 // on the current; counts and maxima are combined per block at its end.  Bound by
-// the float64 operations of the stored values in the outer mode (17 per point:
-// 29 us at 1023^2), by memory latency in the others.  One point per thread with
+// the float64 operations in the outer mode (17 for the stored values and 4
+// differences per point: 36 us at 1023^2), by memory latency in the others.  One point per thread with
 // a few atomics per warp on the scalars, and the screen below on the values, took
 // 117 us for the obstacle game at 1023^2 (48 us now).
 template <int MODE>

@@ -909,10 +909,7 @@ __global__ void __launch_bounds__(kMGThreads) k_mg_cycles(const __grid_constant_
 //    restriction into level l + 1 (with that level's first colour);
 //  - up, coarse level l: the prolongation from level l + 1 and every
 //    post-smoothing colour;
-//  - the finest level, one phase per cycle: prolongation, post-smoothing,
-//    the float64 update v += e (mixed path), the float64 residual of the
-//    stopping test, then the next cycle's pre-smoothing and restriction
-//    (discarded when the test stops the solve).
+// (the finest level keeps one phase per colour: fine.cuh in the mixed path).
 // Each colour update leaves the values it computed exact on a region one
 // point narrower on every side that faces another tile (a point's new value
 // needs its neighbours' current ones), so the halo is as deep as the updates

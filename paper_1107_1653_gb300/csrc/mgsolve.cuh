@@ -83,11 +83,11 @@ void launch_mg_cycles(const SolveArgs& a, cudaStream_t st);
 size_t tail_smem_bytes(const SolveArgs& a);
 
 // Largest dynamic shared memory a tiled cycle launch may take, and what one
-// needs (the tail's and the largest tile's, whichever is more).
+// needs (the tail's levels and the finest level's staging, or the largest tile's).
 constexpr int kTiledSmemMax = 220 * 1024;
 // Largest coarse level side the tiled kernel tiles: a 1023 x 1023 coarse level
 // (the 2047 x 2047 grid's first) measured faster one phase per colour; in
-// float64 (tiles of at most 8 x 8 next-level points: shared memory) already a
+// float64 (smaller tiles: shared memory) already a
 // 511 x 511 one (1023^2 float64 solve 19.8 -> 17.7 ms).
 constexpr int kTiledMaxSide = 511;
 constexpr int kTiledMaxSideF64 = 255;
