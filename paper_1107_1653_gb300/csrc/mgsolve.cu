@@ -1737,7 +1737,9 @@ void launch_mg_cycles(const SolveArgs& a, cudaStream_t st) {
         const size_t per_block = a.mixed ? 512 : 128;
         int nb = (int)std::min<size_t>((a.L[0].n + per_block - 1) / per_block, (size_t)o.sms);
         nb = std::min(std::max(nb, 1 + tiled_max_tiles(a)), o.sms);
-        if (a.L[0].side <= 31) nb = 1;
+        // small grids on one block, where its tail takes every coarse level: tiles
+        // need a second block, since block 0 takes none
+        if (a.L[0].side <= 31 && a.tail <= 1) nb = 1;
         if (a.max_blocks > 0) nb = std::min(nb, a.max_blocks);
         GS_CUDA(cudaLaunchCooperativeKernel(tiled_kernel(kind), dim3(nb), dim3(kTiledThreads), args, smem,
                                             st));

@@ -1,0 +1,39 @@
+"""Isaacs grids where a launch's shape could change a result: grids of side 31
+and below whose coarse levels are not all taken by one thread block (small
+tail_side).
+
+Linear solves are compared with the oracle's direct solve to a tenth of the
+path's value bar (as test_policy_solve_parity), whole solves to the bar.
+"""
+import numpy as np
+import pytest
+
+from test_gpu_isaacs import TOL, oracle_solve, rel_err
+from test_gpu_isaacs_paths import system
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("prec", ["fp64", "mixed", "mixed_bf16"])
+@pytest.mark.parametrize("sweeps", [(1, 1, -1, -1), (1, 2, 0, 1), (0, 2, 0, 2)])
+@pytest.mark.parametrize("tail_side", [1, 3, 7, 15])
+@pytest.mark.parametrize("side,variant", [(7, 0), (15, 1), (31, 0)])
+def test_small_grids_with_grid_wide_coarse_levels(gs, side, variant, tail_side, sweeps, prec):
+    alpha, beta, ref = system(side, variant)
+    nu1, nu2, c1, c2 = sweeps
+    with gs.GameSolver(precision=prec, tail_side=tail_side, nu1=nu1, nu2=nu2, nu1_coarse=c1, nu2_coarse=c2,
+                       coarse_max=1) as s:
+        s.set_isaacs_grid(side, variant, 3)
+        w, st = s.policy_solve(alpha, beta)
+    assert rel_err(w, ref) <= TOL[prec] / 10, st
+
+
+@pytest.mark.parametrize("prec", ["fp64", "mixed"])
+@pytest.mark.parametrize("tail_side", [3, 7])
+def test_fmg_through_small_grids_with_small_tail(gs, tail_side, prec):
+    _, ref = oracle_solve(63, 0, 7)
+    with gs.GameSolver(precision=prec, tail_side=tail_side, fmg=1, fmg_side=15) as s:
+        s.set_isaacs_grid(63, 0, 7)
+        st = s.solve()
+        v = s.get_value()
+    assert st["converged"] == 1 and rel_err(v, ref.v) <= TOL[prec], st
