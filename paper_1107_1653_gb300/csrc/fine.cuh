@@ -49,6 +49,7 @@ struct FineView {
     __device__ explicit FineView(const SolveArgs& a)
         : u((float*)a.L[0].u), f((float*)a.L[0].f), code(a.code), side(a.L[0].side), P(a.L[0].side + 1),
           lg(a.lg0) {}
+    __device__ __forceinline__ bool last(int q) const { return 8 * q + 8 == P; }   // the row's last octet
 };
 
 // Rows [r0, r1) of n of this block.
@@ -109,9 +110,12 @@ struct Octet {
         }
         return make_float4(r[0], r[1], r[2], r[3]);
     }
-    __device__ __forceinline__ void store(float* p) const {   // the eight values of u
+    // The eight values of u.  last: the row's last octet, whose eighth element lies
+    // outside the grid and stays zero whatever its neighbours hold: an iterate
+    // that is not finite must not reach the padding, which no launch clears.
+    __device__ __forceinline__ void store(float* p, bool last) const {
         ((float4*)p)[0] = make_float4(o[1], o[2], o[3], o[4]);
-        ((float4*)p)[1] = make_float4(o[5], o[6], o[7], o[8]);
+        ((float4*)p)[1] = make_float4(o[5], o[6], o[7], last ? 0.0f : o[8]);
     }
 };
 
@@ -133,16 +137,14 @@ __device__ __forceinline__ void for_octets(const FineView& V, int r0, int r1, F&
     }
 }
 
-// One colour of the red-black relaxation (colour 0: i + j even).  The last
-// element of a row, outside the grid, keeps its zero: its code is the stop code
-// and its f zero.
+// One colour of the red-black relaxation (colour 0: i + j even).
 __device__ __noinline__ void fine_relax_wide(const SolveArgs& a, const FineTab& T, int c) {
     const FineView V(a);
     int r0, r1;
     block_rows(V.side, &r0, &r1);
     for_octets(V, r0, r1, [&](int j, int q, Octet& O) {
         O.relax(T, (j + c) & 1);
-        O.store(V.u + (size_t)j * V.P + 8 * q);
+        O.store(V.u + (size_t)j * V.P + 8 * q, V.last(q));
     });
 }
 
@@ -159,8 +161,8 @@ __device__ __noinline__ void fine_update_wide(const SolveArgs& a, const FineTab&
         const int re = min(r1, r0 + chunk);
         for_octets(V, r0, re, [&](int j, int q, Octet& O) {
             O.relax(T, (j + c) & 1);
-            O.store(V.u + (size_t)j * V.P + 8 * q);
-            O.store(stage + ((j - r0) << V.lg) + 8 * q);
+            O.store(V.u + (size_t)j * V.P + 8 * q, V.last(q));
+            O.store(stage + ((j - r0) << V.lg) + 8 * q, V.last(q));
         });
         __syncthreads();
         constexpr int B = 4;

@@ -1,6 +1,7 @@
-"""Isaacs grids where a launch's shape could change a result: grids of side 31
-and below whose coarse levels are not all taken by one thread block (small
-tail_side).
+"""Isaacs grids where a launch's shape or a solver's history could change a
+result: grids of side 31 and below whose coarse levels are not all taken by one
+thread block (small tail_side), and calls on a solver after one that met
+values that are not finite.
 
 Linear solves are compared with the oracle's direct solve to a tenth of the
 path's value bar (as test_policy_solve_parity), whole solves to the bar.
@@ -37,3 +38,23 @@ def test_fmg_through_small_grids_with_small_tail(gs, tail_side, prec):
         st = s.solve()
         v = s.get_value()
     assert st["converged"] == 1 and rel_err(v, ref.v) <= TOL[prec], st
+
+
+@pytest.mark.parametrize("prec", ["fp64", "mixed", "mixed_bf16"])
+@pytest.mark.parametrize("bad", [np.nan, np.inf, 1e300])
+@pytest.mark.parametrize("side,variant", [(7, 0), (31, 1), (63, 0), (127, 0)])
+def test_good_call_after_one_that_was_not_finite(gs, side, variant, bad, prec):
+    """1e300 is finite, but its residual is not in float32."""
+    alpha, beta, ref = system(side, variant)
+    start = np.zeros(side * side)
+    start[[0, side - 1, side * side // 2, side * side - 1]] = bad
+    with gs.GameSolver(precision=prec, max_cycles=40) as s:
+        s.set_isaacs_grid(side, variant, 3)
+        w0, _ = s.policy_solve(alpha, beta)
+        s.policy_solve(alpha, beta, w0=start, allow_notconv=True)
+        w1, st = s.policy_solve(alpha, beta)
+        s.set_initial(v0=start)
+        s.solve(allow_notconv=True)
+        w2, _ = s.policy_solve(alpha, beta)
+    assert np.array_equal(w1, w0) and np.array_equal(w2, w0), st
+    assert rel_err(w0, ref) <= TOL[prec] / 10
