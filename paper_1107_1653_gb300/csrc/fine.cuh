@@ -16,6 +16,7 @@
 // 2047^2 solve 24.7 -> 22.0 ms.
 #pragma once
 
+#include "fine_stage.h"
 #include "mgsolve.cuh"
 #include "stencil.cuh"
 
@@ -27,9 +28,6 @@ struct FineTab {
     float4 w[kCodes];
     float dinv[kCodes], s[kCodes];
 };
-
-// Shared-memory staging of one phase: at most this many floats (64 KB).
-constexpr int kFineStage = 16384;
 
 // Whether the wide phases take a grid: rows of at least 8 elements.
 __host__ __device__ __forceinline__ bool fine_wide(int side) { return side >= 7; }
@@ -156,7 +154,7 @@ __device__ __noinline__ void fine_update_wide(const SolveArgs& a, const FineTab&
     double* __restrict__ v = a.v;
     int r0, r1;
     block_rows(V.side, &r0, &r1);
-    const int chunk = max(1, kFineStage >> V.lg);
+    const int chunk = fine_update_chunk(V.side);
     for (; r0 < r1; r0 += chunk) {
         const int re = min(r1, r0 + chunk);
         for_octets(V, r0, re, [&](int j, int q, Octet& O) {
@@ -253,7 +251,7 @@ __device__ __noinline__ void fine_restrict_wide(const SolveArgs& a, const FineTa
     float* __restrict__ uc = (float*)C.u;
     int J0, J1;
     block_rows(sc, &J0, &J1);
-    const int chunk = max(1, ((kFineStage >> lh) - 1) / 2);
+    const int chunk = fine_restrict_chunk(V.side);
     for (; J0 < J1; J0 += chunk) {
         const int Je = min(J1, J0 + chunk), j0 = 2 * J0, j1 = 2 * Je + 1;
         for_octets(V, j0, j1, [&](int j, int q, Octet& O) {

@@ -1326,7 +1326,7 @@ struct FinePhases {
     const SolveArgs& a;
     const IsaacsConsts* K;
     const FineTab& tab;
-    float* stage;            // kFineStage floats of dynamic shared memory
+    float* stage;            // fine_stage_floats(side) floats of dynamic shared memory
     size_t gt, gs;
     bool wide;
     __device__ void relax(int c, bool zero) const {
@@ -1656,7 +1656,7 @@ size_t tiled_smem_bytes(const SolveArgs& a) {
         return (size_t)std::min(sf, 2 * std::min(tc, sc) + 1 + 2 * H);
     };
     // the tail's levels, the finest level's staging, the largest tile
-    size_t need = (size_t)a.stage_at + (a.mixed ? kFineStage * sizeof(float) : 0);
+    size_t need = (size_t)a.stage_at + (a.mixed ? fine_stage_floats(a.L[0].side) * sizeof(float) : 0);
     for (int l = std::max(1, a.tile_from); l < a.tail; ++l) {
         const LevelArgs& L = a.L[l];
         const int K1 = a.nu1c > 0 ? 4 * a.nu1c - 1 : 0;

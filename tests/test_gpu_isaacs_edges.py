@@ -58,3 +58,26 @@ def test_good_call_after_one_that_was_not_finite(gs, side, variant, bad, prec):
         w2, _ = s.policy_solve(alpha, beta)
     assert np.array_equal(w1, w0) and np.array_equal(w2, w0), st
     assert rel_err(w0, ref) <= TOL[prec] / 10
+
+
+@pytest.mark.parametrize("side", [8191, 16383])
+def test_largest_grids_mixed_against_float64(gs, side):
+    """Sides whose rows fill the finest level's staging, and the largest accepted."""
+    import ctypes
+    import torch
+    n = side * side
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    alpha = torch.randint(0, 4, (n,), dtype=torch.uint8, device="cuda", generator=gen)
+    beta = torch.randint(0, 4, (n, 4), dtype=torch.uint8, device="cuda", generator=gen)
+    w = {}
+    for prec in ("fp64", "mixed", "mixed_bf16"):
+        w[prec] = torch.empty(n, dtype=torch.float64, device="cuda")
+        with gs.GameSolver(precision=prec, nu2=2) as s:
+            s.set_isaacs_grid(side, 0, 1)
+            st = gs.gs_solve_stats()
+            code = gs.gamesolve_policy_solve(s.h, alpha.data_ptr(), beta.data_ptr(), None, w[prec].data_ptr(),
+                                             ctypes.byref(st))
+        assert code == gs.GS_OK and st.converged == 1
+    scale = float(w["fp64"].abs().max())
+    for prec in ("mixed", "mixed_bf16"):
+        assert float((w[prec] - w["fp64"]).abs().max()) <= TOL[prec] * scale, prec
