@@ -357,6 +357,14 @@ gs_status gamesolve_get_level_stats(const gs_solver* s, int32_t* stats, int32_t 
 gs_status gamesolve_selftest_barrier(int32_t blocks, int32_t absent_block, uint64_t limit_ns,
                                      int32_t rounds, void* stream, int32_t* passed);
 
+/* Failure testing of a solver's multigrid launches (Isaacs grids, and games on
+ * options.game_solver 1): with on != 0 the barriers of its later cooperative
+ * launches start with their error flag raised, so that the first wait that is
+ * not over at once gives up, as after the time limit, and the call ends with
+ * GS_ETIMEOUT (launches of one thread block do not wait).  on = 0 ends it.
+ * Errors: GS_EINVAL (s is NULL). */
+gs_status gamesolve_selftest_give_up(gs_solver* s, int32_t on);
+
 /* Kernel classes that gamesolve_trace can time (diagnostics). */
 typedef enum {
     GS_K_NONE = 0,

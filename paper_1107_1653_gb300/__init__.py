@@ -112,6 +112,7 @@ _SIGS = {
     "gamesolve_get_level_stats": (_S, [_P, _P, ctypes.c_int32, ctypes.POINTER(ctypes.c_int32)]),
     "gamesolve_selftest_barrier": (_S, [ctypes.c_int32, ctypes.c_int32, ctypes.c_uint64,
                                         ctypes.c_int32, _P, ctypes.POINTER(ctypes.c_int32)]),
+    "gamesolve_selftest_give_up": (_S, [_P, ctypes.c_int32]),
     "gamesolve_trace": (_S, [_P, ctypes.c_int32]),
     "gamesolve_trace_read": (_S, [_P, ctypes.POINTER(ctypes.c_double), ctypes.POINTER(ctypes.c_int64)]),
     "gamesolve_kernel_launches": (ctypes.c_uint64, []),

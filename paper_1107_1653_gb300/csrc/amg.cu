@@ -305,11 +305,13 @@ __global__ void __launch_bounds__(kLoopThreads) k_colour(int n, int W, const int
 // The points of each smoother class (C or F, colour k) counted, the non-empty
 // classes listed (C colours, then F colours), the points listed by class (order
 // within a class is free: its points are mutually uncoupled).
+// A colouring whose barrier gave up leaves points without a colour (-1): they
+// belong to no class (the host reads the barrier's error after these launches).
 __device__ __forceinline__ int class_key(int8_t cf, int16_t colour) { return (cf == 1 ? 0 : kAmgMaxColours) + colour; }
 __global__ void k_class_count(int n, const int16_t* __restrict__ colour, const int8_t* __restrict__ cf,
                               int* __restrict__ cnt) {
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-        atomicAdd(&cnt[class_key(cf[i], colour[i])], 1);
+        if (colour[i] >= 0) atomicAdd(&cnt[class_key(cf[i], colour[i])], 1);
 }
 __global__ void k_class_list(int* __restrict__ cnt, AmgClasses* __restrict__ cls) {   // cnt becomes the cursors
     __shared__ int s_cnt[2 * kAmgMaxColours];
@@ -333,7 +335,7 @@ __global__ void k_class_list(int* __restrict__ cnt, AmgClasses* __restrict__ cls
 __global__ void k_class_scatter(int n, const int16_t* __restrict__ colour, const int8_t* __restrict__ cf,
                                 int* __restrict__ cursor, int* __restrict__ ord) {
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-        ord[atomicAdd(&cursor[class_key(cf[i], colour[i])], 1)] = i;
+        if (colour[i] >= 0) ord[atomicAdd(&cursor[class_key(cf[i], colour[i])], 1)] = i;
 }
 
 // Exclusive prefix sum of (state == C) in blocks of 1024, then over the blocks.
@@ -1201,8 +1203,9 @@ int loop_blocks(int n, int cap) {
 
 // The C/F splitting's rounds; clears the loop state first.
 void launch_pmis(int n, int W, const int* col, const unsigned long long* S, int8_t* state, const double* w,
-                 int* notmax, AmgLoop* loop, int max_blocks, cudaStream_t st) {
+                 int* notmax, AmgLoop* loop, int max_blocks, bool give_up, cudaStream_t st) {
     GS_CUDA(cudaMemsetAsync(loop, 0, sizeof(AmgLoop), st));
+    if (give_up) raise_error(&loop->bar, st);
     void* args[] = {&n, &W, &col, &S, &state, &w, &notmax, &loop};
     GS_CUDA(cudaLaunchCooperativeKernel((const void*)k_pmis, dim3(loop_blocks(n, max_blocks)), dim3(kLoopThreads),
                                         args, 0, st));
@@ -1299,7 +1302,7 @@ GamePI amgpi_game(gs_solver* s, Problem& P, double eps, bool warm) {
     double lin_res = 0.0, vmax = 0.0;
     auto evaluate = [&](double rel_tol) {
         if (!built) {
-            H.build(B.T, G.sel, mu, (int)n, W0, s->opt, st);
+            H.build(B.T, G.sel, mu, (int)n, W0, s->opt, s->give_up, st);
             built = true;
         }
         const int why = H.solve(G.v, G.rhs, s->opt, rel_tol, &mgd->bar, dout, &hout, &R.cycles, &lin_res,
@@ -1620,7 +1623,7 @@ gs_status run_game_fmg(gs_solver* s, gs_solve_stats* stats) {
         k_pmis_init<<<g, 256, 0, st>>>((int)n, S, lam, cf, w);
         GS_CHECK_LAUNCH_N(3);
         AmgLoop* loop = tmp.alloc<AmgLoop>(1);
-        launch_pmis((int)n, W, col, S, cf, w, flag, loop, s->opt.grid_blocks, st);
+        launch_pmis((int)n, W, col, S, cf, w, flag, loop, s->opt.grid_blocks, s->give_up, st);
         k_rs_second<<<g, 256, 0, st>>>((int)n, W, col, S, cf, flag);
         k_rs_apply<<<g, 256, 0, st>>>((int)n, cf, flag);
         k_promote_lonely<<<g, 256, 0, st>>>((int)n, W, col, S, cf);
@@ -1734,7 +1737,7 @@ gs_status run_game_fmg(gs_solver* s, gs_solve_stats* stats) {
 }
 
 void AmgHierarchy::build(const GameTables& T, const int64_t* sel, double mu, int n, int W0,
-                         const gs_options& opt, cudaStream_t st) {
+                         const gs_options& opt, bool give_up, cudaStream_t st) {
     const bool mixed = opt.precision != GS_PREC_FP64;
     const size_t tb = mixed ? sizeof(float) : sizeof(double);
     ar = std::make_unique<Arena>(0, 0, st);
@@ -1780,7 +1783,7 @@ void AmgHierarchy::build(const GameTables& T, const int64_t* sel, double mu, int
         k_pmis_init<<<grid(nf), 256, 0, st>>>(nf, S, lam, F.cf, w);
         GS_CHECK_LAUNCH_N(2);
         AmgLoop* loop = ar->alloc<AmgLoop>(1);
-        launch_pmis(nf, F.W, F.col, S, F.cf, w, flag, loop, opt.grid_blocks, st);
+        launch_pmis(nf, F.W, F.col, S, F.cf, w, flag, loop, opt.grid_blocks, give_up, st);
         if (opt.amg_coarsening == 1) {
             k_rs_second<<<grid(nf), 256, 0, st>>>(nf, F.W, F.col, S, F.cf, flag);
             k_rs_apply<<<grid(nf), 256, 0, st>>>(nf, F.cf, flag);

@@ -120,8 +120,9 @@ struct AmgHierarchy {
     AmgHierarchy();
     ~AmgHierarchy();
     // Set-up for the rows sel[0..n) of the tables (W0 >= 1 + the longest row).
+    // give_up: the loops' barriers start with their error raised (failure tests).
     void build(const GameTables& T, const int64_t* sel, double mu, int n, int W0,
-               const gs_options& opt, cudaStream_t st);
+               const gs_options& opt, bool give_up, cudaStream_t st);
     // V-cycles on A v = rhs from v until the float64 floor, rel_tol drop or
     // max_cycles; returns the stop reason (1 floor/tolerance, 2 drop, 3 cap).
     int solve(double* v, const double* rhs, const gs_options& opt, double rel_tol,

@@ -14,6 +14,12 @@ struct GridBarrier {
     int pad;
 };
 
+// Failure tests: raises a cleared barrier's error before the launch that uses it,
+// so that a wait which is not over at once gives up, as after the time limit.
+inline void raise_error(GridBarrier* b, cudaStream_t st) {
+    GS_CUDA(cudaMemsetAsync(&b->error, 1, sizeof b->error, st));
+}
+
 constexpr unsigned long long kBarrierTimeoutNs = 2000000000ull;   // 2 s
 
 __device__ __forceinline__ unsigned long long global_ns() {

@@ -7,6 +7,7 @@
 #include <algorithm>
 
 #include "gridsync.cuh"
+#include "solver.cuh"
 
 namespace gs {
 
@@ -87,4 +88,10 @@ extern "C" gs_status gamesolve_selftest_barrier(int32_t blocks, int32_t absent_b
     } catch (const gs::Error& e) {
         return e.st;
     }
+}
+
+extern "C" gs_status gamesolve_selftest_give_up(gs_solver* s, int32_t on) {
+    if (!s) return GS_EINVAL;
+    s->give_up = on != 0;
+    return GS_OK;
 }

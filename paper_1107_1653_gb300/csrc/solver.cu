@@ -449,6 +449,7 @@ int linear_solve(gs_solver* s, IsaacsGrid& g, Counters& cnt, double rel_tol, boo
     while (a.smem_from < a.nlev && tail_smem_bytes(a) > (size_t)kTailSmemMax)
         ++a.smem_from;
     GS_CUDA(cudaMemsetAsync(s->mgd, 0, sizeof(MGState), s->st));
+    if (s->give_up) raise_error(&s->mgd->bar, s->st);
     if (improve) {
         clear_scalars(s);
         a.vmax_out = &s->dsc->vmax;   // the improvement's keep-current tolerance

@@ -180,6 +180,7 @@ struct gs_solver {
     std::unique_ptr<gs::Problem> prob;
     bool init_v = false, init_alpha = false, init_beta = false;
     int last_levels = 0;
+    bool give_up = false;              // failure tests: barriers start with their error raised
     std::vector<int> level_stats;      // per FAMGpi level of the last solve: side, outer, systems
 };
 
