@@ -1,7 +1,7 @@
 // Launchers of the CUDA kernels (host-callable; all asynchronous on `st`).
 #pragma once
 
-#include "common.cuh"
+#include "mgsolve.cuh"
 
 namespace gs {
 
@@ -42,8 +42,10 @@ struct ImproveArgs {
     const uint8_t* beta4;
     DevScalars* sc;
     double tau;
-    const int* skip;   // where *skip is skip_if, nothing is done (null: never)
-    int skip_if;
+    // With both given, nothing is done unless the linear solve they belong to
+    // ended at its floor or its drop (null: always).
+    const SolveOut* solved;
+    const GridBarrier* solve_bar;
 };
 void launch_isaacs_improve(ImproveMode mode, const ImproveArgs& a, cudaStream_t st);
 

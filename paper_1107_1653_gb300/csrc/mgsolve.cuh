@@ -32,12 +32,15 @@ struct LevelArgs {
     void* u2;            // tiled cycles: u after the post-smoothing (levels >= 1)
 };
 
+// Why a solve stopped (SolveOut::reason; 0 until then): tolerance or float64
+// floor, relative drop, cycle cap.
+enum { kLinExact = 1, kLinInexact = 2, kLinCapped = 3 };
 
 struct SolveOut {
     unsigned long long rmax[2];   // |b - A v|_inf per residual evaluation (bits), ping-pong
     unsigned long long vmax[2];   // |v|_inf (bits)
     int cycles;
-    int reason;                   // 1 tolerance or float64 floor, 2 relative drop, 3 cycle cap
+    int reason;
     double res;                   // final |b - A v|_inf
     double vmax_final;            // |v|_inf at the final residual evaluation
 };

@@ -354,7 +354,7 @@ int tail_level(const gs_solver* s, const IsaacsGrid& g) {
 // Improvement arguments on the grid's own arrays.
 ImproveArgs improve_args(gs_solver* s, IsaacsGrid& g, double* fv, double tau) {
     return {g.Kd,   g.side, g.variant, g.v, g.r0,    g.alpha, g.beta, g.alpha,
-            g.beta, g.code, g.rhs,     fv,  nullptr, g.beta4, s->dsc, tau, nullptr, 0};
+            g.beta, g.code, g.rhs,     fv,  nullptr, g.beta4, s->dsc, tau, nullptr, nullptr};
 }
 
 // Solves (I - mu M) v = r for the assembled codes/rhs of g, warm-started from
@@ -367,8 +367,8 @@ ImproveArgs improve_args(gs_solver* s, IsaacsGrid& g, double* fv, double tau) {
 // stopped: kLinExact (float64 floor or tolerance), kLinInexact (the residual
 // fell by rel_tol) or kLinCapped (max_cycles reached short of both).
 // With `improve` MIN's replies at the solution are improved in the same go (one
-// read-back for both; not done where the solve was capped): the changed entries
-// are then in s->hsc.
+// read-back for both; not done where the solve was capped or a wait gave up): the
+// changed entries are then in s->hsc.
 int linear_solve(gs_solver* s, IsaacsGrid& g, Counters& cnt, double rel_tol, bool do_setup, bool improve = false) {
     const bool mixed = s->opt.precision != GS_PREC_FP64;
     SolveArgs a{};
@@ -465,8 +465,8 @@ int linear_solve(gs_solver* s, IsaacsGrid& g, Counters& cnt, double rel_tol, boo
     if (improve) {
         KScope ks(s, GS_K_IMPROVE);
         ImproveArgs A = improve_args(s, g, nullptr, -1.0);
-        A.skip = &s->mgd->out.reason;
-        A.skip_if = kLinCapped;
+        A.solved = &s->mgd->out;
+        A.solve_bar = &s->mgd->bar;
         launch_isaacs_improve(IMP_INNER, A, s->st);
     }
     GS_CUDA(cudaMemcpyAsync(s->mgh, s->mgd, sizeof(MGState), cudaMemcpyDeviceToHost, s->st));
@@ -706,7 +706,7 @@ gs_status run_improve(gs_solver* s, const double* v, uint8_t* alpha_out, uint8_t
     launch_absmax(vd, n, &s->dsc->vmax, s->st);
     const ImproveArgs A{g.Kd, g.side, g.variant, vd, g.r0, g.alpha, g.beta, a,
                         m1 == 4 ? reinterpret_cast<uint32_t*>(b) : nullptr, nullptr, nullptr, fv,
-                        m1 == 5 ? b : nullptr, g.beta4, s->dsc, -1.0, nullptr, 0};
+                        m1 == 5 ? b : nullptr, g.beta4, s->dsc, -1.0, nullptr, nullptr};
     launch_isaacs_improve(IMP_OUTER, A, s->st);
     if (a && !da) GS_CUDA(cudaMemcpyAsync(alpha_out, a, n, cudaMemcpyDefault, s->st));
     if (fv && !df) GS_CUDA(cudaMemcpyAsync(fv_out, fv, nv, cudaMemcpyDefault, s->st));

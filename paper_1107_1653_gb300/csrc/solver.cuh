@@ -147,9 +147,6 @@ struct Counters {
     double last_lin_res = 0;
 };
 
-// Why a multigrid linear solve stopped (SolveOut::reason).
-enum { kLinExact = 1, kLinInexact = 2, kLinCapped = 3 };
-
 }  // namespace gs
 
 namespace gs {
