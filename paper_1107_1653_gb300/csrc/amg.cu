@@ -32,6 +32,7 @@
 #include <cstring>
 
 #include "amg.cuh"
+#include "device_once.h"
 #include "gridsync.cuh"
 #include "solver.cuh"
 
@@ -1191,12 +1192,22 @@ __global__ void k_game_assemble(int64_t n, int m1, int m2, const uint8_t* __rest
     }
 }
 
+// SMs of the current device, with the dynamic shared memory of this file's kernels allowed.
+int amg_device_sms() {
+    static PerDevice<int> sms;
+    const int dev = current_device();
+    return sms.get(dev, [&] {
+        const auto allow = cudaFuncAttributeMaxDynamicSharedMemorySize;
+        GS_CUDA(cudaFuncSetAttribute(k_amg_cycles<float>, allow, kAmgSmemMax));
+        GS_CUDA(cudaFuncSetAttribute(k_amg_cycles<double>, allow, kAmgSmemMax));
+        GS_CUDA(cudaFuncSetAttribute(k_amg_coarse_inv, allow, (int)(2 * kAmgInvSmem * kAmgInvSmem * sizeof(double))));
+        return sm_count(dev);
+    });
+}
+
 // Blocks of the set-up's cooperative loops.
 int loop_blocks(int n, int cap) {
-    int dev = 0, sms = 0;
-    GS_CUDA(cudaGetDevice(&dev));
-    GS_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    int nb = std::min(sms, (n + kLoopThreads - 1) / kLoopThreads);
+    int nb = std::min(amg_device_sms(), (n + kLoopThreads - 1) / kLoopThreads);
     if (cap > 0) nb = std::min(nb, cap);
     return std::max(1, nb);
 }
@@ -1862,12 +1873,7 @@ void AmgHierarchy::build(const GameTables& T, const int64_t* sel, double mu, int
     }
     inv = ar->alloc<double>((size_t)Lc.n * Lc.n);
     GS_CUDA(cudaMemsetAsync(scal, 0, sizeof(int) * 8, st));
-    static bool attr = false;
-    if (!attr) {
-        GS_CUDA(cudaFuncSetAttribute(k_amg_coarse_inv, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)(2 * kAmgInvSmem * kAmgInvSmem * sizeof(double))));
-        attr = true;
-    }
+    amg_device_sms();
     const bool in_smem = Lc.n <= kAmgInvSmem;
     double* gm = in_smem ? nullptr : ar->alloc<double>(2 * (size_t)Lc.n * Lc.n);
     k_amg_coarse_inv<<<1, in_smem ? 256 : 1024, in_smem ? 2 * (size_t)Lc.n * Lc.n * sizeof(double) : 0, st>>>(
@@ -1965,15 +1971,7 @@ int AmgHierarchy::solve(double* v, const double* rhs, const gs_options& opt, dou
     a.bar = bar_state;
     a.out = dout;
     for (int l = 0; l < a.nlev; ++l) a.L[l] = args_of(lv[l]);
-    static int sms = 0;
-    if (!sms) {
-        int dev = 0;
-        GS_CUDA(cudaGetDevice(&dev));
-        GS_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-        GS_CUDA(cudaFuncSetAttribute(k_amg_cycles<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAmgSmemMax));
-        GS_CUDA(cudaFuncSetAttribute(k_amg_cycles<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAmgSmemMax));
-    }
-    int nb = (int)std::min<size_t>((size_t)sms, ((size_t)lv[0].n + 127) / 128);
+    int nb = (int)std::min<size_t>((size_t)amg_device_sms(), ((size_t)lv[0].n + 127) / 128);
     if (opt.grid_blocks > 0) nb = std::min(nb, opt.grid_blocks);
     if (a.tail == 0) nb = 1;   // the whole hierarchy is small
     nb = std::max(1, nb);

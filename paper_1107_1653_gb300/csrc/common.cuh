@@ -174,6 +174,18 @@ __device__ __forceinline__ double f32_to_f64(float v) {
 // Largest Isaacs grid side: keeps every level index below 2^28 (FastDiv).
 constexpr int kIsaacsMaxSide = 16383;
 
+// The device the calling thread works on, and its SMs.
+inline int current_device() {
+    int dev = 0;
+    GS_CUDA(cudaGetDevice(&dev));
+    return dev;
+}
+inline int sm_count(int device) {
+    int sms = 0;
+    GS_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device));
+    return sms;
+}
+
 inline double bits_to_double(unsigned long long b) {
     double d;
     static_assert(sizeof(d) == sizeof(b), "");

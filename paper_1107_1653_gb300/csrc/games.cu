@@ -12,8 +12,8 @@
 // exactly; the other modes contract at the rate of M's second eigenvalue.
 #include <algorithm>
 #include <cfloat>
-#include <mutex>
 
+#include "device_once.h"
 #include "games.cuh"
 #include "gridsync.cuh"
 
@@ -1427,30 +1427,27 @@ void launch_game_prepare(const GameTables& T, int count, const int64_t* st_off, 
 }
 
 int game_grid_blocks(int64_t n, int cap) {
-    static int per_sm = 0, sms = 0;
-    if (!per_sm) {
-        int dev = 0;
-        GS_CUDA(cudaGetDevice(&dev));
-        GS_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    static PerDevice<int64_t> resident;
+    const int dev = current_device();
+    const int64_t all = resident.get(dev, [&] {
         int a = 0, b = 0;
         GS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, k_game_pi_grid<float>, kThreads, 0));
         GS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_game_pi_grid<double>, kThreads, 0));
-        per_sm = std::max(1, std::min(a, b));
-    }
+        return (int64_t)std::max(1, std::min(a, b)) * sm_count(dev);
+    });
     // one warp of states per block until every SM has one
-    int blocks = (int)std::min<int64_t>((n + 31) / 32, (int64_t)per_sm * sms);
+    int blocks = (int)std::min<int64_t>((n + 31) / 32, all);
     if (cap > 0) blocks = std::min(blocks, cap);
     return std::max(1, blocks);
 }
 
-// Whether one cluster of the cluster kernel fits the GPU (per precision, once).
+// Shared memory a block of the one-block kernel may take, and an SM's blocks together.
+constexpr size_t kSmemPerSM = 224 * 1024;
+
+// Whether one cluster of the cluster kernel fits the current device.
 static bool cluster_fits(const void* fn, bool mixed) {
-    static int fits[2] = {-1, -1};
-    static std::mutex mu;
-    std::lock_guard<std::mutex> lk(mu);
-    int& f = fits[mixed ? 1 : 0];
-    if (f < 0) {
-        f = 0;
+    static PerDevice<bool> fits[2];
+    return fits[mixed ? 1 : 0].get(current_device(), [&] {
         cudaLaunchConfig_t cfg{};
         cudaLaunchAttribute at{};
         at.id = cudaLaunchAttributeClusterDimension;
@@ -1461,12 +1458,11 @@ static bool cluster_fits(const void* fn, bool mixed) {
         cfg.attrs = &at;
         cfg.numAttrs = 1;
         int count = 0;
-        if (cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
-            cudaOccupancyMaxActiveClusters(&count, fn, &cfg) == cudaSuccess && count > 0)
-            f = 1;
+        const bool ok = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+                        cudaOccupancyMaxActiveClusters(&count, fn, &cfg) == cudaSuccess && count > 0;
         cudaGetLastError();
-    }
-    return f == 1;
+        return ok;
+    });
 }
 
 void launch_game_pi_grid(const BatchArgs& B, const GridWork& W, int blocks, bool mixed,
@@ -1503,7 +1499,6 @@ size_t games_smem_bytes(int max_n, bool mixed, bool v_in_smem) {
 void launch_games_pi(const BatchArgs& Bin, bool mixed, int threads, cudaStream_t st) {
     // the iterate joins the correction vectors in shared memory where all
     // 512 / threads blocks of an SM still fit
-    constexpr size_t kSmemPerSM = 224 * 1024;
     BatchArgs B = Bin;
     B.v_in_smem = games_smem_bytes(B.max_n, mixed, true) * (512 / threads) <= kSmemPerSM;
     const size_t smem = games_smem_bytes(B.max_n, mixed, B.v_in_smem);
@@ -1512,10 +1507,14 @@ void launch_games_pi(const BatchArgs& Bin, bool mixed, int threads, cudaStream_t
                                     : (mixed ? (const void*)k_games_pi<float, 512>
                                              : (const void*)k_games_pi<double, 512>);
     const int nt = threads == 256 ? 256 : 512;
-    GS_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    int per_sm = 0, dev = 0, sms = 0;
-    GS_CUDA(cudaGetDevice(&dev));
-    GS_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    static PerDevice<int> sms_of[4];
+    const int dev = current_device();
+    // (the limit, not this launch's size: another thread's launch may be between the two)
+    const int sms = sms_of[(threads == 256) * 2 + mixed].get(dev, [&] {
+        GS_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemPerSM));
+        return sm_count(dev);
+    });
+    int per_sm = 0;
     GS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, nt, smem));
     const int blocks = std::max(1, std::min(B.count, std::max(1, per_sm) * sms));
     void* args[] = {(void*)&B};

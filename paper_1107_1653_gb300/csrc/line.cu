@@ -14,6 +14,7 @@
 #include <cstdint>
 
 #include "common.cuh"
+#include "device_once.h"
 #include "line.cuh"
 
 namespace gs {
@@ -515,7 +516,12 @@ size_t line_smem_bytes(int n) {
 
 void launch_line_pi(const LineArgs& A, cudaStream_t st) {
     const size_t smem = line_smem_bytes(A.n);
-    GS_CUDA(cudaFuncSetAttribute(k_line_pi, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    static PerDevice<bool> allowed;
+    allowed.get(current_device(), [] {
+        GS_CUDA(cudaFuncSetAttribute(k_line_pi, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)line_smem_bytes(kLineMaxStates)));
+        return true;
+    });
     k_line_pi<<<1, kLineThreads, smem, st>>>(A);
     GS_CHECK_LAUNCH();
 }

@@ -6,8 +6,8 @@
 // gives up sets an error flag and the kernels return.
 #include <algorithm>
 #include <cmath>
-#include <mutex>
 
+#include "device_once.h"
 #include "gridsync.cuh"
 #include "mgsolve.cuh"
 #include "fine.cuh"
@@ -1595,14 +1595,13 @@ const void* tiled_kernel(int kind) {
                        : (const void*)k_mg_cycles_tiled<float, float>;
 }
 
-Occupancy& occupancy() {
-    static Occupancy o;
-    static std::mutex mu;
-    std::lock_guard<std::mutex> lk(mu);
-    if (!o.sms) {
-        int dev = 0;
-        GS_CUDA(cudaGetDevice(&dev));
-        GS_CUDA(cudaDeviceGetAttribute(&o.sms, cudaDevAttrMultiProcessorCount, dev));
+// Of the current device, with the kernels' dynamic shared memory allowed on it.
+const Occupancy& occupancy() {
+    static PerDevice<Occupancy> all;
+    const int dev = current_device();
+    return all.get(dev, [&] {
+        Occupancy o;
+        o.sms = sm_count(dev);
         const int big = kTailSmemMax;
         GS_CUDA(cudaFuncSetAttribute(k_mg_setup, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      64 * 128 * 8));
@@ -1625,8 +1624,8 @@ Occupancy& occupancy() {
             &o.cyc_per_sm[2], k_mg_cycles<float, __nv_bfloat16>, kMGThreads, big));
         o.setup_per_sm = o.setup_per_sm < 1 ? 1 : o.setup_per_sm;
         for (int& c : o.cyc_per_sm) c = c < 1 ? 1 : c;
-    }
-    return o;
+        return o;
+    });
 }
 
 int grid_blocks(const SolveArgs& a, int per_sm, int sms) {
