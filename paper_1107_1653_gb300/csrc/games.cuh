@@ -148,6 +148,14 @@ constexpr int64_t kGameGridMinStates = 512;
 // one block each, and must give the bits they give alone (GridCtx::sum).
 constexpr int64_t kGameBatchedStates = 4096;
 
+// Whether a game set alone takes a cluster or the whole grid.  Both sum like one
+// block of 512 threads: a caller's choice of 256 keeps games that a server may
+// batch on one block of 256 (3001 states, mixed: 6.3 ms, a cluster 1.9 ms), so
+// that they give the same bits alone and in a batch.
+inline bool game_takes_grid(int64_t n, int game_threads) {
+    return n >= kGameGridMinStates && (n >= kGameBatchedStates || game_threads != 256);
+}
+
 // Random games drawn on the device (randgame.cu): n states, m1 x m2 rows per
 // state, k <= 8 successors per row; CSR table into device buffers of
 // n*m1*m2 + 1, n*m1*m2*k, n*m1*m2*k and n*m1*m2 entries, row_ptr offset by

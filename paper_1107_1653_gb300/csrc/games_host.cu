@@ -36,7 +36,7 @@ std::unique_ptr<Problem> build_game_problem(gs_solver* s, int count, int m1, int
     }
     const bool mixed = s->opt.precision != GS_PREC_FP64;
     const int64_t cap = mixed ? kGameMaxStatesMixed : kGameMaxStatesFP64;
-    const bool grid = count == 1 && max_n >= kGameGridMinStates;
+    const bool grid = count == 1 && game_takes_grid(max_n, s->opt.game_threads);
     if (!grid && max_n > cap) {
         set_last_error("set_game: a game has %lld states; this build takes at most %lld per game",
                        (long long)max_n, (long long)cap);

@@ -1,0 +1,40 @@
+"""Finite games below 4096 states with the block shape chosen by the caller: the
+same bits alone and in a batch, on a solver and on a server whatever waits
+together."""
+import numpy as np
+import pytest
+
+import synth
+from test_gpu_games import batch
+from test_gpu_game_paths import solve
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("prec", ["fp64", "mixed"])
+@pytest.mark.parametrize("threads", [256, 512])
+def test_alone_equals_batch_bits_by_shape(gs, threads, prec):
+    sizes = np.array([31, 511, 512, 513, 1025, 3001, 4095])
+    (off, rp, col, prob, rew, mu), parts = batch(sizes, 23)
+    with gs.GameSolver(precision=prec, game_threads=threads) as s:
+        s.set_game_batch(off, 4, 4, rp, col, prob, rew, mu)
+        assert s.solve()["converged"] == 1
+        v = s.get_value()
+        a, b = s.get_policy()
+    for g, n in enumerate(sizes):
+        x0, x1 = off[g], off[g + 1]
+        w, c, d, _ = solve(gs, int(n), 4, 4, parts[g], prec, game_threads=threads)
+        assert np.array_equal(w, v[x0:x1]) and np.array_equal(c, a[x0:x1]) and np.array_equal(d, b[x0:x1]), n
+
+
+@pytest.mark.parametrize("threads", [0, 256, 512])
+def test_server_results_do_not_depend_on_the_queue(gs, threads):
+    sizes = [600, 3001, 900, 4095, 513]
+    tables = [synth.random_game(n, 60 + n) for n in sizes]
+    alone = [solve(gs, n, 4, 4, t, "mixed", game_threads=threads)[0] for n, t in zip(sizes, tables)]
+    with gs.GameServer(slots=1, precision="mixed", game_threads=threads) as srv:
+        # the first request occupies the slot while the others queue up
+        tickets = [srv.submit_isaacs(255, 0, 1)] + [srv.submit_game(n, 4, 4, *t) for n, t in zip(sizes, tables)]
+        got = [srv.result(t)[0] for t in tickets if srv.wait(t)]
+    for n, v, w in zip(sizes, got[1:], alone):
+        assert np.array_equal(v, w), n
