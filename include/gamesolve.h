@@ -248,7 +248,9 @@ gs_status gamesolve_set_stopping_line(gs_solver* s, int32_t n, const double* c,
 gs_status gamesolve_get_batch_stats(const gs_solver* s, int32_t* stats, double* res);
 
 /* Threads per game the last solve of a game batch ran with (256 or 512; 0 for
- * a single large game run on the whole grid).  Games are taken largest first.
+ * a single game of at least 4096 states, run on the whole grid; 512 for a
+ * smaller one that ran on several blocks, whose sums are those of one block of
+ * 512).  Games are taken largest first.
  * Errors: GS_EINVAL (NULL argument), GS_ESTATE when no solved batch is held. */
 gs_status gamesolve_get_batch_shape(const gs_solver* s, int32_t* threads);
 

@@ -249,7 +249,8 @@ gs_status run_games(gs_solver* s, gs_solve_stats* stats) {
     B.order = G.order;
     B.cp = G.cp;
     const int shape = G.grid ? 0 : tuned_shape(s, G, B, mixed);
-    G.shape = shape;
+    // a game of a batch's size on a cluster or the grid sums like one block of 512
+    G.shape = G.grid && G.n_total < kGameBatchedStates ? 512 : shape;
     cudaEvent_t e0, e1;
     GS_CUDA(cudaEventCreate(&e0));
     GS_CUDA(cudaEventCreate(&e1));

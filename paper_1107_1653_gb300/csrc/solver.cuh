@@ -101,7 +101,7 @@ struct GameProblem {
     int* order = nullptr;                  // games largest first (the queue's order)
     int* sample = nullptr;                 // every k-th entry of order (shape autotuning)
     int n_sample = 0;
-    int shape = 0;                         // threads per game of the last solve (0: grid)
+    int shape = 0;                         // gamesolve_get_batch_shape of the last solve
     bool grid = false;                     // one large game on the whole grid
     double *wr = nullptr, *we = nullptr, *wt = nullptr, *part = nullptr;
     GridScal* gscal = nullptr;

@@ -38,3 +38,12 @@ def test_server_results_do_not_depend_on_the_queue(gs, threads):
         got = [srv.result(t)[0] for t in tickets if srv.wait(t)]
     for n, v, w in zip(sizes, got[1:], alone):
         assert np.array_equal(v, w), n
+
+
+@pytest.mark.parametrize("threads", [0, 256, 512])
+@pytest.mark.parametrize("n", [300, 512, 4095, 4096])
+def test_reported_shape_of_a_single_game(gs, n, threads):
+    with gs.GameSolver(precision="mixed", game_threads=threads) as s:
+        s.set_random_game(n, 4, 4, 3, 0.95)
+        s.solve()
+        assert s.batch_shape() == (0 if n >= 4096 else threads or 512)
