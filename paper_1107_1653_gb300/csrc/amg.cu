@@ -35,6 +35,7 @@
 #include "device_once.h"
 #include "gridsync.cuh"
 #include "solver.cuh"
+#include "weight_order.h"
 
 namespace gs {
 
@@ -531,7 +532,7 @@ __global__ void __launch_bounds__(32 * kInterpWarps) k_interp(
         // rank of each candidate; the first kPMax are kept, in that order
         for (int q = lane; q < m; q += 32) {
             int rank = 0;
-            for (int t = 0; t < m; ++t) rank += w[t] > w[q] || (w[t] == w[q] && t < q);
+            for (int t = 0; t < m; ++t) rank += weight_before(w[t], t, w[q], q);
             if (rank < kPMax) {
                 pc[rank] = cidx[key[q]];
                 pv[rank] = w[q];
