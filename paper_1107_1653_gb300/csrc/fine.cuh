@@ -23,7 +23,8 @@
 namespace gs {
 
 // Weights of one policy code: w = minus the couplings (W, E, S, N), the inverse
-// diagonal and the row sum.
+// diagonal (rounded once from its float64 value; the residual these corrections
+// answer is formed in float64 with the exact rows) and the row sum.
 struct FineTab {
     float4 w[kCodes];
     float dinv[kCodes], s[kCodes];

@@ -8,8 +8,10 @@
 //  - u: planes of (M + 2)^2 with a border of zeros, so that a colour's eight
 //    neighbours are eight fixed offsets into the other planes and no point
 //    needs a bounds test;
-//  - the operator: per colour the eight couplings, the inverse diagonal, and the
-//    row sum (float32) or the diagonal (float64);
+//  - the operator: per colour the eight couplings, the inverse diagonal (its
+//    rounding is one of the relaxation's weight: the tail computes a correction,
+//    whose residual the finest level forms anew), and the row sum (float32) or the
+//    diagonal (float64);
 //    points outside the grid (the last row and column of cells) have zero
 //    couplings and a zero inverse, and stay zero.
 // A cell's operator, weights, f and residuals are one record (57 numbers, an odd
