@@ -422,8 +422,9 @@ gs_status gamesolve_isaacs_policy_solve_static(int32_t side, int32_t variant, ui
 /* ---------------------------------------------------------------- serving
  * A request loop around the solvers: requests are queued in arrival order and
  * admitted to worker slots as slots and device memory free up.  Each slot has
- * its own CUDA stream and solver, its grid-wide launches capped to a share of
- * the GPU, so the work of the requests in flight overlaps on the device.
+ * its own CUDA stream and solver; with several requests in flight its
+ * grid-wide launches are capped to a share of the GPU, so that their work
+ * overlaps on the device.
  * Games of fewer than 4096 states (those a solver runs one thread block per
  * game) that wait together with the same kind and action counts are taken by
  * one slot as a batch of up to 256 and solved by one persistent launch
@@ -465,10 +466,10 @@ typedef struct {
 
 /* Starts `slots` worker threads on the current device, each creating a solver
  * with `opt` (NULL = defaults) on its own stream.  Unless opt->grid_blocks is
- * set, a slot's grid-wide launches are capped at 2 x (SMs) / slots blocks; on
- * a mixed stream of Isaacs grids and large games 2 slots served the most
- * requests per second (whole-GPU launches, one request's host steps hidden
- * behind the other's kernels).  mem_budget: device bytes the
+ * set, a slot's multigrid launches (Isaacs grids, tables on game_solver 1) take
+ * the whole GPU while no other request is running or waiting and (SMs) / slots
+ * blocks otherwise, and the launch of a game of at least 4096 states takes 2 x
+ * (SMs) / slots blocks at any time.  mem_budget: device bytes the
  * requests in flight may hold together (0 = half the free memory); a request
  * larger than the budget runs when nothing else is in flight.
  * Errors: GS_EINVAL (slots outside [1, 64] or bad options), GS_ECUDA. */

@@ -1313,11 +1313,13 @@ GamePI amgpi_game(gs_solver* s, Problem& P, double eps, bool warm) {
     bool capped = false, built = false;
     double lin_res = 0.0, vmax = 0.0;
     auto evaluate = [&](double rel_tol) {
+        gs_options o = s->opt;
+        o.grid_blocks = multigrid_blocks(s);
         if (!built) {
-            H.build(B.T, G.sel, mu, (int)n, W0, s->opt, s->give_up, st);
+            H.build(B.T, G.sel, mu, (int)n, W0, o, s->give_up, st);
             built = true;
         }
-        const int why = H.solve(G.v, G.rhs, s->opt, rel_tol, &mgd->bar, dout, &hout, &R.cycles, &lin_res,
+        const int why = H.solve(G.v, G.rhs, o, rel_tol, &mgd->bar, dout, &hout, &R.cycles, &lin_res,
                                 &vmax, st);
         sync_v32();
         absmax_v();
@@ -1635,7 +1637,7 @@ gs_status run_game_fmg(gs_solver* s, gs_solve_stats* stats) {
         k_pmis_init<<<g, 256, 0, st>>>((int)n, S, lam, cf, w);
         GS_CHECK_LAUNCH_N(3);
         AmgLoop* loop = tmp.alloc<AmgLoop>(1);
-        launch_pmis((int)n, W, col, S, cf, w, flag, loop, s->opt.grid_blocks, s->give_up, st);
+        launch_pmis((int)n, W, col, S, cf, w, flag, loop, multigrid_blocks(s), s->give_up, st);
         k_rs_second<<<g, 256, 0, st>>>((int)n, W, col, S, cf, flag);
         k_rs_apply<<<g, 256, 0, st>>>((int)n, cf, flag);
         k_promote_lonely<<<g, 256, 0, st>>>((int)n, W, col, S, cf);

@@ -2,13 +2,14 @@
 // finite games given as tables, random games given by a seed) are queued in
 // arrival order and admitted to worker slots as slots and device memory free
 // up; every slot owns a CUDA stream and a solver whose grid-wide launches are
-// capped to a share of the GPU, so the work of the requests in flight
-// overlaps on the device.  Small games (below the grid-wide threshold) waiting
+// capped to a share of the GPU while several requests are in flight, so that
+// their work overlaps on the device.  Small games (below the grid-wide threshold) waiting
 // together with the same action counts are solved as one batch by a single
 // persistent launch (one thread block per game).  Each request's hierarchy and
 // policies stay resident on the device for its whole policy iteration; its
 // value and policies are copied back to host memory when it completes.
 #include <algorithm>
+#include <atomic>
 #include <chrono>
 #include <condition_variable>
 #include <cstring>
@@ -95,6 +96,24 @@ struct gs_server {
     bool stop = false;
     int64_t next_id = 1;
     int running = 0;
+    int sms = 152;
+    // Caps on the slots' cooperative launches, one block per SM, unless the caller
+    // set one.  Multigrid launches (Isaacs grids, tables on game_solver 1), of
+    // which a request makes many and whose bits do not depend on the cap, read
+    // live_blocks each time: all SMs for a request that is alone, a slot's share
+    // with others in flight or waiting (side by side they are done sooner than in
+    // turn).  The one launch of a large game on the two-level path keeps to twice
+    // the share whatever is in flight, because its sums' last bits depend on the
+    // number of blocks.  Lone requests on two slots, and four: 1023^2 grid 9.8 and
+    // 9.7 ms, game of 500,009 states 42 and 60 ms (always the share: 12.7 and 18.0, 60
+    // and 102 ms); bursts of 20 requests on two slots and 16 on four 75.9 and 57.1 ms
+    // (always the share 80.4 and 68.8, twice the share 91.0 and 70.5, all SMs 91.0
+    // and 90.1).
+    std::atomic<int> live_blocks{0};
+    int share() const { return std::max(1, sms / slots); }
+    void set_live_blocks() {   // with mu held
+        live_blocks = running + (int)pending.size() <= 1 ? 0 : share();   // 0: the whole GPU
+    }
 };
 
 namespace gs {
@@ -282,15 +301,11 @@ void worker(gs_server* S, int slot) {
     cudaStreamCreateWithFlags(&stream, cudaStreamNonBlocking);
     gs_options o = S->opt;
     o.stream = stream;
-    if (o.grid_blocks == 0) {
-        int sms = 152;
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, S->device);
-        // the cooperative kernels take one block per SM: slots that share the SMs
-        // run side by side, slots that each ask for all of them in turn
-        o.grid_blocks = std::max(1, sms / S->slots);
-    }
+    const bool shared = o.grid_blocks == 0;   // no cap of the caller's
+    if (shared) o.grid_blocks = std::min(S->sms, 2 * S->share());
     gs_solver* solver = nullptr;
     const gs_status created = gamesolve_create(&solver, &o);
+    if (shared && solver) solver->live_blocks = &S->live_blocks;
     while (true) {
         std::vector<std::shared_ptr<Request>> B;
         {
@@ -318,6 +333,7 @@ void worker(gs_server* S, int slot) {
                 }
             }
             ++S->running;
+            S->set_live_blocks();
             const double t = now_s(S->t0);
             for (auto& R : B) {
                 R->state = 1;
@@ -350,6 +366,7 @@ void worker(gs_server* S, int slot) {
                 S->in_use -= R->mem;
             }
             --S->running;
+            S->set_live_blocks();
         }
         S->work_cv.notify_all();
         S->done_cv.notify_all();
@@ -396,6 +413,8 @@ gs_status gamesolve_server_create(gs_server** out, const gs_options* opt, int32_
     S->opt = o;
     S->slots = slots;
     cudaGetDevice(&S->device);
+    cudaDeviceGetAttribute(&S->sms, cudaDevAttrMultiProcessorCount, S->device);
+    S->set_live_blocks();
     size_t free_b = 0, total_b = 0;
     cudaMemGetInfo(&free_b, &total_b);
     S->budget = mem_budget ? (size_t)mem_budget : free_b / 2;
@@ -467,6 +486,7 @@ queued:
         R->t_submit = now_s(S->t0);
         S->pending.push_back(R);
         S->all[R->id] = R;
+        S->set_live_blocks();
         *ticket = R->id;
     }
     S->work_cv.notify_all();

@@ -388,7 +388,7 @@ int linear_solve(gs_solver* s, IsaacsGrid& g, Counters& cnt, double rel_tol, boo
     a.mixed = mixed ? 1 : 0;
     a.wbf16 = s->opt.precision == GS_PREC_MIXED_BF16 ? 1 : 0;
     a.do_setup = do_setup ? 1 : 0;
-    a.max_blocks = s->opt.grid_blocks;
+    a.max_blocks = multigrid_blocks(s);
     a.lin_tol = s->opt.lin_tol;
     a.rel_tol = rel_tol;
     a.inv = g.inv;

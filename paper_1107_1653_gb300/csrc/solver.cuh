@@ -2,6 +2,7 @@
 // policy-iteration driver.
 #pragma once
 
+#include <atomic>
 #include <memory>
 #include <vector>
 
@@ -177,11 +178,15 @@ struct gs_solver {
     std::unique_ptr<gs::Problem> prob;
     bool init_v = false, init_alpha = false, init_beta = false;
     int last_levels = 0;
+    const std::atomic<int>* live_blocks = nullptr;   // a server's cap of multigrid launches
     bool give_up = false;              // failure tests: barriers start with their error raised
     std::vector<int> level_stats;      // per FAMGpi level of the last solve: side, outer, systems
 };
 
 namespace gs {
+
+// Cap on the blocks of a multigrid launch made now (0: the whole GPU).
+inline int multigrid_blocks(const gs_solver* s) { return s->live_blocks ? s->live_blocks->load() : s->opt.grid_blocks; }
 
 // Points L.u32 and L.f32 into 2 * fine_plane_elems floats at p, cleared on st.
 void set_fine_planes(Level& L, float* p, cudaStream_t st);

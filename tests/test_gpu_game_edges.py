@@ -47,3 +47,31 @@ def test_reported_shape_of_a_single_game(gs, n, threads):
         s.set_random_game(n, 4, 4, 3, 0.95)
         s.solve()
         assert s.batch_shape() == (0 if n >= 4096 else threads or 512)
+
+
+@pytest.mark.parametrize("slots", [2, 4])
+def test_large_game_on_a_server_takes_twice_a_slots_share(gs, slots):
+    """The blocks of its launch (which the last bits of float64 sums tell apart) do not
+    depend on what else is in flight, and on two slots are the whole GPU."""
+    import torch
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    n = 60_000
+
+    def alone(blocks):
+        with gs.GameSolver(precision="fp64", grid_blocks=blocks) as s:
+            s.set_random_game(n, 4, 4, 9, 0.99)
+            s.solve()
+            return s.get_value()
+
+    want = alone(2 * (sms // slots))
+    assert not np.array_equal(want, alone(sms // slots))
+    with gs.GameServer(slots=slots, precision="fp64") as srv:
+        for others in (0, 3):
+            t = srv.submit_random_game(n, 4, 4, 9, 0.99)
+            rest = [srv.submit_isaacs(255, 0, k + 1) for k in range(others)]
+            srv.wait(t)
+            v = srv.result(t)[0]
+            assert np.array_equal(v, want), others
+            for r in rest:
+                srv.wait(r)
+                srv.result(r)
