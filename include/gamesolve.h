@@ -159,8 +159,10 @@ gs_status gamesolve_create(gs_solver** out, const gs_options* opt);
  * Rows may be substochastic (the missing mass leaves the game), so a row
  * without successors is a "stop" action.
  * A game of at least 4096 states runs on the whole GPU (one cooperative
- * launch: policy iteration on the device with bounded grid barriers); a
- * smaller one runs in one thread block.  Warm starts (set_initial), improve
+ * launch: policy iteration on the device with bounded grid barriers); one of
+ * 512 to 4095 states on a cluster of 16 thread blocks (the bits of one block of
+ * 512 threads; with options.game_threads 256 on one block); a smaller one in
+ * one thread block.  Warm starts (set_initial), improve
  * and policy_solve are for Isaacs grids.
  * Errors (GS_EINVAL, solver unchanged): n < 1 or too large, m1 outside
  * [1, 64] or m2 outside [1, 255] (games with more than 8 MAX actions take the
@@ -425,8 +427,8 @@ gs_status gamesolve_isaacs_policy_solve_static(int32_t side, int32_t variant, ui
  * its own CUDA stream and solver; with several requests in flight its
  * grid-wide launches are capped to a share of the GPU, so that their work
  * overlaps on the device.
- * Games of fewer than 4096 states (those a solver runs one thread block per
- * game) that wait together with the same kind and action counts are taken by
+ * Games of fewer than 4096 states (those that give the same bits alone and in
+ * a batch) that wait together with the same kind and action counts are taken by
  * one slot as a batch of up to 256 and solved by one persistent launch
  * (gamesolve_set_game_batch); they share t_start and t_end.  A request's
  * multigrid hierarchy and policies stay on the device for its whole policy

@@ -20,8 +20,8 @@
 //    weights kept, rescaled to the row's full sum); a C point copies its
 //    coarse value;
 //  - restriction R = P^T and the Galerkin coarse operator A_c = R A P,
-//    accumulated in float64, each coarse row by one thread in a fixed order;
-//  - down to at most 64 unknowns, solved by the coarsest operator's inverse.
+//    accumulated in float64, each coarse row by one warp in a fixed order;
+//  - down to at most 128 unknowns, solved by the coarsest operator's inverse.
 // Cycles: V-cycles on the correction of the float64 iterate (float32 in the
 // mixed path, rows in leakage form: row sum kept beside the off-diagonals),
 // C/F Gauss-Seidel (the C points, then the F points, each set colour by
@@ -718,9 +718,9 @@ __global__ void __launch_bounds__(32 * kRapWarps) k_rap(int nc, const AmgLevelAr
     }
 }
 
-// Inverse of the coarsest operator (n <= 64) by Gauss-Jordan with partial
-// pivoting in one block; status 1 if singular.
-// Dynamic shared memory: the n x 2n augmented matrix.
+// Inverse of the coarsest operator (n <= kAmgCoarsest) by Gauss-Jordan with
+// partial pivoting in one block; status 1 if singular.
+// Dynamic shared memory: the n x 2n augmented matrix, for n <= kAmgInvSmem.
 struct Aug {
     double* m;
     int w;
@@ -1930,7 +1930,6 @@ AmgLevelArgs AmgHierarchy::args_of(const AmgLevelMem& m) {
     A.rcol = m.rcol;
     A.r64 = m.r64;
     A.r32 = m.r32;
-    A.cf = m.cf;
     A.ord = m.ord;
     A.cls = m.cls;
     A.g = m.W <= 8 ? 1 : m.W <= 16 ? 4 : 8;

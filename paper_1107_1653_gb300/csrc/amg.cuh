@@ -53,7 +53,6 @@ struct AmgLevelArgs {
     const int* rcol;        // [n_{l+1}][WR]
     const double* r64;
     const float* r32;
-    const int8_t* cf;       // 1 C point, 2 F point (this level's splitting)
     const int* ord;         // the points ordered by smoother class
     const AmgClasses* cls;  // the classes (levels above the coarsest)
     int g;                  // lanes that share a row (1, 4 or 8)

@@ -931,8 +931,7 @@ struct Eval {
 __device__ __forceinline__ unsigned long long abs_bits(double x) { return bits_of(x) & 0x7fffffffffffffffull; }
 
 // One state's part of the residual check: r = rhs - (v - mu M v) (float64, Mv
-// given), C.r = r and, for slot-major rows, the correction's first Jacobi sweep
-// from zero, C.e = r / diag.
+// given) -> C.r.
 template <typename T, class Ctx>
 __device__ __forceinline__ double check_tail(const Game& G, const Ctx& C, int64_t i, double Mv, double vi, double rhs) {
     const double r = rhs - (vi - G.mu * Mv);

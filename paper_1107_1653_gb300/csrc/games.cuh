@@ -138,11 +138,11 @@ void launch_game_pi_grid(const BatchArgs& B, const GridWork& W, int blocks, bool
 void launch_game_improve_one(const BatchArgs& B, int mode, int64_t n, int* scal, cudaStream_t st);
 
 // Games of at least this many states, set alone, run on a cluster or the whole
-// grid; below, one block's barriers are cheaper than its share of the work is
-// long (4 x 4 actions, set and solved, one block against a cluster: 512 states
-// 1.71 and 1.50 ms in float64, 1.62 and 1.51 ms mixed; 1000 states 2.39 and 1.53,
-// 2.12 and 1.55; 300 states 1.4 ms on one block, more than which a cluster's
-// shorter passes do not save).
+// grid; smaller ones on one block, whose barriers cost less than a cluster's
+// shorter passes save (4 x 4 actions, set and solved, one block against a cluster:
+// 300 states 1.4 ms on one block, and a cluster takes 1.5 at any small size; 512
+// states 1.71 and 1.50 ms in float64, 1.62 and 1.51 ms mixed; 1000 states 2.39 and
+// 1.53, 2.12 and 1.55).
 constexpr int64_t kGameGridMinStates = 512;
 // Games below this size that wait together at a server are solved as a batch,
 // one block each, and must give the bits they give alone (GridCtx::sum).

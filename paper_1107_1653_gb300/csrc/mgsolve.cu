@@ -1379,7 +1379,8 @@ struct FinePhases {
         }
         prolong_colour1<T, W>(a, uc, gt, gs);
     }
-    // skip: this block takes no part (it stages the tail while the others check)
+    // first_check: in launches of several blocks, by blocks 1 .. alone (block 0
+    // stages the tail meanwhile)
     __device__ __noinline__ void check(int slot, bool first_check) const {
         unsigned long long rm = 0, vm = 0;
         bool done = false;

@@ -65,9 +65,8 @@ size_t estimate_bytes(const gs_request& r) {
     return r.kind == 3 ? base + 2 * rows * (8 + 12 * (size_t)succ_of(r)) : base;
 }
 
-// Games solved together by one batched launch: below the threshold where a
-// game alone takes the whole grid, so the batch runs the kernel each of them
-// would run alone.
+// Games solved together by one batched launch: those that give the same bits
+// alone (on one block, a cluster or a few blocks) and in a batch.
 constexpr int kServeBatchMax = 256;
 bool batchable(const Request& R) {
     return (R.spec.kind == 2 || R.spec.kind == 3) && R.spec.n < kGameBatchedStates;
