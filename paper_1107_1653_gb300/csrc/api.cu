@@ -325,6 +325,7 @@ gs_status gamesolve_set_initial(gs_solver* s, const double* v0, const uint8_t* a
             for (uint8_t x : b)
                 if (x >= 4) { set_last_error("set_initial: beta out of range"); return GS_EINVAL; }
         }
+        ensure_start(s, g);   // what is not given
         if (v0) {
             GS_CUDA(cudaMemcpyAsync(g.v, v0, g.n * sizeof(double), cudaMemcpyDefault, s->st));
             s->init_v = true;

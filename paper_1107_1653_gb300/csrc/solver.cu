@@ -571,6 +571,13 @@ void default_policies(gs_solver* s, IsaacsGrid& g) {
 
 }  // namespace
 
+void ensure_start(gs_solver* s, IsaacsGrid& g) {
+    if (g.written) return;
+    default_policies(s, g);
+    GS_CUDA(cudaMemsetAsync(g.v, 0, g.n * sizeof(double), s->st));
+    g.written = true;
+}
+
 bool solve_policy_system(gs_solver* s, IsaacsGrid& g, int* cycles, double* res) {
     Counters cnt;
     g.hier_valid = false;
@@ -607,6 +614,7 @@ gs_status run_solve(gs_solver* s, gs_solve_stats* stats) {
             s->level_stats.insert(s->level_stats.end(),
                                   {g.side, cnt.outer - outer0, cnt.systems - systems0});
             if (cnt.lin_capped) {   // the finer levels are not reached
+                ensure_start(s, fine);
                 converged = false;
                 break;
             }
@@ -614,6 +622,7 @@ gs_status run_solve(gs_solver* s, gs_solve_stats* stats) {
                 IsaacsGrid& f = *P.grids[k + 1];
                 launch_fmg_interp(g.side, g.v, g.alpha, g.beta, g.beta4, f.v, f.alpha, f.beta,
                                   f.beta4, s->st);
+                f.written = true;
                 beta_given = true;
             }
         }
@@ -629,6 +638,7 @@ gs_status run_solve(gs_solver* s, gs_solve_stats* stats) {
                 GS_CUDA(cudaMemsetAsync(fine.beta4, 0, fine.n, s->st));
             }
         }
+        fine.written = true;
         if (!s->init_v) GS_CUDA(cudaMemsetAsync(fine.v, 0, fine.n * sizeof(double), s->st));
         converged = amgpi(s, fine, s->opt.eps, s->init_beta, cnt);
         s->level_stats = {fine.side, cnt.outer, cnt.systems};
@@ -685,6 +695,7 @@ gs_status run_improve(gs_solver* s, const double* v, uint8_t* alpha_out, uint8_t
                       double* fv_out) {
     Problem& P = *s->prob;
     IsaacsGrid& g = *P.grids.back();
+    ensure_start(s, g);
     const int m1 = g.variant == 1 ? 5 : 4;
     const size_t n = g.n, nv = n * sizeof(double), nb = n * m1;
     const bool apart = !overlap(v, nv, alpha_out, n) && !overlap(v, nv, beta_out, nb) &&
@@ -785,6 +796,7 @@ gs_status run_policy_solve(gs_solver* s, const uint8_t* alpha, const uint8_t* be
         set_last_error("policy_solve: action out of range");
         return GS_EINVAL;
     }
+    ensure_start(s, g);   // (beta4 stays as it is in the plain variant)
     GS_CUDA(cudaMemcpyAsync(g.alpha, a, g.n, cudaMemcpyDeviceToDevice, s->st));
     k_pack_beta<<<div_up(g.n, 256), 256, 0, s->st>>>(bst, m1, g.n, g.beta, g.beta4);
     GS_CHECK_LAUNCH();

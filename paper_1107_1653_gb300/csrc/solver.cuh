@@ -79,6 +79,7 @@ struct IsaacsGrid {
     std::vector<Level> lv;
     double* inv = nullptr;     // explicit inverse of the coarsest operator
     int* dstatus = nullptr;
+    bool written = false;      // v, alpha, beta and beta4 have been written since the grid was set
     bool hier_valid = false;   // hierarchy built for (nearly) the current codes
     long long stale_rows = 0;  // rows whose code changed since the hierarchy was built
 };
@@ -223,6 +224,10 @@ void trace_harvest(gs_solver* s);
 unsigned long long launch_count();
 void trace_reset(gs_solver* s, int cls);
 void pack_beta_upload(gs_solver* s, IsaacsGrid& g, const uint8_t* beta_host);
+// Gives a grid whose value and policies have not been written yet the default
+// start (v = 0, action 0 or stop everywhere for the obstacle variant, replies 0):
+// calls that read them, or write only some, come before any solve too.
+void ensure_start(gs_solver* s, IsaacsGrid& g);
 void unpack_beta_download(gs_solver* s, const IsaacsGrid& g, uint8_t* beta_out);
 
 }  // namespace gs
