@@ -217,7 +217,10 @@ struct ImprovePoint {
 template <int MODE>
 __global__ void __launch_bounds__(kBlock) k_isaacs_improve(const __grid_constant__ ImproveArgs A, double tau_host,
                                                            float tau_host_f, int tau_from_vmax) {
-    if (A.solved && (A.solve_bar->error || (A.solved->reason != kLinExact && A.solved->reason != kLinInexact))) return;
+    if (A.solved) {
+        const int gave_up = A.solve_bar->error, reason = A.solved->reason;   // (one round trip for both)
+        if (gave_up || (reason != kLinExact && reason != kLinInexact)) return;
+    }
     const IsaacsConsts* __restrict__ K = A.K;
     const int side = A.side, variant = A.variant;
     const double tau = tau_from_vmax ? tau_of_vmax(A.sc) : tau_host;
